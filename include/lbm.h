@@ -225,10 +225,14 @@ lbm_status lbm_set_valve_schedule(lbm_handle h, int64_t period, int32_t n,
                                   const uint32_t* states);
 
 /* Advance n >= 0 coupled time steps, asynchronously on the handle's stream.
- * Each step is one launch of the fused kernel: pull-stream of f and g,
- * bounce-back, open-port completion, moments, collision of f, collision of
- * g with the same step's velocity, and per-block partial sums of the
- * diagnostics (lbm_get_diagnostics adds them up).  Returns LBM_ERR_NUMERIC (after
+ * A step is pull-stream of f and g, bounce-back, open-port completion,
+ * moments, collision of f and collision of g with the same step's velocity;
+ * the call's last step also leaves per-block partial sums of the
+ * diagnostics (lbm_get_diagnostics adds them up).  Each step is one launch,
+ * or, where that is faster and variant, block_threads, max_blocks and
+ * multi_step are left at 0 (halfway bounce-back walls), two steps before the
+ * last are one launch that keeps the state between them on the chip.
+ * Results are the same bits either way.  Returns LBM_ERR_NUMERIC (after
  * issuing the steps) while a previous synchronising call has found the
  * numeric error flag set and lbm_clear_error has not reset it. */
 lbm_status lbm_step(lbm_handle h, int64_t n);

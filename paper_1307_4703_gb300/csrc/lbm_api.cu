@@ -19,6 +19,7 @@
 
 #include "lbm.h"
 #include "lbm_internal.h"
+#include "lbm_plan.h"
 
 namespace {
 
@@ -68,6 +69,7 @@ struct lbm_ctx {
     int precision = lbm::kFP32;
     size_t elem = sizeof(float);
     int cur = 0;   // buffer holding the current state
+    int order = 0; // direction of the next single step's tile order (alternates from step to step)
     int gbuf = 0;  // buffer holding the current scalar planes: cur, except after
                    // an odd number of scalar-only steps (joined lazily)
     uint8_t* links = nullptr;
@@ -91,6 +93,11 @@ struct lbm_ctx {
     int diag_grid = 0;     // blocks whose partials the last step wrote
     int scalar_grid = 0;  // one wave of the scalar-only step kernel (set on first use)
     bool scalar_regs = true;  // scalar-only step: register variant (else the bulk-copy pipeline)
+    int4* pair_items = nullptr;   // the two-step kernel's strips (lbm_pair.cu), its blocks' first strips
+    int* pair_first = nullptr;
+    CUtensorMap pair_map[2];      // of the two state buffers
+    int pair_grid = 0;            // its blocks; 0: this handle has none
+    bool pairs = false;           // lbm_step takes two steps a launch
     int multi_step = 0;           // lbm_step: steps per cooperative launch (0 = one launch per step)
     int coop_grid = 0;            // blocks of that launch (all resident)
     unsigned* bar = nullptr;      // its grid-barrier count
@@ -123,10 +130,11 @@ struct lbm_ctx {
     float4* rates = nullptr; // per-row relaxation rates of a batch
 
     // CUDA graphs of graph_steps consecutive step launches, one per valve
-    // words and starting buffer, captured on a private stream.
+    // words, starting buffer and order, captured on a private stream.
     struct Graph {
         uint32_t words[lbm::kMaskWords];
-        int parity;
+        int parity, order;
+        int launches;
         cudaGraphExec_t exec;
     };
     int graph_steps = 0;
@@ -300,13 +308,37 @@ cudaError_t launch_full_step(const lbm_ctx* h, const lbm::StepArgs& a, const lbm
     return lbm::launch_step(a, L, s);
 }
 
+// After a step by itself.
+void swap_buffers(lbm_ctx* h)
+{
+    h->cur = 1 - h->cur;
+    h->order = 1 - h->order;
+}
+
+// Two steps in one launch: a holds the first one's arguments (src, dst and
+// reverse among them), words the valve words of the second.
+cudaError_t launch_pair(const lbm_ctx* h, const lbm::StepArgs& a, const uint32_t (&words)[lbm::kMaskWords],
+                        const CUtensorMap& src_map, cudaStream_t s)
+{
+    lbm::PairArgs p{a, a, h->pair_items, h->pair_first};
+    std::memcpy(p.second.open_mask, words, sizeof(words));
+    p.second.plane = lbm::kTileNodes;
+    return lbm::launch_step_pair(p, src_map, h->pair_grid, h->precision, s);
+}
+
+// Whether the next two of `left` steps go as one launch.  The last step of a
+// call (and of a graph) is always one by itself, which leaves the call's
+// diagnostics as every single step does; the steps before it leave none, which
+// nothing could read.
+bool pair_next(const lbm_ctx* h, int64_t left) { return h->pairs && left >= 3; }
+
 // The cached graph of graph_steps launches for the valve words in
 // a.open_mask starting from buffer cur, captured on first use.
-lbm_status step_graph(lbm_ctx* h, lbm::StepArgs a, cudaGraphExec_t* out)
+lbm_status step_graph(lbm_ctx* h, lbm::StepArgs a, const lbm_ctx::Graph** out)
 {
     for (auto& g : h->graphs)
-        if (g.parity == h->cur && std::memcmp(g.words, a.open_mask, sizeof(g.words)) == 0) {
-            *out = g.exec;
+        if (g.parity == h->cur && g.order == h->order && std::memcmp(g.words, a.open_mask, sizeof(g.words)) == 0) {
+            *out = &g;
             return LBM_OK;
         }
     if (int(h->graphs.size()) >= kMaxGraphs) {  // keep the cache small: start over
@@ -316,11 +348,21 @@ lbm_status step_graph(lbm_ctx* h, lbm::StepArgs a, cudaGraphExec_t* out)
     }
     LBM_CUDA(h, cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaSuccess;
-    for (int j = 0; j < h->graph_steps && e == cudaSuccess; ++j) {
-        a.src = h->pop[(h->cur + j) & 1];
-        a.dst = h->pop[(h->cur + j + 1) & 1];
-        a.reverse = (h->cur + j) & 1;
-        e = launch_full_step(h, a, h->launch, h->cap_stream);
+    int launches = 0;  // each swaps the buffers
+    for (int j = 0; j < h->graph_steps && e == cudaSuccess; ++launches) {
+        const int from = (h->cur + launches) & 1;
+        a.src = h->pop[from];
+        a.dst = h->pop[1 - from];
+        if (pair_next(h, h->graph_steps - j)) {
+            a.reverse = from;
+            e = launch_pair(h, a, a.open_mask, h->pair_map[from], h->cap_stream);
+            j += 2;
+        } else {
+            a.reverse = (h->order + j) & 1;
+            a.partials = h->graph_steps - j > 1 ? nullptr : h->partials;
+            e = launch_full_step(h, a, h->launch, h->cap_stream);
+            ++j;
+        }
     }
     cudaGraph_t graph = nullptr;
     const cudaError_t e_end = cudaStreamEndCapture(h->cap_stream, &graph);
@@ -332,9 +374,11 @@ lbm_status step_graph(lbm_ctx* h, lbm::StepArgs a, cudaGraphExec_t* out)
     lbm_ctx::Graph g;
     std::memcpy(g.words, a.open_mask, sizeof(g.words));
     g.parity = h->cur;
+    g.order = h->order;
+    g.launches = launches;
     g.exec = exec;
     h->graphs.push_back(g);
-    *out = exec;
+    *out = &h->graphs.back();
     return LBM_OK;
 }
 
@@ -646,9 +690,11 @@ lbm_status create_impl(lbm_handle* out, int32_t nx, int32_t ny, const uint8_t* m
             const int gran = pass == 0 ? lbm::kTileStart : lbm::kTileNodes;
             bool fits = true;
             int t0 = -1, q0 = 0, q1 = 0;
+            int wall = -1;          // last quad after the first one with a wall link
+            bool scattered = false; // such a quad before the last one
             auto push = [&]() {
                 tiles.push_back(make_uint2((uint32_t(y) << lbm::kColBits) | uint32_t(t0 / lbm::kTileStart),
-                                           uint32_t(q0) | (uint32_t(q1) << 8)));
+                                           uint32_t(q0) | (uint32_t(q1) << 8) | (scattered ? lbm::kWallTile : 0u)));
             };
             for (int x = 0; x < nx && fits; ++x) {
                 if (L[x] == lbm::kSolid) continue;
@@ -657,8 +703,12 @@ lbm_status create_impl(lbm_handle* out, int32_t nx, int32_t ny, const uint8_t* m
                     t0 = x / gran * gran;
                     if (t0 + lbm::kTileNodes > pitch) fits = false;
                     q0 = (x - t0) / 4;
+                    wall = -1;
+                    scattered = false;
                 }
                 q1 = (x - t0) / 4;
+                scattered |= wall >= 0 && q1 > wall;
+                if (L[x] != 0 && q1 > q0) wall = q1;
             }
             if (fits) {
                 if (t0 >= 0) push();
@@ -721,9 +771,8 @@ lbm_status create_impl(lbm_handle* out, int32_t nx, int32_t ny, const uint8_t* m
             std::swap(rows[1], rows[2]);
         }
     };
-    const int n_thr = (long long)nx * ny < (1 << 20)
-                          ? 1
-                          : std::max(1, std::min({16, ny, int(std::thread::hardware_concurrency())}));
+    const int n_thr = int(std::max<long long>(
+        1, std::min<long long>({16, ny, (long long)std::thread::hardware_concurrency(), (long long)nx * ny >> 17})));
     std::vector<RowsOut> parts(n_thr);
     {
         std::vector<std::thread> pool;
@@ -880,6 +929,30 @@ lbm_status create_impl(lbm_handle* out, int32_t nx, int32_t ny, const uint8_t* m
     h->diag = static_cast<double*>(dev_alloc(h, 4 * sizeof(double)));
     h->fields_tmp = static_cast<float*>(dev_alloc(h, size_t(4) * nx * ny * sizeof(float)));
     if (batch) h->rates = static_cast<float4*>(dev_alloc(h, size_t(ny) * sizeof(float4)));
+    // The two-step launches, for handles that leave the step kernel and its
+    // launch shape to the library.  One that cannot have them (no tensor maps,
+    // no memory for the strips) steps one launch at a time.
+    lbm::PairPlan plan;
+    if (opt.variant == 0 && opt.block_threads == 0 && opt.max_blocks == 0 && opt.multi_step == 0 &&
+        opt.wall_scheme == LBM_WALL_BOUNCE_BACK && h->pop[0] && h->pop[1]) {
+        int pair_per_sm = 0;
+        bool have = lbm::pair_occupancy(h->precision, &pair_per_sm) == cudaSuccess && pair_per_sm > 0;
+        for (int b = 0; b < 2 && have; ++b)
+            have = lbm::pair_tensor_map(&h->pair_map[b], h->pop[b], ny, pitch, h->precision) == cudaSuccess;
+        if (have) {
+            plan = lbm::plan_pairs(h->tiles_rows, rowbc, nx, ny, pitch, h->precision, lbm::pair_warps(h->precision),
+                                   pair_per_sm * sms);
+            h->pair_items = static_cast<int4*>(dev_alloc(h, plan.items.size() * sizeof(int4)));
+            h->pair_first = static_cast<int*>(dev_alloc(h, plan.block_first.size() * sizeof(int)));
+            have = h->pair_items && h->pair_first;
+        } else {
+            cudaGetLastError();
+        }
+        if (have) {
+            h->pair_grid = plan.grid;
+            h->pairs = plan.worth;
+        }
+    }
     std::vector<long long> woff;
     if (opt.wall_scheme == LBM_WALL_EQUILIBRIUM) {
         for (size_t o = 0; o < links.size(); ++o)
@@ -900,6 +973,11 @@ lbm_status create_impl(lbm_handle* out, int32_t nx, int32_t ny, const uint8_t* m
         e = cudaMemcpyAsync(h->rowbc, rowbc.data(), rowbc.size() * sizeof(lbm::RowBC),
                             cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = arrange_tiles(h, h->launch);
+    if (e == cudaSuccess && h->pair_grid > 0)
+        e = cudaMemcpyAsync(h->pair_items, plan.items.data(), plan.items.size() * sizeof(int4), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess && h->pair_grid > 0)
+        e = cudaMemcpyAsync(h->pair_first, plan.block_first.data(), plan.block_first.size() * sizeof(int),
+                            cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess && batch)
         e = cudaMemcpyAsync(h->rates, batch->rates.data(), size_t(ny) * sizeof(float4), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess && !woff.empty())
@@ -1156,12 +1234,12 @@ lbm_status lbm_step(lbm_handle h, int64_t n)
                 // other buffer when m is odd
                 a.src = h->pop[h->cur];
                 a.dst = h->pop[1 - h->cur];
-                a.reverse = h->cur;
+                a.reverse = h->order;
                 a.barrier_extra = h->barrier_extra;
                 cudaError_t e =
                     lbm::launch_steps_coop(a, int(m), 0, h->bar, h->coop_grid, kDefaultRegsBlock, h->stream);
                 if (e != cudaSuccess) return cuda_fail(h, e, "multi-step launch");
-                if (m & 1) h->cur = 1 - h->cur;
+                if (m & 1) swap_buffers(h);
                 h->gbuf = h->cur;
                 h->diag_grid = h->coop_grid;
                 h->step += m;
@@ -1170,12 +1248,13 @@ lbm_status lbm_step(lbm_handle h, int64_t n)
             }
         }
         if (G > 0 && n - k >= G && h->mask_constant(h->step, G)) {
-            // G steps (an even number: the state ends in the buffer it
-            // started from) as one graph launch
-            cudaGraphExec_t exec = nullptr;
-            lbm_status s = step_graph(h, a, &exec);
+            // G steps as one graph launch
+            const lbm_ctx::Graph* g = nullptr;
+            lbm_status s = step_graph(h, a, &g);
             if (s != LBM_OK) return s;
-            LBM_CUDA(h, cudaGraphLaunch(exec, h->stream));
+            LBM_CUDA(h, cudaGraphLaunch(g->exec, h->stream));
+            if (g->launches & 1) h->cur = 1 - h->cur;
+            h->gbuf = h->cur;
             h->step += G;
             k += G;
             h->diag_grid = h->launch.grid;
@@ -1183,10 +1262,23 @@ lbm_status lbm_step(lbm_handle h, int64_t n)
         }
         a.src = h->pop[h->cur];
         a.dst = h->pop[1 - h->cur];
-        a.reverse = h->cur;  // alternate the tile order from step to step
+        if (pair_next(h, n - k)) {
+            a.reverse = h->cur;  // alternate the march from launch to launch
+            uint32_t next[lbm::kMaskWords];
+            h->mask_words(h->step + 1, next);
+            cudaError_t e = launch_pair(h, a, next, h->pair_map[h->cur], h->stream);
+            if (e != cudaSuccess) return cuda_fail(h, e, "two-step launch");
+            h->cur = 1 - h->cur;
+            h->gbuf = h->cur;
+            h->step += 2;
+            k += 2;
+            continue;
+        }
+        a.reverse = h->order;  // alternate the tile order from step to step
+        a.partials = n - k > 1 ? nullptr : h->partials;
         cudaError_t e = launch_full_step(h, a, h->launch, h->stream);
         if (e != cudaSuccess) return cuda_fail(h, e, "coupled step launch");
-        h->cur = 1 - h->cur;
+        swap_buffers(h);
         h->gbuf = h->cur;
         h->diag_grid = h->launch.grid;
         ++h->step;
@@ -1231,12 +1323,12 @@ lbm_status lbm_step_diagnostics(lbm_handle h, int64_t n, double* out)
         h->mask_words(h->step, a.open_mask);
         a.src = h->pop[h->cur];
         a.dst = h->pop[1 - h->cur];
-        a.reverse = h->cur;
+        a.reverse = h->order;
         a.diag_out = fold ? dev + 4 * k : nullptr;  // the step's last block writes the totals here
         cudaError_t e = launch_full_step(h, a, h->launch, h->stream);
         if (e == cudaSuccess && !fold) e = lbm::launch_diag_finish(h->partials, h->launch.grid, dev + 4 * k, h->stream);
         if (e != cudaSuccess) return cuda_fail(h, e, "coupled step launch");
-        h->cur = 1 - h->cur;
+        swap_buffers(h);
         h->gbuf = h->cur;
         h->diag_grid = h->launch.grid;
         ++h->step;
@@ -1683,7 +1775,7 @@ lbm_status lbm_adjoint(lbm_handle h, const lbm_objective* obj, int64_t n, int32_
         a.partials = h->partials;
         cudaError_t e = lbm::launch_step(a, h->launch, st);
         if (e != cudaSuccess) return cuda_fail(h, e, "coupled step launch");
-        h->cur = 1 - h->cur;
+        swap_buffers(h);
         h->gbuf = h->cur;
         h->diag_grid = h->launch.grid;
         h->step += n;
@@ -1700,7 +1792,7 @@ lbm_status lbm_adjoint(lbm_handle h, const lbm_objective* obj, int64_t n, int32_
             cudaError_t e = lbm::launch_step(a, h->launch, st);
             if (e != cudaSuccess) return cuda_fail(h, e, "coupled step launch");
         }
-        h->cur = 1 - h->cur;
+        swap_buffers(h);
         h->gbuf = h->cur;
         h->diag_grid = h->launch.grid;
         h->step += n;
@@ -1715,11 +1807,11 @@ lbm_status lbm_adjoint(lbm_handle h, const lbm_objective* obj, int64_t n, int32_
                 LBM_CUDA(h, cudaMemcpyAsync(ckpt + size_t(t / K) * S, h->pop[h->cur], S, cudaMemcpyDeviceToDevice, st));
             a.src = h->pop[h->cur];
             a.dst = h->pop[1 - h->cur];
-            a.reverse = h->cur;
+            a.reverse = h->order;
             a.open_mask[0] = h->mask_at(t0 + t);
             cudaError_t e = lbm::launch_step(a, h->launch, st);
             if (e != cudaSuccess) return cuda_fail(h, e, "coupled step launch");
-            h->cur = 1 - h->cur;
+            swap_buffers(h);
             h->gbuf = h->cur;
             h->diag_grid = h->launch.grid;
             ++h->step;
@@ -1731,7 +1823,7 @@ lbm_status lbm_adjoint(lbm_handle h, const lbm_objective* obj, int64_t n, int32_
             float* slot1 = reinterpret_cast<float*>(seg);
             a.src = last;
             a.dst = slot1;
-            a.reverse = h->cur;
+            a.reverse = h->order;
             a.open_mask[0] = h->mask_at(t0 + s_last);
             cudaError_t e = lbm::launch_step(a, h->launch, st);
             if (e != cudaSuccess) return cuda_fail(h, e, "coupled step launch");
@@ -1740,12 +1832,12 @@ lbm_status lbm_adjoint(lbm_handle h, const lbm_objective* obj, int64_t n, int32_
         }
         a.src = last;
         a.dst = h->pop[1 - h->cur];
-        a.reverse = int((h->cur + len - 1) & 1);
+        a.reverse = int((h->order + len - 1) & 1);
         a.open_mask[0] = h->mask_at(t0 + n - 1);
         a.partials = h->partials;
         cudaError_t e = lbm::launch_step(a, h->launch, st);
         if (e != cudaSuccess) return cuda_fail(h, e, "coupled step launch");
-        h->cur = 1 - h->cur;
+        swap_buffers(h);
         h->gbuf = h->cur;
         h->diag_grid = h->launch.grid;
         h->step += len;
@@ -2035,9 +2127,8 @@ lbm_status lbm_autotune(lbm_handle h, int32_t trial_steps)
     const size_t state_bytes = size_t(h->plane) * lbm::kPlanes * h->elem;
     void* buf0 = sc.get(state_bytes);
     void* buf1 = sc.get(state_bytes);
-    float2* part = static_cast<float2*>(sc.get(size_t(h->partials_cap) * 4 * sizeof(float2)));
     unsigned* err = static_cast<unsigned*>(sc.get(sizeof(unsigned)));
-    if (!buf0 || !buf1 || !part || !err) return fail(h, LBM_ERR_OOM, "no device memory for the trial steps");
+    if (!buf0 || !buf1 || !err) return fail(h, LBM_ERR_OOM, "no device memory for the trial steps");
     LBM_CUDA(h, lbm::prepare_step_kernels());
     LBM_CUDA(h, cudaMemcpyAsync(buf0, h->pop[h->cur], state_bytes, cudaMemcpyDeviceToDevice, h->stream));
     float* const bufs[2] = {static_cast<float*>(buf0), static_cast<float*>(buf1)};
@@ -2062,7 +2153,7 @@ lbm_status lbm_autotune(lbm_handle h, int32_t trial_steps)
     a.inv_cs2g = h->inv_cs2g;
     a.decay = h->decay;
     a.wallv = h->wallv;
-    a.partials = part;
+    a.partials = nullptr;  // as every step of lbm_step but a call's last
     a.err = err;
     if (h->precision != LBM_FP32) {
         a.gref0 = h->wg0 * lbm::kCRef;
@@ -2141,16 +2232,49 @@ lbm_status lbm_autotune(lbm_handle h, int32_t trial_steps)
             best_ms = ms;
         }
     }
+    // two steps a launch against the fastest single step, over as many steps
+    bool pairs = false;
+    if (e == cudaSuccess && best.grid > 0 && h->pair_grid > 0) {
+        CUtensorMap maps[2];
+        for (int b = 0; b < 2 && e == cudaSuccess; ++b)
+            e = lbm::pair_tensor_map(&maps[b], bufs[b], h->ny, h->pitch, h->precision);
+        const int launches = (trial_steps + 1) / 2;
+        int64_t k = 0;
+        auto trial_pair = [&]() {
+            a.src = bufs[k & 1];
+            a.dst = bufs[1 - (k & 1)];
+            a.reverse = int(k & 1);
+            const CUtensorMap& m = maps[k & 1];
+            ++k;
+            return launch_pair(h, a, a.open_mask, m, h->stream);
+        };
+        if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, sizeof(unsigned), h->stream);
+        for (int j = 0; j < 3 && e == cudaSuccess; ++j) e = trial_pair();
+        float ms = 0.f;
+        for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) {
+            if (e == cudaSuccess) e = cudaEventRecord(e0, h->stream);
+            for (int j = 0; j < launches && e == cudaSuccess; ++j) e = trial_pair();
+            if (e == cudaSuccess) e = cudaEventRecord(e1, h->stream);
+            if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+            float t = 0.f;
+            if (e == cudaSuccess) e = cudaEventElapsedTime(&t, e0, e1);
+            if (rep == 0 || t < ms) ms = t;
+        }
+        unsigned ew = 0;
+        if (e == cudaSuccess) e = cudaMemcpy(&ew, err, sizeof(unsigned), cudaMemcpyDeviceToHost);
+        pairs = e == cudaSuccess && (ew & 2u) == 0 && ms * float(trial_steps) < best_ms * float(2 * launches);
+    }
     cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     if (e != cudaSuccess) return cuda_fail(h, e, "autotune trial");
     if (best.grid == 0) return fail(h, LBM_ERR_STATE, "no launch shape completed its trial steps");
-    if (best.variant != h->launch.variant || best.block != h->launch.block || best.stages != h->launch.stages ||
+    if (pairs != h->pairs || best.variant != h->launch.variant || best.block != h->launch.block || best.stages != h->launch.stages ||
         best.grid != h->launch.grid) {
         LBM_CUDA(h, cudaStreamSynchronize(h->stream));
         for (auto& g : h->graphs) cudaGraphExecDestroy(g.exec);  // captured with the old shape
         h->graphs.clear();
         h->launch = best;
+        h->pairs = pairs;
     }
     LBM_CUDA(h, arrange_tiles(h, h->launch));  // the order of the shape kept
     return LBM_OK;

@@ -152,9 +152,17 @@ struct Codec<F32Coherent> {
     static __device__ __forceinline__ void st1(F32Coherent* p, float v, float) { *f(p) = v; }
 };
 
+// Elements of type T in shared memory, for the code shared with global
+// sources (the read-only path of __ldg serves global memory only).
+template <typename T>
+struct Shared {
+    T v;
+};
+
 // Storage types that hold FP32 values as they are (no deviation offsets).
 template <typename T>
-constexpr bool kStoresF32 = std::is_same<T, float>::value || std::is_same<T, F32Coherent>::value;
+constexpr bool kStoresF32 = std::is_same<T, float>::value || std::is_same<T, F32Coherent>::value ||
+                            std::is_same<T, Shared<float>>::value;
 
 template <>
 struct Codec<__half> {
@@ -222,6 +230,18 @@ struct Codec<__nv_bfloat16> {
     static __device__ __forceinline__ float lds1(const __nv_bfloat16* p, float off)
     {
         return add_offset(__bfloat162float(*p), off);
+    }
+};
+
+template <typename T>
+struct Codec<Shared<T>> {
+    static __device__ __forceinline__ float4 ld4(const Shared<T>* p, float off)
+    {
+        return Codec<T>::lds4(reinterpret_cast<const T*>(p), off);
+    }
+    static __device__ __forceinline__ float ld1(const Shared<T>* p, float off)
+    {
+        return Codec<T>::lds1(reinterpret_cast<const T*>(p), off);
     }
 };
 

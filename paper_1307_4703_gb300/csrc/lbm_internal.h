@@ -23,6 +23,7 @@
 
 #include <cstdint>
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 namespace lbm {
@@ -50,6 +51,9 @@ constexpr int kPairTileNodes = 64;  // nodes per warp tile of variant 5: 32 lane
 // (of either side; whether its valve is open is decided per step).  Tiles
 // without one run a step without any port code.
 constexpr uint32_t kPortTile = 1u << 16;
+// Bit of a host tile entry's .y: wall links within the tile, not only in the
+// quads where its fluid begins and ends (lbm_plan.cu; kernels ignore it).
+constexpr uint32_t kWallTile = 1u << 17;
 constexpr int kSegBits64 = 13;      // 64-node tile encoding: segment in the low 13 bits
 enum Precision { kFP32 = 0, kFP16 = 1, kBF16 = 2 };
 constexpr float kCRef = 0.5f;  // reference concentration of 16-bit scalar storage
@@ -115,6 +119,24 @@ struct StepArgs {
     unsigned int* diag_ticket;  // blocks of the step that have written their partials (zero
                                 // between steps: the last block resets it)
 };
+
+// Two coupled steps in one launch (lbm_pair.cu).  `items` are strips of 128
+// columns: x = first column, y = first | (last << 8) lane the second step
+// writes | kPairPort, z and w = first and one past the last row it writes;
+// block b takes items block_first[b] .. block_first[b + 1] - 1.
+constexpr int kPairPort = 1 << 16;      // some node the strip computes is a port node
+constexpr int kPairSide = 1 << 17;      // two lanes lie along a side wall, named in the bits from
+constexpr int kPairLaneBit = 18;        // here on, five each
+struct PairArgs {
+    StepArgs first;         // time t: reads src
+    StepArgs second;        // time t + 1: writes dst; plane = kTileNodes (its own-node reads go to the ring)
+    const int4* items;
+    const int* block_first;
+};
+cudaError_t pair_occupancy(int precision, int* per_sm);
+int pair_warps(int precision);  // of a block
+cudaError_t pair_tensor_map(CUtensorMap* map, void* pop, int ny, int pitch, int precision);
+cudaError_t launch_step_pair(const PairArgs& p, const CUtensorMap& map, int grid, int precision, cudaStream_t s);
 
 // One adjoint step (lbm_adjoint.cu): A(t) from A(t+1) and the state P(t).
 struct AdjointArgs {

@@ -1,0 +1,286 @@
+// lbm_plan.cu -- host-side plan of the two-step kernel (lbm_pair.cu): strips
+// of the lattice and their split over the blocks of one wave.
+#include <algorithm>
+#include <vector>
+
+#include "lbm_plan.h"
+
+namespace lbm {
+namespace {
+
+// Strips begin and end on multiples of this many columns: whole 32-byte
+// sectors of FP32 rows (at multiples of 4 the large chip took 45.6 against 44.7
+// us a step, its blocks sharing sectors).
+constexpr int kAlign = 8;
+
+struct Span {
+    int b, e;  // columns [b, e)
+};
+
+// A strip's columns: lanes l0 .. l1 of the 128 columns from x0 are written.
+struct Strip {
+    int x0, l0, l1;
+    int begin() const { return x0 + 4 * l0; }
+    int end() const { return x0 + 4 * (l1 + 1); }
+};
+
+// Strips that cover the spans from the left.  A strip writes its lanes
+// 1 .. 30: lanes 0 and 31 are computed for the second step of their
+// neighbours only, except at the lattice's own edges.
+std::vector<Strip> cover(const std::vector<Span>& spans, int nx, int pitch)
+{
+    std::vector<Strip> out;
+    for (const Span& s : spans) {
+        int p = s.b;
+        while (p < s.e) {
+            if (!out.empty() && p < out.back().end()) {
+                p = out.back().end();
+                continue;
+            }
+            p = p / kAlign * kAlign;
+            const int x0 = std::min(std::max(p - 4, 0), pitch - kTileNodes);
+            int l1 = x0 + kTileNodes >= nx ? 31 : 30;
+            if (l1 == 30) l1 = (x0 + 124) / kAlign * kAlign / 4 - x0 / 4 - 1;
+            const Strip t{x0, (p - x0) / 4, l1};
+            out.push_back(t);
+            p = t.end();
+        }
+    }
+    return out;
+}
+
+// Strips of `strips` that a row's spans touch, and whether they cover them all.
+int touched(const std::vector<Strip>& strips, const std::vector<Span>& spans, bool& covered)
+{
+    int hits = 0;
+    covered = true;
+    for (const Strip& t : strips)
+        for (const Span& s : spans)
+            if (s.b < t.end() && t.begin() < s.e) {
+                ++hits;
+                break;
+            }
+    size_t k = 0;
+    for (const Span& s : spans)
+        for (int p = s.b; p < s.e;) {
+            while (k < strips.size() && strips[k].end() <= p) ++k;
+            if (k == strips.size() || strips[k].begin() > p) {
+                covered = false;
+                return hits;
+            }
+            p = strips[k].end();
+        }
+    return hits;
+}
+
+// What a strip's rows hold.  The costs are of an iteration of the march,
+// measured on the 4096 x 2048 chip and the batch of 64 chips (the splits that
+// were fastest): side walls add the side lanes' work, ports that of a lane
+// that completes its node alone while its warp waits, and walls anywhere a
+// wait for the nodes' own values in global memory.
+enum Kind { kPlain, kSide, kScattered, kPort, kScatteredPort };
+constexpr int kCost[5] = {16, 18, 28, 24, 36};
+
+struct Run {
+    Strip t;
+    int ya, yb;
+    Kind kind;
+    int side;  // kPairSide and the lanes along the walls
+};
+
+constexpr int kBandRows = 8;  // rows that must gain from new strips before the strips change
+
+// Consecutive rows [ya, yb) whose fluid covers the same columns (whole quads).
+struct Rows {
+    int ya, yb;
+    std::vector<Span> spans;
+    std::vector<Strip> own;  // the strips that cover them alone
+};
+
+std::vector<Rows> row_groups(const std::vector<uint2>& tiles, int nx, int ny, int pitch)
+{
+    std::vector<Rows> out;
+    std::vector<Span> spans;
+    size_t t = 0;
+    for (int y = 0; y < ny; ++y) {
+        spans.clear();
+        for (; t < tiles.size() && int(tiles[t].x >> kColBits) == y; ++t) {
+            const int x0 = int(tiles[t].x & ((1u << kColBits) - 1)) * kTileStart;
+            const Span s{x0 + 4 * int(tiles[t].y & 0xFFu), x0 + 4 * int((tiles[t].y >> 8) & 0xFFu) + 4};
+            if (!spans.empty() && spans.back().e == s.b) spans.back().e = s.e;
+            else spans.push_back(s);
+        }
+        if (!out.empty() && out.back().spans.size() == spans.size() &&
+            std::equal(spans.begin(), spans.end(), out.back().spans.begin(),
+                       [](const Span& a, const Span& b) { return a.b == b.b && a.e == b.e; }))
+            out.back().yb = y + 1;
+        else
+            out.push_back({y, y + 1, spans, cover(spans, nx, pitch)});
+    }
+    return out;
+}
+
+std::vector<Run> strip_runs(const std::vector<Rows>& groups)
+{
+    std::vector<Run> runs;
+    std::vector<Strip> cur;
+    std::vector<int> open;  // index of each strip's run in `runs`, -1 = none
+    for (size_t k = 0; k < groups.size(); ++k) {
+        const Rows& g = groups[k];
+        bool covered = false;
+        if (!g.spans.empty()) touched(cur, g.spans, covered);
+        bool fresh = !covered;
+        if (covered) {  // would other strips do with fewer, and for long enough?
+            int gain = 0;
+            for (size_t n = k; n < groups.size() && gain < kBandRows; ++n) {
+                bool c = false;
+                if (groups[n].spans.empty() ||
+                    touched(cur, groups[n].spans, c) <= int(groups[n].own.size()))
+                    break;
+                gain += groups[n].yb - groups[n].ya;
+            }
+            fresh = gain >= kBandRows;
+        }
+        if (fresh) {
+            cur = g.own;
+            open.assign(cur.size(), -1);
+        }
+        for (size_t n = 0; n < cur.size(); ++n) {
+            bool hit = false;
+            for (const Span& s : g.spans) hit |= s.b < cur[n].end() && cur[n].begin() < s.e;
+            if (!hit) open[n] = -1;
+            else if (open[n] >= 0) runs[size_t(open[n])].yb = g.yb;
+            else {
+                open[n] = int(runs.size());
+                runs.push_back({cur[n], g.ya, g.yb, kPlain, 0});
+            }
+        }
+    }
+    return runs;
+}
+
+// Runs split where they start or stop holding port nodes or side walls, and
+// their kinds: scattered walls where more than half of the rows have some
+// within the strip (kWallTile).
+std::vector<Run> split_kinds(const std::vector<Run>& runs, const std::vector<Rows>& groups,
+                             const std::vector<uint2>& tiles, const std::vector<RowBC>& bc, int ny)
+{
+    std::vector<Run> out;
+    std::vector<int> group_of(static_cast<size_t>(ny));
+    for (size_t k = 0; k < groups.size(); ++k)
+        for (int y = groups[k].ya; y < groups[k].yb; ++y) group_of[size_t(y)] = int(k);
+    std::vector<std::vector<int>> walls(static_cast<size_t>(ny));  // first columns of each row's tiles with scattered walls
+    for (const uint2& t : tiles)
+        if (t.y & kWallTile)
+            walls[size_t(t.x >> kColBits)].push_back(int(t.x & ((1u << kColBits) - 1)) * kTileStart);
+    for (const Run& r : runs) {
+        const int x0 = r.t.x0, x1 = x0 + kTileNodes;
+        // the lanes where the row's fluid begins and ends within the strip; -1: more than two
+        auto side = [&](int y) {
+            int lanes = 0, n = 0;
+            for (const Span& s : groups[size_t(group_of[size_t(y)])].spans) {
+                if (s.b >= x0 && s.b < x1 && n++ < 2) lanes |= (s.b - x0) / 4 << (kPairLaneBit + 5 * (n - 1));
+                if (s.e > x0 && s.e <= x1 && n++ < 2) lanes |= (s.e - 4 - x0) / 4 << (kPairLaneBit + 5 * (n - 1));
+            }
+            return n == 1 || n == 2 ? lanes | kPairSide : n ? -1 : 0;
+        };
+        auto port = [&](int y) {
+            for (int yy = std::max(y - 1, 0); yy <= std::min(y + 1, ny - 1); ++yy)
+                for (int s = 0; s < 2; ++s) {
+                    const int px = bc[size_t(s) * ny + yy].x;
+                    if (px >= x0 && px < x1) return true;
+                }
+            return false;
+        };
+        auto scattered = [&](int y) {
+            for (int x : walls[size_t(y)])
+                if (x < x1 && x0 < x + kTileNodes) return true;
+            return false;
+        };
+        for (int y = r.ya; y < r.yb;) {
+            const bool ports = port(y);
+            const int first = side(y);
+            bool same = first >= 0;
+            int last = group_of[size_t(y)], lanes = first, rough = 0, e = y;
+            for (; e < r.yb && port(e) == ports; ++e) {
+                if (group_of[size_t(e)] != last) {
+                    last = group_of[size_t(e)];
+                    lanes = side(e);
+                    if ((lanes != 0) != (first != 0)) break;
+                    same &= lanes == first;
+                }
+                rough += scattered(e);
+            }
+            const bool walls_anywhere = 2 * rough > e - y || !same;
+            const Kind kind = ports ? (walls_anywhere ? kScatteredPort : kPort)
+                              : walls_anywhere ? kScattered : first ? kSide : kPlain;
+            out.push_back({r.t, y, e, kind, same ? first : 0});
+            y = e;
+        }
+    }
+    return out;
+}
+
+// The runs cut into items of whole iterations, block after block, with at
+// most `m` units of cost a block; returns the blocks this takes.
+int split(const std::vector<Run>& runs, int W, int m, PairPlan* out)
+{
+    int blocks = 1, left = m;
+    if (out) {
+        out->items.clear();
+        out->block_first.assign(1, 0);
+    }
+    auto next_block = [&]() {
+        ++blocks;
+        left = m;
+        if (out) out->block_first.push_back(int(out->items.size()));
+    };
+    for (const Run& r : runs) {
+        const int cost = kCost[r.kind];
+        for (int y = r.ya; y < r.yb;) {
+            if (left < m && left / cost * W - 2 < std::min(r.yb - y, W)) next_block();
+            const int h = std::min(r.yb - y, std::max(left / cost * W - 2, 1));
+            left -= (h + 2 + W - 1) / W * cost;
+            if (out)
+                out->items.push_back(make_int4(r.t.x0, r.t.l0 | (r.t.l1 << 8) | (r.kind >= kPort ? kPairPort : 0) | r.side, y, y + h));
+            y += h;
+        }
+    }
+    if (out) out->block_first.push_back(int(out->items.size()));
+    return blocks;
+}
+
+}  // namespace
+
+PairPlan plan_pairs(const std::vector<uint2>& tiles, const std::vector<RowBC>& bc, int nx, int ny, int pitch,
+                    int precision, int warps, int resident)
+{
+    PairPlan plan;
+    const std::vector<Rows> groups = row_groups(tiles, nx, ny, pitch);
+    const std::vector<Run> runs = split_kinds(strip_runs(groups), groups, tiles, bc, ny);
+    long long cost = 0;
+    int least = 0;
+    for (const Run& r : runs) {
+        cost += (long long)((r.yb - r.ya + 2 + warps - 1) / warps) * kCost[r.kind];
+        least = std::max(least, kCost[r.kind]);
+    }
+    // the least cost of the costliest block for which one wave holds the blocks
+    int m = int(std::max<long long>(least, cost / resident));
+    while (split(runs, warps, m, nullptr) > resident) m += std::max(1, m / 64);
+    split(runs, warps, m, &plan);
+    plan.grid = int(plan.block_first.size()) - 1;
+    // Where two single steps are the better choice (FP32 only): a lattice whose
+    // blocks fill most of the GPU and repeat so many rows that they do more than
+    // 0.85 of the single steps' work, counted in plain rows of 128 nodes.
+    // Measured, single against two-step launches in us a step: 0.59 of the work
+    // 61.2 / 39.3 (4096 x 2048), 0.69 111.3 / 84 (64 chips), 0.81 7.25 / 7.08 (1024 x
+    // 768), 1.2 5.42 / 5.41 (1024 x 512) and 4.90 / 5.12 (700 x 500); a GPU less than
+    // half full: 3.63 / 2.70 (256 x 128), 3.81 / 2.90 (400 x 300).  16-bit storage gains
+    // throughout (37.4 / 29.9, 89.8 / 69.9, 6.20 / 5.58, 5.96 / 5.30, 5.29 / 3.83, 4.81 /
+    // 2.96): its single step is bound by issue and starts up longer.
+    const double work = double(plan.grid) * warps * m / kCost[kPlain];
+    plan.worth = precision != kFP32 || 2 * plan.grid <= resident || work < 0.85 * 2.0 * double(tiles.size());
+    return plan;
+}
+
+}  // namespace lbm
