@@ -146,7 +146,8 @@ typedef struct {
                                steps with unchanged valve words as one cached CUDA graph (captured
                                on first use, at most 16 per handle), which removes the per-launch
                                host cost on small chips.  Results are identical either way. */
-    int32_t scalar_variant; /* kernel of lbm_scalar_step: 0 = default (1), 1 = registers and warp
+    int32_t scalar_variant; /* kernel of lbm_scalar_step: 0 = default (1, and several steps in one
+                               launch), 1 = registers and warp
                                shuffles, 2 = bulk-copy pipeline.  Results are identical. */
     int32_t multi_step;     /* 0 = off; else <= 65536: lbm_step runs up to this many consecutive
                                steps with unchanged valve words in ONE cooperative launch of the
@@ -323,7 +324,9 @@ lbm_status lbm_set_velocity_field(lbm_handle h, uint32_t open_mask, const float*
  * stored for its valve word (lbm_set_valves / lbm_set_valve_schedule)
  * multiplied by u_scale, with the same scalar ports and walls as lbm_step
  * (held concentration, do-nothing, no-flux).  The fluid populations do not
- * change; the step counter advances.  LBM_ERR_STATE (nothing launched) if a
+ * change; the step counter advances.  With scalar_variant 0, steps of one
+ * valve word go three to a launch where that is faster, with the same bits;
+ * the call's last step is always one by itself.  LBM_ERR_STATE (nothing launched) if a
  * valve word the steps use has no stored field.  Diagnostics: out[1] and
  * out[3] of lbm_get_diagnostics come from the last scalar step, out[0] and
  * out[2] stay those of the last coupled step. */

@@ -70,6 +70,7 @@ struct lbm_ctx {
     size_t elem = sizeof(float);
     int cur = 0;   // buffer holding the current state
     int order = 0; // direction of the next single step's tile order (alternates from step to step)
+    int gorder = 0;  // and of the next scalar-only step's
     int gbuf = 0;  // buffer holding the current scalar planes: cur, except after
                    // an odd number of scalar-only steps (joined lazily)
     uint8_t* links = nullptr;
@@ -92,6 +93,11 @@ struct lbm_ctx {
     int partials_cap = 0;  // blocks the partials buffer holds (any launch shape fits)
     int diag_grid = 0;     // blocks whose partials the last step wrote
     int scalar_grid = 0;  // one wave of the scalar-only step kernel (set on first use)
+    std::vector<lbm::RowBC> rowbc_host;
+    bool scalar_levels = false;  // scalar_variant 0: several scalar-only steps a launch where that is faster
+    int4* scalar_items = nullptr;  // their strips, made with the first stored field
+    int* scalar_first = nullptr;
+    int scalar_level_grid = 0;     // 0: none
     bool scalar_regs = true;  // scalar-only step: register variant (else the bulk-copy pipeline)
     int4* pair_items = nullptr;   // the two-step kernel's strips (lbm_pair.cu), its blocks' first strips
     int* pair_first = nullptr;
@@ -308,11 +314,19 @@ cudaError_t launch_full_step(const lbm_ctx* h, const lbm::StepArgs& a, const lbm
     return lbm::launch_step(a, L, s);
 }
 
+// The scalar planes are in the current buffer.
+void join_buffers(lbm_ctx* h)
+{
+    h->gbuf = h->cur;
+    h->gorder = h->order;
+}
+
 // After a step by itself.
 void swap_buffers(lbm_ctx* h)
 {
     h->cur = 1 - h->cur;
     h->order = 1 - h->order;
+    join_buffers(h);
 }
 
 // Two steps in one launch: a holds the first one's arguments (src, dst and
@@ -474,6 +488,7 @@ lbm_status check_ctx(lbm_ctx* h)
 // steps left them in the other buffer (one device copy of 5 planes).
 lbm_status join_scalar(lbm_ctx* h)
 {
+    h->gorder = h->order;
     if (h->gbuf == h->cur) return LBM_OK;
     const size_t off = size_t(9) * h->plane * h->elem;
     char* to = reinterpret_cast<char*>(h->pop[h->cur]) + off;
@@ -840,6 +855,8 @@ lbm_status create_impl(lbm_handle* out, int32_t nx, int32_t ny, const uint8_t* m
     h->elem = opt.precision == LBM_FP32 ? sizeof(float) : sizeof(uint16_t);
     h->graph_steps = opt.graph_steps;
     h->scalar_regs = opt.scalar_variant != 2;
+    h->scalar_levels = opt.scalar_variant == 0 && opt.precision == LBM_FP32 && !batch;
+    if (h->scalar_levels) h->rowbc_host = rowbc;
     h->multi_step = opt.multi_step;
     h->decay = float(opt.decay);
     h->wall_scheme = opt.wall_scheme;
@@ -932,7 +949,7 @@ lbm_status create_impl(lbm_handle* out, int32_t nx, int32_t ny, const uint8_t* m
     // The two-step launches, for handles that leave the step kernel and its
     // launch shape to the library.  One that cannot have them (no tensor maps,
     // no memory for the strips) steps one launch at a time.
-    lbm::PairPlan plan;
+    lbm::StripPlan plan;
     if (opt.variant == 0 && opt.block_threads == 0 && opt.max_blocks == 0 && opt.multi_step == 0 &&
         opt.wall_scheme == LBM_WALL_BOUNCE_BACK && h->pop[0] && h->pop[1]) {
         int pair_per_sm = 0;
@@ -1240,7 +1257,6 @@ lbm_status lbm_step(lbm_handle h, int64_t n)
                     lbm::launch_steps_coop(a, int(m), 0, h->bar, h->coop_grid, kDefaultRegsBlock, h->stream);
                 if (e != cudaSuccess) return cuda_fail(h, e, "multi-step launch");
                 if (m & 1) swap_buffers(h);
-                h->gbuf = h->cur;
                 h->diag_grid = h->coop_grid;
                 h->step += m;
                 k += m;
@@ -1254,7 +1270,7 @@ lbm_status lbm_step(lbm_handle h, int64_t n)
             if (s != LBM_OK) return s;
             LBM_CUDA(h, cudaGraphLaunch(g->exec, h->stream));
             if (g->launches & 1) h->cur = 1 - h->cur;
-            h->gbuf = h->cur;
+            join_buffers(h);
             h->step += G;
             k += G;
             h->diag_grid = h->launch.grid;
@@ -1269,7 +1285,7 @@ lbm_status lbm_step(lbm_handle h, int64_t n)
             cudaError_t e = launch_pair(h, a, next, h->pair_map[h->cur], h->stream);
             if (e != cudaSuccess) return cuda_fail(h, e, "two-step launch");
             h->cur = 1 - h->cur;
-            h->gbuf = h->cur;
+            join_buffers(h);
             h->step += 2;
             k += 2;
             continue;
@@ -1279,7 +1295,6 @@ lbm_status lbm_step(lbm_handle h, int64_t n)
         cudaError_t e = launch_full_step(h, a, h->launch, h->stream);
         if (e != cudaSuccess) return cuda_fail(h, e, "coupled step launch");
         swap_buffers(h);
-        h->gbuf = h->cur;
         h->diag_grid = h->launch.grid;
         ++h->step;
         ++k;
@@ -1329,7 +1344,6 @@ lbm_status lbm_step_diagnostics(lbm_handle h, int64_t n, double* out)
         if (e == cudaSuccess && !fold) e = lbm::launch_diag_finish(h->partials, h->launch.grid, dev + 4 * k, h->stream);
         if (e != cudaSuccess) return cuda_fail(h, e, "coupled step launch");
         swap_buffers(h);
-        h->gbuf = h->cur;
         h->diag_grid = h->launch.grid;
         ++h->step;
     }
@@ -1776,7 +1790,6 @@ lbm_status lbm_adjoint(lbm_handle h, const lbm_objective* obj, int64_t n, int32_
         cudaError_t e = lbm::launch_step(a, h->launch, st);
         if (e != cudaSuccess) return cuda_fail(h, e, "coupled step launch");
         swap_buffers(h);
-        h->gbuf = h->cur;
         h->diag_grid = h->launch.grid;
         h->step += n;
     } else if (K == 1) {
@@ -1793,7 +1806,6 @@ lbm_status lbm_adjoint(lbm_handle h, const lbm_objective* obj, int64_t n, int32_
             if (e != cudaSuccess) return cuda_fail(h, e, "coupled step launch");
         }
         swap_buffers(h);
-        h->gbuf = h->cur;
         h->diag_grid = h->launch.grid;
         h->step += n;
     } else {
@@ -1812,7 +1824,6 @@ lbm_status lbm_adjoint(lbm_handle h, const lbm_objective* obj, int64_t n, int32_
             cudaError_t e = lbm::launch_step(a, h->launch, st);
             if (e != cudaSuccess) return cuda_fail(h, e, "coupled step launch");
             swap_buffers(h);
-            h->gbuf = h->cur;
             h->diag_grid = h->launch.grid;
             ++h->step;
         }
@@ -1838,7 +1849,6 @@ lbm_status lbm_adjoint(lbm_handle h, const lbm_objective* obj, int64_t n, int32_
         cudaError_t e = lbm::launch_step(a, h->launch, st);
         if (e != cudaSuccess) return cuda_fail(h, e, "coupled step launch");
         swap_buffers(h);
-        h->gbuf = h->cur;
         h->diag_grid = h->launch.grid;
         h->step += len;
     }
@@ -1985,6 +1995,35 @@ float* field_slot(lbm_ctx* h, uint32_t word)
     if (u) h->fields.push_back({word, u});
     return u;
 }
+// The strips of the several-steps launches, with the first stored field; a
+// handle that cannot have them steps one launch at a time.
+void plan_scalar_levels(lbm_ctx* h)
+{
+    if (!h->scalar_levels) return;
+    h->scalar_levels = false;  // once
+    int per_sm = 0;
+    CUtensorMap probe;
+    if (lbm::scalar_levels_occupancy(&per_sm) != cudaSuccess || per_sm < 1 ||
+        lbm::scalar_tensor_map(&probe, h->pop[0], lbm::kPlanes, h->ny, h->pitch) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    const lbm::StripPlan p = lbm::plan_scalar(h->tiles_rows, h->rowbc_host, h->nx, h->ny, h->pitch, lbm::kScalarLevels,
+                                              lbm::scalar_level_warps(), per_sm * h->sms);
+    if (!p.worth) return;
+    h->scalar_items = static_cast<int4*>(dev_alloc(h, p.items.size() * sizeof(int4)));
+    h->scalar_first = static_cast<int*>(dev_alloc(h, p.block_first.size() * sizeof(int)));
+    if (!h->scalar_items || !h->scalar_first) return;
+    if (cudaMemcpyAsync(h->scalar_items, p.items.data(), p.items.size() * sizeof(int4), cudaMemcpyHostToDevice,
+                        h->stream) != cudaSuccess ||
+        cudaMemcpyAsync(h->scalar_first, p.block_first.data(), p.block_first.size() * sizeof(int),
+                        cudaMemcpyHostToDevice, h->stream) != cudaSuccess ||
+        cudaStreamSynchronize(h->stream) != cudaSuccess) {  // the host tables go out of scope
+        cudaGetLastError();
+        return;
+    }
+    h->scalar_level_grid = p.grid;
+}
 const float* find_field(const lbm_ctx* h, uint32_t word)
 {
     for (auto& f : h->fields)
@@ -2001,6 +2040,7 @@ lbm_status lbm_store_velocity(lbm_handle h, uint32_t open_mask)
     float* u = field_slot(h, open_mask);
     if (!u) return fail(h, LBM_ERR_OOM, "no room for the velocity field of valve word %u (at most %d fields)",
                         open_mask, LBM_MAX_FIELDS);
+    plan_scalar_levels(h);
     cudaError_t e = lbm::launch_velocity_of_state(h->pop[h->cur], h->links, h->plane, u, u + h->plane, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "velocity kernel launch");
     return LBM_OK;
@@ -2015,6 +2055,7 @@ lbm_status lbm_set_velocity_field(lbm_handle h, uint32_t open_mask, const float*
     float* u = field_slot(h, open_mask);
     if (!u) return fail(h, LBM_ERR_OOM, "no room for the velocity field of valve word %u (at most %d fields)",
                         open_mask, LBM_MAX_FIELDS);
+    plan_scalar_levels(h);
     const size_t row = size_t(h->nx) * sizeof(float), pitch = size_t(h->pitch) * sizeof(float);
     LBM_CUDA(h, cudaMemcpy2DAsync(u, pitch, ux, row, row, size_t(h->ny), cudaMemcpyHostToDevice, h->stream));
     LBM_CUDA(h, cudaMemcpy2DAsync(u + h->plane, pitch, uy, row, row, size_t(h->ny), cudaMemcpyHostToDevice, h->stream));
@@ -2066,7 +2107,8 @@ lbm_status lbm_scalar_step(lbm_handle h, int64_t n, double u_scale)
     const int scalar_grid = std::min(h->scalar_grid, h->partials_cap);
     a.n_partials = std::max(h->diag_grid, scalar_grid);
     int g = h->gbuf;  // buffer holding the current scalar planes
-    for (int64_t k = 0; k < n; ++k) {
+    float2* const partials = a.partials;
+    for (int64_t k = 0; k < n;) {
         const uint32_t w = h->mask_at(h->step);
         const float* u = find_field(h, w);
         if (!u) {
@@ -2075,19 +2117,37 @@ lbm_status lbm_scalar_step(lbm_handle h, int64_t n, double u_scale)
         }
         a.src = h->pop[g] + 9 * h->plane;
         a.dst = h->pop[1 - g] + 9 * h->plane;
-        a.reverse = g;
         a.ux = u;
         a.uy = u + h->plane;
         a.open_mask = w;
-        cudaError_t e = h->scalar_regs
-                            ? lbm::launch_scalar_step_regs(a, scalar_grid, kScalarRegsBlock, h->stream)
-                            : lbm::launch_scalar_step_bulk(a, scalar_grid, kScalarConsumers, kScalarStagesPer, h->stream);
+        // several steps of one valve word in one launch; the call's last step
+        // is always one by itself, which leaves the diagnostics
+        const bool levels = h->scalar_level_grid > 0 && n - k > lbm::kScalarLevels &&
+                            h->mask_run(h->step, lbm::kScalarLevels) == lbm::kScalarLevels;
+        cudaError_t e;
+        if (levels) {
+            a.reverse = g;
+            CUtensorMap map, umap;
+            e = lbm::scalar_tensor_map(&map, h->pop[g], lbm::kPlanes, h->ny, h->pitch);
+            if (e == cudaSuccess) e = lbm::scalar_tensor_map(&umap, const_cast<float*>(u), 2, h->ny, h->pitch);
+            if (e == cudaSuccess)
+                e = lbm::launch_scalar_levels(a, h->scalar_items, h->scalar_first, h->scalar_level_grid, map, umap, h->stream);
+        } else {
+            a.reverse = h->gorder;
+            a.partials = n - k > 1 ? nullptr : partials;  // only the last step's can be read
+            e = h->scalar_regs
+                    ? lbm::launch_scalar_step_regs(a, scalar_grid, kScalarRegsBlock, h->stream)
+                    : lbm::launch_scalar_step_bulk(a, scalar_grid, kScalarConsumers, kScalarStagesPer, h->stream);
+        }
         if (e != cudaSuccess) {
             h->gbuf = g;
             return cuda_fail(h, e, "scalar step launch");
         }
+        const int m = levels ? lbm::kScalarLevels : 1;
         g = 1 - g;
-        ++h->step;
+        h->gorder ^= m & 1;
+        h->step += m;
+        k += m;
     }
     h->gbuf = g;  // joined with the fluid planes when a call needs both
     if (n > 0) h->diag_grid = std::max(h->diag_grid, scalar_grid);

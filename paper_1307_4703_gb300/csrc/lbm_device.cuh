@@ -354,6 +354,27 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
         : "memory");
 }
 
+// Global -> shared tensor copy of a box starting at (x, y, z) of the map,
+// completing on an mbarrier (x a multiple of 16 bytes; what lies outside the
+// tensor arrives as zeros).
+__device__ __forceinline__ void tensor_g2s(void* dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(
+            smem_u32(dst)),
+        "l"(map), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
+        : "memory");
+}
+// Per-lane asynchronous copies of 4 and 8 bytes (cp_async16 copies 16).
+__device__ __forceinline__ void cp_async4(void* dst, const void* src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async8(void* dst, const void* src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+
 // Grid-wide barrier of a cooperative launch (every block resident): thread 0
 // of each block adds one to *count and waits until it reaches target.  The
 // wait is bounded like the mbarrier waits (kWaitCycles, about a second); a

@@ -135,6 +135,9 @@ struct PairArgs {
 };
 cudaError_t pair_occupancy(int precision, int* per_sm);
 int pair_warps(int precision);  // of a block
+// A tensor map of `planes` planes of ny rows of `pitch` elements of `elem`
+// bytes at base, with boxes of cols x rows of one plane.
+cudaError_t rows_tensor_map(CUtensorMap* map, void* base, int planes, int ny, int pitch, int elem, int cols, int rows);
 cudaError_t pair_tensor_map(CUtensorMap* map, void* pop, int ny, int pitch, int precision);
 cudaError_t launch_step_pair(const PairArgs& p, const CUtensorMap& map, int grid, int precision, cudaStream_t s);
 
@@ -207,7 +210,7 @@ struct ScalarArgs {
     float omega_g, wg0, wg1, inv_cs2g;
     float decay;            // k of the reaction term R = -k C (0: none)
     uint32_t open_mask;
-    float2* partials;       // writes slots 1 and 3 of each block's four (double-float pairs)
+    float2* partials;       // writes slots 1 and 3 of each block's four (double-float pairs); null: no diagnostics
     int n_partials;         // entries of `partials` (>= grid); those beyond the grid get 0
     int fluid_blocks;       // entries holding the last coupled step's fluid partials (slots 0, 2);
                             // blocks at or beyond it zero their slots 0 and 2
@@ -221,6 +224,16 @@ cudaError_t scalar_bulk_occupancy(int consumers, int per, int* blocks_per_sm);
 // The register variant of the same step (blocks of `block` threads).
 cudaError_t launch_scalar_step_regs(const ScalarArgs& a, int grid, int block, cudaStream_t s);
 cudaError_t scalar_regs_occupancy(int block, int* blocks_per_sm);
+// kScalarLevels scalar-only steps of one valve word in one launch: strips
+// (items, block_first) as in PairArgs, planned for scalar_level_warps() rows
+// an iteration; map: the source buffer, umap: the stored field's two planes.
+constexpr int kScalarLevels = 3, kScalarWarps = 8, kScalarBlocks = 2;  // steps, warps a block, resident blocks an SM
+int scalar_level_warps();
+// A map of `planes` planes of ny x pitch floats at base for that kernel's copies.
+cudaError_t scalar_tensor_map(CUtensorMap* map, void* base, int planes, int ny, int pitch);
+cudaError_t scalar_levels_occupancy(int* blocks_per_sm);
+cudaError_t launch_scalar_levels(const ScalarArgs& a, const int4* items, const int* block_first, int grid,
+                                 const CUtensorMap& map, const CUtensorMap& umap, cudaStream_t s);
 cudaError_t launch_velocity_of_state(const float* pop, const uint8_t* links, long long plane, float* ux, float* uy,
                                      cudaStream_t s);
 

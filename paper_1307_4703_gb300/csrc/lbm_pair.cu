@@ -103,23 +103,6 @@ __device__ __forceinline__ int box_offset(int x0)
     return sizeof(T) == 4 ? 4 : 4 + (~x0 & 4);
 }
 
-__device__ __forceinline__ void tensor_g2s(void* dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(
-            smem_u32(dst)),
-        "l"(map), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
-        : "memory");
-}
-// Per-lane asynchronous copies of 4 and 8 bytes (cp_async16 copies 16).
-__device__ __forceinline__ void cp_async4(void* dst, const void* src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async8(void* dst, const void* src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
 template <typename T>
 __device__ __forceinline__ void cp_async_quad(T* dst, const T* src)
 {
@@ -511,27 +494,36 @@ cudaError_t pair_occupancy(int precision, int* per_sm)
     return occupancy<float>(per_sm);
 }
 
-cudaError_t pair_tensor_map(CUtensorMap* map, void* pop, int ny, int pitch, int precision)
+int pair_warps(int precision) { return precision == kFP32 ? kPairWarps<float> : kPairWarps<__half>; }
+
+cudaError_t rows_tensor_map(CUtensorMap* map, void* base, int planes, int ny, int pitch, int elem, int cols, int rows)
 {
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult found;
-    cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &found);
-    if (e != cudaSuccess) return e;
-    if (found != cudaDriverEntryPointSuccess) return cudaErrorNotSupported;
-    const cuuint64_t elem = precision == kFP32 ? 4 : 2;
-    const cuuint64_t dims[3] = {cuuint64_t(pitch), cuuint64_t(ny), cuuint64_t(kPlanes)};
+    // looked up once: the driver's entry point, without linking against it
+    static const PFN_cuTensorMapEncodeTiled_v12000 encode = [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        const cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &found);
+        return e == cudaSuccess && found == cudaDriverEntryPointSuccess
+                   ? reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn)
+                   : nullptr;
+    }();
+    if (!encode) return cudaErrorNotSupported;
+    const cuuint64_t dims[3] = {cuuint64_t(pitch), cuuint64_t(ny), cuuint64_t(planes)};
     const cuuint64_t strides[2] = {cuuint64_t(pitch) * elem, cuuint64_t(pitch) * cuuint64_t(ny) * elem};
-    const cuuint32_t box[3] = {cuuint32_t(precision == kFP32 ? kBoxCols<float> : kBoxCols<__half>),
-                               cuuint32_t(precision == kFP32 ? kPairWarps<float> : kPairWarps<__half>), 1};
+    const cuuint32_t box[3] = {cuuint32_t(cols), cuuint32_t(rows), 1};
     const cuuint32_t steps[3] = {1, 1, 1};
-    const CUresult r = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn)(
-        map, precision == kFP32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_UINT16, 3, pop, dims, strides,
-        box, steps, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    const CUresult r = encode(map, elem == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_UINT16, 3, base,
+                              dims, strides, box, steps, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                              CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-int pair_warps(int precision) { return precision == kFP32 ? kPairWarps<float> : kPairWarps<__half>; }
+cudaError_t pair_tensor_map(CUtensorMap* map, void* pop, int ny, int pitch, int precision)
+{
+    const bool f32 = precision == kFP32;
+    return rows_tensor_map(map, pop, kPlanes, ny, pitch, f32 ? 4 : 2, f32 ? kBoxCols<float> : kBoxCols<__half>,
+                           pair_warps(precision));
+}
 
 cudaError_t launch_step_pair(const PairArgs& p, const CUtensorMap& map, int grid, int precision, cudaStream_t s)
 {

@@ -73,13 +73,15 @@ int touched(const std::vector<Strip>& strips, const std::vector<Span>& spans, bo
     return hits;
 }
 
-// What a strip's rows hold.  The costs are of an iteration of the march,
-// measured on the 4096 x 2048 chip and the batch of 64 chips (the splits that
-// were fastest): side walls add the side lanes' work, ports that of a lane
-// that completes its node alone while its warp waits, and walls anywhere a
-// wait for the nodes' own values in global memory.
+// What a strip's rows hold.  The costs are of an iteration of the march (of the
+// two coupled steps, of the scalar-only steps), measured on the 4096 x 2048 chip
+// and the batch of 64 chips (the splits that were fastest): side walls add the
+// side lanes' work, ports that of a lane that completes its node alone while
+// its warp waits, and walls anywhere a wait for the nodes' own values in global
+// memory.
 enum Kind { kPlain, kSide, kScattered, kPort, kScatteredPort };
-constexpr int kCost[5] = {16, 18, 28, 24, 36};
+constexpr int kPairCost[5] = {16, 18, 28, 24, 36};
+constexpr int kScalarCost[5] = {16, 20, 24, 28, 32};
 
 struct Run {
     Strip t;
@@ -163,7 +165,7 @@ std::vector<Run> strip_runs(const std::vector<Rows>& groups)
 // their kinds: scattered walls where more than half of the rows have some
 // within the strip (kWallTile).
 std::vector<Run> split_kinds(const std::vector<Run>& runs, const std::vector<Rows>& groups,
-                             const std::vector<uint2>& tiles, const std::vector<RowBC>& bc, int ny)
+                             const std::vector<uint2>& tiles, const std::vector<RowBC>& bc, int ny, int halo)
 {
     std::vector<Run> out;
     std::vector<int> group_of(static_cast<size_t>(ny));
@@ -185,7 +187,7 @@ std::vector<Run> split_kinds(const std::vector<Run>& runs, const std::vector<Row
             return n == 1 || n == 2 ? lanes | kPairSide : n ? -1 : 0;
         };
         auto port = [&](int y) {
-            for (int yy = std::max(y - 1, 0); yy <= std::min(y + 1, ny - 1); ++yy)
+            for (int yy = std::max(y - halo, 0); yy <= std::min(y + halo, ny - 1); ++yy)
                 for (int s = 0; s < 2; ++s) {
                     const int px = bc[size_t(s) * ny + yy].x;
                     if (px >= x0 && px < x1) return true;
@@ -223,7 +225,7 @@ std::vector<Run> split_kinds(const std::vector<Run>& runs, const std::vector<Row
 
 // The runs cut into items of whole iterations, block after block, with at
 // most `m` units of cost a block; returns the blocks this takes.
-int split(const std::vector<Run>& runs, int W, int m, PairPlan* out)
+int split(const std::vector<Run>& runs, const int (&costs)[5], int halo, int W, int m, StripPlan* out)
 {
     int blocks = 1, left = m;
     if (out) {
@@ -236,11 +238,11 @@ int split(const std::vector<Run>& runs, int W, int m, PairPlan* out)
         if (out) out->block_first.push_back(int(out->items.size()));
     };
     for (const Run& r : runs) {
-        const int cost = kCost[r.kind];
+        const int cost = costs[r.kind];
         for (int y = r.ya; y < r.yb;) {
-            if (left < m && left / cost * W - 2 < std::min(r.yb - y, W)) next_block();
-            const int h = std::min(r.yb - y, std::max(left / cost * W - 2, 1));
-            left -= (h + 2 + W - 1) / W * cost;
+            if (left < m && left / cost * W - 2 * halo < std::min(r.yb - y, W)) next_block();
+            const int h = std::min(r.yb - y, std::max(left / cost * W - 2 * halo, 1));
+            left -= (h + 2 * halo + W - 1) / W * cost;
             if (out)
                 out->items.push_back(make_int4(r.t.x0, r.t.l0 | (r.t.l1 << 8) | (r.kind >= kPort ? kPairPort : 0) | r.side, y, y + h));
             y += h;
@@ -252,35 +254,57 @@ int split(const std::vector<Run>& runs, int W, int m, PairPlan* out)
 
 }  // namespace
 
-PairPlan plan_pairs(const std::vector<uint2>& tiles, const std::vector<RowBC>& bc, int nx, int ny, int pitch,
-                    int precision, int warps, int resident)
+namespace {
+// Strips of the runs over one wave of `resident` blocks.
+StripPlan plan(const std::vector<Run>& runs, const int (&costs)[5], int halo, int warps, int resident)
 {
-    PairPlan plan;
-    const std::vector<Rows> groups = row_groups(tiles, nx, ny, pitch);
-    const std::vector<Run> runs = split_kinds(strip_runs(groups), groups, tiles, bc, ny);
+    StripPlan out;
     long long cost = 0;
     int least = 0;
     for (const Run& r : runs) {
-        cost += (long long)((r.yb - r.ya + 2 + warps - 1) / warps) * kCost[r.kind];
-        least = std::max(least, kCost[r.kind]);
+        cost += (long long)((r.yb - r.ya + 2 * halo + warps - 1) / warps) * costs[r.kind];
+        least = std::max(least, costs[r.kind] * ((1 + 2 * halo + warps - 1) / warps));
     }
     // the least cost of the costliest block for which one wave holds the blocks
     int m = int(std::max<long long>(least, cost / resident));
-    while (split(runs, warps, m, nullptr) > resident) m += std::max(1, m / 64);
-    split(runs, warps, m, &plan);
-    plan.grid = int(plan.block_first.size()) - 1;
+    while (split(runs, costs, halo, warps, m, nullptr) > resident) m += std::max(1, m / 64);
+    split(runs, costs, halo, warps, m, &out);
+    out.grid = int(out.block_first.size()) - 1;
+    // the work of the launch in plain rows of 128 nodes, blocks that end early included
+    out.work = double(out.grid) * warps * m / costs[kPlain];
+    return out;
+}
+
+std::vector<Run> runs_of(const std::vector<uint2>& tiles, const std::vector<RowBC>& bc, int nx, int ny, int pitch, int halo)
+{
+    const std::vector<Rows> groups = row_groups(tiles, nx, ny, pitch);
+    return split_kinds(strip_runs(groups), groups, tiles, bc, ny, halo);
+}
+}  // namespace
+
+StripPlan plan_pairs(const std::vector<uint2>& tiles, const std::vector<RowBC>& bc, int nx, int ny, int pitch,
+                     int precision, int warps, int resident)
+{
+    StripPlan p = plan(runs_of(tiles, bc, nx, ny, pitch, 1), kPairCost, 1, warps, resident);
     // Where two single steps are the better choice (FP32 only): a lattice whose
     // blocks fill most of the GPU and repeat so many rows that they do more than
-    // 0.85 of the single steps' work, counted in plain rows of 128 nodes.
+    // 0.85 of the single steps' work.
     // Measured, single against two-step launches in us a step: 0.59 of the work
-    // 61.2 / 39.3 (4096 x 2048), 0.69 111.3 / 84 (64 chips), 0.81 7.25 / 7.08 (1024 x
+    // 61.2 / 39.3 (4096 x 2048), 0.69 111.3 / 80 (64 chips), 0.81 7.25 / 6.89 (1024 x
     // 768), 1.2 5.42 / 5.41 (1024 x 512) and 4.90 / 5.12 (700 x 500); a GPU less than
-    // half full: 3.63 / 2.70 (256 x 128), 3.81 / 2.90 (400 x 300).  16-bit storage gains
-    // throughout (37.4 / 29.9, 89.8 / 69.9, 6.20 / 5.58, 5.96 / 5.30, 5.29 / 3.83, 4.81 /
-    // 2.96): its single step is bound by issue and starts up longer.
-    const double work = double(plan.grid) * warps * m / kCost[kPlain];
-    plan.worth = precision != kFP32 || 2 * plan.grid <= resident || work < 0.85 * 2.0 * double(tiles.size());
-    return plan;
+    // half full: 3.63 / 2.66 (256 x 128), 3.81 / 2.79 (400 x 300).  16-bit storage gains
+    // throughout (37.4 / 30.1, 89.8 / 67.9, 6.20 / 5.55, 5.96 / 5.25, 5.29 / 3.73, 4.81 /
+    // 2.95): its single step is bound by issue and starts up longer.
+    p.worth = precision != kFP32 || 2 * p.grid <= resident || p.work < 0.85 * 2.0 * double(tiles.size());
+    return p;
+}
+
+StripPlan plan_scalar(const std::vector<uint2>& tiles, const std::vector<RowBC>& bc, int nx, int ny, int pitch, int levels,
+                      int warps, int resident)
+{
+    StripPlan p = plan(runs_of(tiles, bc, nx, ny, pitch, levels - 1), kScalarCost, levels - 1, warps, resident);
+    p.worth = true;
+    return p;
 }
 
 }  // namespace lbm

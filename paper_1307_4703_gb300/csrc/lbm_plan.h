@@ -1,4 +1,5 @@
-// lbm_plan.h -- host-side plan of the two-step kernel (lbm_plan.cu).
+// lbm_plan.h -- host-side plans of the kernels that march several steps along
+// strips (lbm_plan.cu).
 #pragma once
 
 #include <vector>
@@ -7,16 +8,19 @@
 
 namespace lbm {
 
-struct PairPlan {
+struct StripPlan {
     std::vector<int4> items;       // strips (PairArgs::items)
     std::vector<int> block_first;  // grid + 1 entries
     int grid = 0;
-    bool worth = false;            // faster than two single steps
+    double work = 0;
+    bool worth = false;            // faster than single steps
 };
 
 // tiles: the lattice's 128-node tiles in row order; bc: 2 ny port entries;
 // warps: of a block; resident: blocks in one wave.
-PairPlan plan_pairs(const std::vector<uint2>& tiles, const std::vector<RowBC>& bc, int nx, int ny, int pitch,
-                    int precision, int warps, int resident);
+StripPlan plan_pairs(const std::vector<uint2>& tiles, const std::vector<RowBC>& bc, int nx, int ny, int pitch,
+                     int precision, int warps, int resident);
+StripPlan plan_scalar(const std::vector<uint2>& tiles, const std::vector<RowBC>& bc, int nx, int ny, int pitch, int levels,
+                      int warps, int resident);
 
 }  // namespace lbm

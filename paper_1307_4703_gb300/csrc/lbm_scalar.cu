@@ -15,35 +15,22 @@
 namespace lbm {
 namespace {
 
-// Bounce-back, ports, relaxation and stores of one lane's quad.  v: the
-// streamed scalar populations; ux4, uy4: the stored field at the quad; sc,
-// sq: the lane's scalar and outlet-flux sums.
-__device__ __forceinline__ void scalar_quad(float4 (&v)[5], unsigned lk, int x0, const RowBC& bw, const RowBC& be,
-                                            float4 ux4, float4 uy4, const ScalarArgs& a, const float* S, long long P,
-                                            long long oC, KahanF& sc, KahanF& sq, bool& bad)
+// Ports and relaxation of one lane's quad.  v: the pulled scalar populations,
+// walls bounced back, on entry, the post-collision ones on exit; ux4, uy4: the
+// stored field at the quad; own(i, k): the stored population i of node k; sc,
+// sq: the quad's scalar and outlet-flux sums.  kPorts = false: none of the
+// nodes is a port; kAllFluid: none of them is solid either (the selects of the
+// solid nodes are a third of the instructions).
+template <bool kPorts, bool kAllFluid = false, typename Own>
+__device__ __forceinline__ void scalar_nodes(float4 (&v)[5], unsigned lk, int x0, const RowBC& bw, const RowBC& be,
+                                             float4 ux4, float4 uy4, const ScalarArgs& a, const Own& own, float& tc,
+                                             float& tq, bool& bad)
 {
-    // ---- no-flux walls: halfway bounce-back of g ----
-    unsigned wall = 0;
+    const bool open_w = kPorts && bw.x >= 0 && ((a.open_mask >> (bw.chan_kind & 31)) & 1u);
+    const bool open_e = kPorts && be.x >= 0 && ((a.open_mask >> (be.chan_kind & 31)) & 1u);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const unsigned lb = (lk >> (8 * k)) & 0xFFu;
-        if (lb != kSolid) wall |= lb;
-    }
-#pragma unroll
-    for (int i = 1; i <= 4; ++i) {
-        if (wall & (1u << (i - 1))) {
-            const float4 own = ldg4(S + opp(i) * P + oC);
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if ((lk >> (8 * k + i - 1)) & 1u) at(v[i], k) = at(own, k);
-        }
-    }
-    const bool open_w = bw.x >= 0 && ((a.open_mask >> (bw.chan_kind & 31)) & 1u);
-    const bool open_e = be.x >= 0 && ((a.open_mask >> (be.chan_kind & 31)) & 1u);
-    float tc = 0.f, tq = 0.f;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const bool fluid = ((lk >> (8 * k)) & 0xFFu) != kSolid;
+        const bool fluid = kAllFluid || ((lk >> (8 * k)) & 0xFFu) != kSolid;
         float g[5];
 #pragma unroll
         for (int i = 0; i < 5; ++i) g[i] = fluid ? at(v[i], k) : 0.f;
@@ -63,7 +50,7 @@ __device__ __forceinline__ void scalar_quad(float4 (&v)[5], unsigned lk, int x0,
                     if (i != gi) others += g[i];
                 g[gi] = b.c - others;
             } else {          // do-nothing
-                g[gi] = __ldg(S + gi * P + oC + k);
+                g[gi] = own(gi, k);
                 pressure_node = kind != 3;
                 if (kind == 3) {  // the paper's inlet: scaled to C_in
                     const float Cs = ((g[0] + g[1]) + (g[2] + g[3])) + g[4];
@@ -104,6 +91,32 @@ __device__ __forceinline__ void scalar_quad(float4 (&v)[5], unsigned lk, int x0,
             if (pressure_node) tq += C * ux;
         }
     }
+}
+
+// Bounce-back, ports, relaxation and stores of one lane's quad.  v: the
+// streamed scalar populations; sc, sq: the lane's scalar and outlet-flux sums.
+__device__ __forceinline__ void scalar_quad(float4 (&v)[5], unsigned lk, int x0, const RowBC& bw, const RowBC& be,
+                                            float4 ux4, float4 uy4, const ScalarArgs& a, const float* S, long long P,
+                                            long long oC, KahanF& sc, KahanF& sq, bool& bad)
+{
+    // ---- no-flux walls: halfway bounce-back of g ----
+    unsigned wall = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const unsigned lb = (lk >> (8 * k)) & 0xFFu;
+        if (lb != kSolid) wall |= lb;
+    }
+#pragma unroll
+    for (int i = 1; i <= 4; ++i) {
+        if (wall & (1u << (i - 1))) {
+            const float4 own = ldg4(S + opp(i) * P + oC);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if ((lk >> (8 * k + i - 1)) & 1u) at(v[i], k) = at(own, k);
+        }
+    }
+    float tc = 0.f, tq = 0.f;
+    scalar_nodes<true>(v, lk, x0, bw, be, ux4, uy4, a, [&](int i, int k) { return __ldg(S + i * P + oC + k); }, tc, tq, bad);
     sc.add(tc);
     if (tq != 0.f) sq.add(tq);
 #pragma unroll
@@ -114,6 +127,7 @@ __device__ __forceinline__ void scalar_quad(float4 (&v)[5], unsigned lk, int x0,
 // partials (and the bookkeeping of the slots of the coupled step's grid).
 __device__ __forceinline__ void scalar_partials(const ScalarArgs& a, const KahanF& sc, const KahanF& sq)
 {
+    if (a.partials == nullptr) return;  // a step whose diagnostics nothing reads (uniform over the grid)
     __shared__ DF red[32][2];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const DF s1 = warp_sum(sc.pair()), s3 = warp_sum(sq.pair());
@@ -309,6 +323,303 @@ __global__ void __launch_bounds__(128) scalar_frozen_regs(const ScalarArgs a)
     scalar_partials(a, sc, sq);
 }
 
+// ---------------------------------------------------------------------------
+// Several steps in one launch
+// ---------------------------------------------------------------------------
+// kLevels steps of one valve word in one launch, as coupled_step_pair takes
+// two (lbm_pair.cu): a block marches along y over a strip of 128 columns, W
+// rows an iteration; level l takes a row l - 1 rows behind level 1, from the
+// ring of rows level l - 1 has left in shared memory, and the last level
+// stores to the destination buffer.  Strips repeat each other's columns and
+// rows at their sides and ends, so blocks never wait for each other.  Each
+// level spoils one column more from the strip's outer lanes inwards, up to
+// kLevels - 2 of the four of a side lane, none of them stored.
+// What bounds it: three levels move 49 MB a step on the 4096 x 2048 chip (161
+// MB one by one), which HBM would take 8 us for; the levels' turns (barrier,
+// gather from shared memory, arithmetic) at 16 warps an SM take 13.4 us, with
+// 54% of the issue slots used (25.5 us one step a launch, at 0.92 of the HBM
+// rate; 1024 x 768 4.1 -> 3.0, 256 x 128 2.5 -> 1.5).  Tried: four levels (19.2-20.6
+// us: shared memory for 10 or 12 warps only), five (24.4), 6 warps x 3 blocks (16.7
+// where 8 x 2 took 16.5), 4 x 4 (17.3).
+constexpr int kLevels = kScalarLevels, kScalarW = kScalarWarps;
+constexpr int kScalarBox = kTileNodes + 8;  // columns of a staged row: from x0 - 4 on
+struct ScalarRow {
+    float pl[5][kTileNodes];
+};
+struct alignas(16) ScalarInfo {  // what every level needs of a row beside populations
+    float u[2][kTileNodes];
+    unsigned links[kTileNodes / 4];
+    RowBC bc[2];
+};
+struct alignas(128) ScalarSmem {
+    struct alignas(128) Box {
+        float row[kScalarW][kScalarBox];
+    } box[7];                                  // five scalar planes, each at its pull offset, and u_x, u_y
+    ScalarRow ring[kLevels - 1][kScalarW + 2];  // ring l - 1: rows of level l
+    ScalarInfo info[kScalarW + kLevels - 1];
+    struct alignas(16) Stage {
+        unsigned links[kTileNodes / 4];
+        RowBC bc[2];
+    } stage[kScalarW];
+    uint64_t full;  // the boxes have arrived
+    uint64_t step;  // every warp has left its row of a level: kLevels - 1 phases an iteration
+};
+static_assert(offsetof(ScalarSmem, ring) % 16 == 0 && offsetof(ScalarSmem, info) % 16 == 0 &&
+                  offsetof(ScalarSmem, stage) % 16 == 0 && offsetof(ScalarSmem, full) % 8 == 0 &&
+                  sizeof(ScalarSmem::Box) % 128 == 0 && sizeof(ScalarInfo) % 16 == 0 && sizeof(ScalarRow) % 16 == 0 &&
+                  offsetof(ScalarInfo, links) % 16 == 0 && offsetof(ScalarInfo, bc) % 16 == 0,
+              "targets of vector accesses, copies and barriers");
+static_assert(kLevels >= 3 && kLevels <= 5, "with two levels a row would be rewritten while it may still be read");
+
+// Free flight of one lane's quad from three rows (lanes 0 and 31 take no
+// value from beyond the strip: see above).
+template <typename RowOf>
+__device__ __forceinline__ void pull_rows(float4 (&v)[5], const RowOf& row, int lane)
+{
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        float4 r = *reinterpret_cast<const float4*>(row(i) + 4 * lane);
+        if (src_col(i) == 1) r = make_float4(__shfl_up_sync(kFull, r.w, 1), r.x, r.y, r.z);
+        else if (src_col(i) == 2) r = make_float4(r.y, r.z, r.w, __shfl_down_sync(kFull, r.x, 1));
+        v[i] = r;
+    }
+}
+
+__device__ __forceinline__ void bounce_link(float4& v, unsigned lk, int i, const float4& own)
+{
+#pragma unroll
+    for (int k = 0; k < 4; ++k) at(v, k) = (lk >> (8 * k + i - 1)) & 1u ? at(own, k) : at(v, k);
+}
+
+__global__ void __launch_bounds__(32 * kScalarW, kScalarBlocks)
+    scalar_frozen_levels(const ScalarArgs a, const int4* items, const int* block_first,
+                         const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap umap)
+{
+    constexpr int W = kScalarW, K = kLevels, R = W + 2, RI = W + K - 1;
+    extern __shared__ __align__(128) unsigned char smem[];
+    ScalarSmem& sm = *reinterpret_cast<ScalarSmem*>(smem);
+    const int lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5;
+    const int reverse = a.reverse, pitch = a.pitch, ny = a.ny;
+    const long long P = a.plane;
+    ScalarSmem::Stage& stage = sm.stage[warp];
+    bool bad = false, late = false;
+
+    if (threadIdx.x == 0) {
+        mbar_init(&sm.full, 1);
+        mbar_init(&sm.step, W);
+        mbar_fence_init();
+    }
+    int i = block_first[blockIdx.x];
+    const int i_end = block_first[blockIdx.x + 1];
+    int4 st = items[i];
+    __syncthreads();
+    grid_dependency_sync();
+
+    // march row j of the strip's level 1: rows ya - (K - 1) .. yb + K - 2
+    auto row_of = [&](const int4& s, int j) { return reverse ? s.w + K - 2 - j : s.z - (K - 1) + j; };
+    auto total = [&](const int4& s) { return s.w - s.z + 2 * (K - 1); };
+    auto inside = [&](int y) { return y >= 0 && y < ny; };
+    auto issue_boxes = [&](const int4& s, int j) {
+        if (threadIdx.x != 0) return;
+        const int y = reverse ? row_of(s, j + W - 1) : row_of(s, j);  // lowest row
+        mbar_arrive_expect_tx(&sm.full, uint32_t(7 * W * kScalarBox * sizeof(float)));
+#pragma unroll
+        for (int q = 0; q < 5; ++q)
+            tensor_g2s(&sm.box[q], &map, s.x - 4, y - (src_row(q) == 1) + (src_row(q) == 2), 9 + q, &sm.full);
+        for (int q = 0; q < 2; ++q) tensor_g2s(&sm.box[5 + q], &umap, s.x - 4, y, q, &sm.full);
+    };
+    auto issue_row = [&](const int4& s, int y) {
+        const int l0 = s.y & 0xFF, l1 = (s.y >> 8) & 0xFF;
+        if (lane >= l0 - 1 && lane <= l1 + 1)
+            cp_async4(&stage.links[lane], a.links + (long long)y * pitch + s.x + 4 * lane);
+        if ((s.y & kPairPort) && lane < 2) cp_async16(&stage.bc[lane], a.rowbc + (lane == 0 ? y : ny + y));
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+
+    unsigned issued = 1, phase = 0;
+    issue_boxes(st, 0);
+    bool here = inside(row_of(st, warp)) && warp < total(st);
+    if (here) issue_row(st, row_of(st, warp));
+
+    int base = 0;             // first march row of the iteration
+    int sp = warp, ip = warp;  // ring and info slots of the warp's level-1 row
+    for (unsigned t = 0;; ++t) {
+        const int j = base + warp, n_rows = total(st);
+        const int l0 = st.y & 0xFF, l1 = (st.y >> 8) & 0xFF;
+        const bool port = st.y & kPairPort;
+        const int x0 = st.x + 4 * lane;
+        int4 nst = st;
+        int nbase = base + W;
+        bool more = true;
+        if (nbase >= n_rows) {
+            nbase = 0;
+            more = i + 1 < i_end;
+            if (more) nst = items[i + 1];
+        }
+        const int yn = row_of(nst, nbase + warp);
+        const bool next = more && nbase + warp < total(nst) && inside(yn);
+
+        // ---- level 1, from the boxes ----
+        if (!late) late = !mbar_wait(&sm.full, t & 1u);
+        float4 v[5], ux4, uy4;
+        unsigned lk = 0xFFFFFFFFu;
+        RowBC bc[2];
+        const int y1 = row_of(st, j), r = reverse ? W - 1 - warp : warp;
+        if (here) {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            __syncwarp();
+            auto row = [&](int q) { return &sm.box[q].row[r][4]; };
+            pull_rows(v, row, lane);
+            if (lane == 0) v[1].x = sm.box[1].row[r][3];
+            if (lane == 31) v[3].w = sm.box[3].row[r][4 + kTileNodes];
+            ux4 = *reinterpret_cast<const float4*>(row(5) + 4 * lane);
+            uy4 = *reinterpret_cast<const float4*>(row(6) + 4 * lane);
+            if (lane >= l0 - 1 && lane <= l1 + 1) lk = stage.links[lane];
+            if (port) {
+                bc[0] = stage.bc[0];
+                bc[1] = stage.bc[1];
+            }
+        }
+        late = __any_sync(kFull, late);
+        if (next && !late) issue_row(nst, yn);
+        ScalarInfo& info = sm.info[ip];
+        if (here) {
+            // this warp was the slot's last reader (level K of the iteration before)
+            *reinterpret_cast<float4*>(&info.u[0][4 * lane]) = ux4;
+            *reinterpret_cast<float4*>(&info.u[1][4 * lane]) = uy4;
+            info.links[lane] = lk;
+            if (port && lane < 2) info.bc[lane] = bc[lane];
+        }
+        const bool open1 = __all_sync(kFull, lk == 0u || lk == 0xFFFFFFFFu);  // a row without walls
+        if (lk != 0xFFFFFFFFu && open1) {
+            float tc = 0.f, tq = 0.f;
+            bool b = false;
+            scalar_nodes<false, true>(v, lk, x0, RowBC{}, RowBC{}, ux4, uy4, a, [](int, int) { return 0.f; }, tc, tq, b);
+            bad |= b && lane >= l0 && lane <= l1;
+        } else if (lk != 0xFFFFFFFFu) {
+            // walls: along the row from the box, which holds the row's own values of
+            // directions 1 and 3; across it from global memory
+            const float4 g1 = *reinterpret_cast<const float4*>(&sm.box[1].row[r][4 + 4 * lane]);
+            const float4 g3 = *reinterpret_cast<const float4*>(&sm.box[3].row[r][4 + 4 * lane]);
+            unsigned wall = 0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const unsigned lb = (lk >> (8 * k)) & 0xFFu;
+                if (lb != kSolid) wall |= lb;
+            }
+            if (wall & 0x5u) {
+                bounce_link(v[1], lk, 1, g3);
+                bounce_link(v[3], lk, 3, g1);
+            }
+            if (wall & 0xAu) {
+                const long long o = (long long)y1 * pitch + x0;
+                const float4 g4 = ldg4(a.src + 4 * P + o), g2 = ldg4(a.src + 2 * P + o);
+                bounce_link(v[2], lk, 2, g4);
+                bounce_link(v[4], lk, 4, g2);
+            }
+            float tc = 0.f, tq = 0.f;
+            bool b = false;
+            auto own = [&](int q, int k) { return q == 1 ? at(g1, k) : at(g3, k); };
+            if (port) scalar_nodes<true>(v, lk, x0, bc[0], bc[1], ux4, uy4, a, own, tc, tq, b);
+            else scalar_nodes<false>(v, lk, x0, RowBC{}, RowBC{}, ux4, uy4, a, own, tc, tq, b);
+            bad |= b && lane >= l0 && lane <= l1;
+        }
+        if (lk != 0xFFFFFFFFu) {
+            ScalarRow& out = sm.ring[0][sp];
+#pragma unroll
+            for (int q = 0; q < 5; ++q) *reinterpret_cast<float4*>(&out.pl[q][4 * lane]) = v[q];
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.step);
+        if (!late) late = !mbar_wait(&sm.step, phase & 1u);
+        ++phase;
+        if (more && !late) {  // every warp has pulled its row from the boxes
+            issue_boxes(nst, nbase);
+            ++issued;
+        }
+
+        // ---- levels 2 .. K: row j - (l - 1) from the ring of level l - 1 ----
+#pragma unroll
+        for (int l = 2; l <= K; ++l) {
+            const int jl = j - (l - 1), yl = row_of(st, jl);
+            const bool on = j >= 2 * (l - 1) && j < n_rows && inside(yl);
+            int sc = sp - (l - 1), ic = ip - (l - 1);  // slots of row j - (l - 1)
+            if (sc < 0) sc += R;
+            if (ic < 0) ic += RI;
+            const int sa = sc == R - 1 ? 0 : sc + 1, sb = sc == 0 ? R - 1 : sc - 1;  // rows one on and one back
+            lk = 0xFFFFFFFFu;
+            if (on) {
+                const ScalarRow* ring = sm.ring[l - 2];
+                const ScalarInfo& in = sm.info[ic];
+                const ScalarRow& rS = ring[reverse ? sa : sb];
+                const ScalarRow& rN = ring[reverse ? sb : sa];
+                const ScalarRow& rC = ring[sc];
+                auto row = [&](int q) { return src_row(q) == 0 ? rC.pl[q] : src_row(q) == 1 ? rS.pl[q] : rN.pl[q]; };
+                pull_rows(v, row, lane);
+                const int w = l < K ? 1 : 0;
+                if (lane >= l0 - w && lane <= l1 + w) lk = in.links[lane];
+                ux4 = *reinterpret_cast<const float4*>(&in.u[0][4 * lane]);
+                uy4 = *reinterpret_cast<const float4*>(&in.u[1][4 * lane]);
+                float tc = 0.f, tq = 0.f;
+                bool b = false;
+                if (__all_sync(kFull, lk == 0u || lk == 0xFFFFFFFFu)) {
+                    if (lk == 0u)
+                        scalar_nodes<false, true>(v, lk, x0, RowBC{}, RowBC{}, ux4, uy4, a, [](int, int) { return 0.f; }, tc,
+                                                  tq, b);
+                } else if (lk != 0xFFFFFFFFu) {
+                    unsigned wall = 0;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const unsigned lb = (lk >> (8 * k)) & 0xFFu;
+                        if (lb != kSolid) wall |= lb;
+                    }
+                    if (wall & 0xFu) {
+#pragma unroll
+                        for (int q = 1; q <= 4; ++q)
+                            bounce_link(v[q], lk, q, *reinterpret_cast<const float4*>(&rC.pl[opp(q)][4 * lane]));
+                    }
+                    auto own = [&](int q, int k) { return rC.pl[q][4 * lane + k]; };
+                    if (port) scalar_nodes<true>(v, lk, x0, in.bc[0], in.bc[1], ux4, uy4, a, own, tc, tq, b);
+                    else scalar_nodes<false>(v, lk, x0, RowBC{}, RowBC{}, ux4, uy4, a, own, tc, tq, b);
+                }
+                bad |= b && lane >= l0 && lane <= l1 && yl >= st.z && yl < st.w;
+            }
+            if (l < K) {
+                if (lk != 0xFFFFFFFFu) {
+                    ScalarRow& out = sm.ring[l - 1][sc];
+#pragma unroll
+                    for (int q = 0; q < 5; ++q) *reinterpret_cast<float4*>(&out.pl[q][4 * lane]) = v[q];
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sm.step);
+                if (!late) late = !mbar_wait(&sm.step, phase & 1u);
+                ++phase;
+            } else if (lk != 0xFFFFFFFFu) {
+                float* const D = a.dst + (long long)yl * pitch + x0;
+#pragma unroll
+                for (int q = 0; q < 5; ++q) stg4(D + q * P, v[q]);
+            }
+        }
+        if (!more) break;
+        if (nbase == 0) ++i;
+        st = nst;
+        base = nbase;
+        here = next;
+        sp += W;
+        if (sp >= R) sp -= R;
+        ip += W;
+        if (ip >= RI) ip -= RI;
+    }
+    if (late) {
+        // no copy may still be writing this block's shared memory at exit
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        mbar_wait(&sm.full, (issued - 1) & 1u);
+        atomicOr(a.err, 2u);
+    }
+    if (__any_sync(kFull, bad) && lane == 0) atomicOr(a.err, 1u);
+}
+
 // Velocity of the stored populations (f as deviations) into two planes.
 __global__ void velocity_of_state(const float* pop, const uint8_t* links, long long plane, int n, float* ux,
                                   float* uy)
@@ -386,6 +697,40 @@ cudaError_t launch_scalar_step_regs(const ScalarArgs& a, int grid, int block, cu
 cudaError_t scalar_regs_occupancy(int block, int* blocks_per_sm)
 {
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, scalar_frozen_regs, block, 0);
+}
+
+int scalar_level_warps() { return kScalarW; }
+
+cudaError_t scalar_tensor_map(CUtensorMap* map, void* base, int planes, int ny, int pitch)
+{
+    return rows_tensor_map(map, base, planes, ny, pitch, sizeof(float), kScalarBox, kScalarW);
+}
+
+cudaError_t scalar_levels_occupancy(int* blocks_per_sm)
+{
+    cudaError_t e = cudaFuncSetAttribute(scalar_frozen_levels, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         int(sizeof(ScalarSmem)));
+    if (e != cudaSuccess) return e;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, scalar_frozen_levels, 32 * kScalarW,
+                                                         sizeof(ScalarSmem));
+}
+
+cudaError_t launch_scalar_levels(const ScalarArgs& a, const int4* items, const int* block_first, int grid,
+                                 const CUtensorMap& map, const CUtensorMap& umap, cudaStream_t s)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(32 * kScalarW);
+    cfg.dynamicSmemBytes = sizeof(ScalarSmem);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, scalar_frozen_levels, a, items, block_first, map, umap);
+    if (e != cudaSuccess) return e;
+    return cudaGetLastError();
 }
 
 cudaError_t launch_velocity_of_state(const float* pop, const uint8_t* links, long long plane, float* ux, float* uy,
