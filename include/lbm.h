@@ -360,7 +360,10 @@ typedef struct {
  * take 117 GB).
  * Device memory: ceil(n_steps / ckpt_every) + ckpt_every - 1 population
  * copies and three adjoint buffers, taken through the handle's allocator
- * and released before returning (LBM_ERR_OOM if they do not fit).  The
+ * hooks and released before returning (LBM_ERR_OOM if they do not fit);
+ * without hooks, from a memory pool of the device that all handles share and
+ * that keeps at most 1/16 of the device's memory between calls, and nothing
+ * once the handles that have used it are destroyed.  The
  * derivatives are accumulated in FP64 (d/d(1/tau_c): compensated FP32 per
  * lane and double-float pairs within a block for each reverse step, FP64
  * across blocks and steps); the adjoint populations are FP32.
