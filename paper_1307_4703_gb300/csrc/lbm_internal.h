@@ -260,6 +260,9 @@ cudaError_t step_walls_occupancy(const StepLaunch& l, int* blocks_per_sm);
 cudaError_t prepare_walls_kernels();
 
 cudaError_t launch_diag_finish(const float2* partials, int n_blocks, double* out, cudaStream_t s);
+// The totals of `rows` steps at once, out[4 j ..] for step j: sets of n_blocks
+// partials one after the other, the last step's at `last`.
+cudaError_t launch_diag_rows(const float2* sets, const float2* last, int n_blocks, int rows, double* out, cudaStream_t s);
 // A step that also forms its totals in its last block (a.diag_out set):
 // variants 1 and 4 without the paper's walls (lbm_fold_steps.cu); cfg is the
 // step's launch configuration.  Other launch shapes return

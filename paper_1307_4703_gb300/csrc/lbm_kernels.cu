@@ -47,6 +47,15 @@ __global__ void diag_finish(const float2* partials, int n_blocks, double* out)
     finish_partials(partials, n_blocks, out);
 }
 
+// The same for several steps: block j forms the totals of step j, whose
+// partials are the j-th set of n_blocks; the last step's are at `last`.
+__global__ void diag_rows(const float2* sets, const float2* last, int n_blocks, double* out)
+{
+    grid_dependency_sync();
+    const int j = blockIdx.x;
+    finish_partials(j + 1 < int(gridDim.x) ? sets + (long long)j * 4 * n_blocks : last, n_blocks, out + 4 * j);
+}
+
 // Many steps in one cooperative launch (every block resident): the register
 // variant's tile loop once per step, the two buffers swapping roles (or,
 // with seq_stride > 0, step s reading src + s seq_stride and writing the
@@ -497,18 +506,33 @@ size_t async_smem_bytes(int block, int precision)
     return per_warp * size_t(block / 32);
 }
 
-cudaError_t launch_diag_finish(const float2* partials, int n_blocks, double* out, cudaStream_t s)
+static cudaLaunchConfig_t dependent(cudaLaunchAttribute (&attr)[1], int grid, int block, cudaStream_t s)
 {
-    // a programmatic dependent of the step before it, like the steps
+    // a programmatic dependent of the kernel before it
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(1);
-    cfg.blockDim = dim3(kFoldThreads);
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+    return cfg;
+}
+
+cudaError_t launch_diag_rows(const float2* sets, const float2* last, int n_blocks, int rows, double* out, cudaStream_t s)
+{
+    cudaLaunchAttribute attr[1];
+    const cudaLaunchConfig_t cfg = dependent(attr, rows, kFoldThreads, s);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, diag_rows, sets, last, n_blocks, out);
+    if (e != cudaSuccess) return e;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_diag_finish(const float2* partials, int n_blocks, double* out, cudaStream_t s)
+{
+    cudaLaunchAttribute attr[1];
+    const cudaLaunchConfig_t cfg = dependent(attr, 1, kFoldThreads, s);
     cudaError_t e = cudaLaunchKernelEx(&cfg, diag_finish, partials, n_blocks, out);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
