@@ -152,8 +152,8 @@ struct lbm_ctx {
     float decay = 0.f;         // k of the reaction term R = -k C
     int wall_scheme = 0;       // LBM_WALL_BOUNCE_BACK or LBM_WALL_EQUILIBRIUM
     void* wallv = nullptr;     // the paper's walls: 8 planes of wall values for the step
-    long long* woff = nullptr; // offsets of the fluid nodes with wall links
-    int n_wall = 0;
+    lbm::WallLink* wall_list = nullptr;  // the links it holds values of
+    long long n_wall = 0;
     bool paper_ports = false;  // some port has a rescaling kind (no adjoint)
     std::vector<Graph> graphs;
 
@@ -372,7 +372,7 @@ bool is_fluid(const uint8_t* mask, int nx, int ny, int x, int y)
 cudaError_t launch_full_step(const lbm_ctx* h, const lbm::StepArgs& a, const lbm::StepLaunch& L, cudaStream_t s)
 {
     if (h->wallv) {
-        cudaError_t e = lbm::launch_wall_values(a.src, h->wallv, h->links, h->woff, h->n_wall, h->plane, h->pitch,
+        cudaError_t e = lbm::launch_wall_values(a.src, h->wallv, h->wall_list, h->n_wall, h->plane, h->pitch,
                                                 h->precision, s);
         if (e != cudaSuccess) return e;
     }
@@ -1036,17 +1036,31 @@ lbm_status create_impl(lbm_handle* out, int32_t nx, int32_t ny, const uint8_t* m
             h->pairs = plan.worth;
         }
     }
-    std::vector<long long> woff;
+    std::vector<lbm::WallLink> wall_list;
     if (opt.wall_scheme == LBM_WALL_EQUILIBRIUM) {
-        for (size_t o = 0; o < links.size(); ++o)
-            if (links[o] != 0 && links[o] != lbm::kSolid) woff.push_back((long long)o);
-        h->n_wall = int(woff.size());
+        static const int ex[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1}, ey[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
+        for (size_t o = 0; o < links.size(); ++o) {
+            if (links[o] == 0 || links[o] == lbm::kSolid) continue;
+            for (int i = 1; i <= 8; ++i) {
+                if (!((links[o] >> (i - 1)) & 1)) continue;
+                // bit of "x + e_i is not fluid": the source of the opposite direction
+                const int back = i <= 4 ? (i + 1) & 3 : ((i - 3) & 3) + 4;
+                int ahead = 0;
+                if (!((links[o] >> back) & 1)) {
+                    const size_t o1 = size_t((long long)o + ex[i] + (long long)ey[i] * pitch);
+                    ahead = (links[o1] >> back) & 1 ? 1 : 2;
+                }
+                wall_list.push_back({(long long)o, i, ahead});
+            }
+        }
+        h->n_wall = (long long)wall_list.size();
         h->wallv = dev_alloc(h, size_t(8) * h->plane * h->elem);
-        h->woff = static_cast<long long*>(dev_alloc(h, std::max<size_t>(1, woff.size()) * sizeof(long long)));
+        h->wall_list = static_cast<lbm::WallLink*>(
+            dev_alloc(h, std::max<size_t>(1, wall_list.size()) * sizeof(lbm::WallLink)));
     }
     if (!h->pop[0] || !h->pop[1] || !h->links || !h->rowbc || !h->tiles || !h->tiles64 || !h->partials ||
         !h->err || !h->diag || !h->fields_tmp || (batch && !h->rates) ||
-        (opt.wall_scheme == LBM_WALL_EQUILIBRIUM && (!h->wallv || !h->woff)))
+        (opt.wall_scheme == LBM_WALL_EQUILIBRIUM && (!h->wallv || !h->wall_list)))
         return bail(fail(h, LBM_ERR_OOM, "device allocation of %zu bytes failed", 2 * pop_bytes));
     if (batch) h->inst = batch->inst;
 
@@ -1063,8 +1077,9 @@ lbm_status create_impl(lbm_handle* out, int32_t nx, int32_t ny, const uint8_t* m
                             cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess && batch)
         e = cudaMemcpyAsync(h->rates, batch->rates.data(), size_t(ny) * sizeof(float4), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess && !woff.empty())
-        e = cudaMemcpyAsync(h->woff, woff.data(), woff.size() * sizeof(long long), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess && !wall_list.empty())
+        e = cudaMemcpyAsync(h->wall_list, wall_list.data(), wall_list.size() * sizeof(lbm::WallLink),
+                            cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->err, 0, 2 * sizeof(unsigned), st);
     if (e == cudaSuccess)
         e = cudaMemsetAsync(h->partials, 0, size_t(h->partials_cap) * 4 * sizeof(float2), st);
@@ -2307,7 +2322,7 @@ lbm_status lbm_autotune(lbm_handle h, int32_t trial_steps)
     }
     h->mask_words(h->step, a.open_mask);
     if (h->wallv)
-        LBM_CUDA(h, lbm::launch_wall_values(a.src, h->wallv, h->links, h->woff, h->n_wall, h->plane, h->pitch,
+        LBM_CUDA(h, lbm::launch_wall_values(a.src, h->wallv, h->wall_list, h->n_wall, h->plane, h->pitch,
                                             h->precision, h->stream));
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     LBM_CUDA(h, cudaEventCreate(&e0));

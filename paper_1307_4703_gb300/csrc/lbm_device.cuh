@@ -579,37 +579,26 @@ __device__ __forceinline__ void node_moments(const T* S, long long P, long long 
 }
 
 // The paper's wall ("Boundary Conditions") for population i of the fluid
-// node at offset own, whose source x - e_i is not fluid (lb: the node's
-// wall-link byte, bit j-1 set = the source x - e_j is not fluid): the
-// equilibrium, as a deviation f_eq - w_i, of a density extrapolated to first
-// order from the fluid along e_i, 2 rho(x + e_i) - rho(x + 2 e_i), and the
-// momentum interpolated between zero at the wall, half a link behind the
-// node, and x + e_i, one and a half links from it: j(x + e_i) / 3.  Moments
-// of the stored state S (the start of the step).  Where x + 2 e_i is not
-// fluid the density is that of x + e_i; where x + e_i is not fluid either,
-// the node's own density with zero momentum.
+// node at offset own, whose source x - e_i is not fluid: the equilibrium, as a
+// deviation f_eq - w_i, of a density extrapolated to first order from the
+// fluid along e_i, 2 rho(x + e_i) - rho(x + 2 e_i), and the momentum
+// interpolated between zero at the wall, half a link behind the node, and
+// x + e_i, one and a half links from it: j(x + e_i) / 3.  Moments of the stored
+// state S (the start of the step).  `ahead` = 2: both nodes are fluid; 1: x + 2
+// e_i is not, and the density is that of x + e_i; 0: x + e_i is not fluid
+// either, and the node's own density comes with zero momentum.
 template <typename T>
-__device__ __forceinline__ float equilibrium_wall(int i, unsigned lb, const T* S, const uint8_t* links, long long P,
-                                                  long long own, int pitch)
+__device__ __forceinline__ float equilibrium_wall(int i, int ahead, const T* S, long long P, long long own, int pitch)
 {
-    const int back = opp(i) - 1;  // bit of "x + e_i is not fluid"
+    const long long step = dir_x(i) + (long long)dir_y(i) * pitch;
     float rd, jx = 0.f, jy = 0.f;
-    if (!((lb >> back) & 1u)) {
-        const long long o1 = own + dir_x(i) + (long long)dir_y(i) * pitch;
-        float r1, x1, y1;
-        node_moments(S, P, o1, r1, x1, y1);
-        if (!((links[o1] >> back) & 1u)) {
-            float r2, x2, y2;
-            node_moments(S, P, o1 + dir_x(i) + (long long)dir_y(i) * pitch, r2, x2, y2);
-            rd = 2.f * r1 - r2;  // 2 rho1 - rho2 - 1
-        } else {
-            rd = r1;
-        }
+    float r1, x1, y1, r2 = 0.f, x2, y2;
+    node_moments(S, P, ahead ? own + step : own, r1, x1, y1);
+    if (ahead == 2) node_moments(S, P, own + 2 * step, r2, x2, y2);
+    rd = ahead == 2 ? 2.f * r1 - r2 : r1;  // 2 rho1 - rho2 - 1
+    if (ahead) {
         jx = x1 * (1.f / 3.f);
         jy = y1 * (1.f / 3.f);
-    } else {
-        float ox, oy;
-        node_moments(S, P, own, rd, ox, oy);
     }
     const float rho = 1.f + rd;
     const float ux = jx / rho, uy = jy / rho;

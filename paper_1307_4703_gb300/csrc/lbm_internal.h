@@ -244,21 +244,26 @@ size_t async_smem_bytes(int block, int precision);
 int bulk_stage_bytes(int precision = 0);
 cudaError_t prepare_step_kernels();
 cudaError_t launch_step(const StepArgs& a, const StepLaunch& l, cudaStream_t s);
-// out[0..3] = sum of the n_blocks x 4 block partials, in a fixed order.
+// One missing population of the paper's walls: population i of the fluid node
+// at offset o, and how many of the nodes x + e_i, x + 2 e_i in turn are fluid.
+struct alignas(16) WallLink {
+    long long o;
+    int i, ahead;
+};
 // The paper's wall values for the step that reads src (lbm_device.cuh,
-// equilibrium_wall): for every fluid node with wall links (offsets
-// woff[0..n)), the value of each population i whose source is not fluid
-// goes to plane i - 1 of W (8 planes of the storage type), which the step
-// kernels' kWalls instantiations read instead of bounce-back.  A
-// programmatic dependent of the previous kernel.
-cudaError_t launch_wall_values(const void* src, void* W, const uint8_t* links, const long long* woff, int n,
-                               long long plane, int pitch, int precision, cudaStream_t s);
+// equilibrium_wall): the value of each of the n links goes to plane i - 1 of W
+// (8 planes of the storage type), which the step kernels' kWalls
+// instantiations read instead of bounce-back.  A programmatic dependent of the
+// previous kernel.
+cudaError_t launch_wall_values(const void* src, void* W, const WallLink* list, long long n, long long plane,
+                               int pitch, int precision, cudaStream_t s);
 
 // The step kernels with the paper's walls (lbm_walls.cu): variants 1 and 2.
 cudaError_t launch_step_walls(const StepArgs& a, const StepLaunch& l, cudaStream_t s);
 cudaError_t step_walls_occupancy(const StepLaunch& l, int* blocks_per_sm);
 cudaError_t prepare_walls_kernels();
 
+// out[0..3] = sum of the n_blocks x 4 block partials, in a fixed order.
 cudaError_t launch_diag_finish(const float2* partials, int n_blocks, double* out, cudaStream_t s);
 // The totals of `rows` steps at once, out[4 j ..] for step j: sets of n_blocks
 // partials one after the other, the last step's at `last`.

@@ -369,45 +369,57 @@ int elementwise_grid(long long n)
     return int(want < 65536 ? want : 65536);
 }
 
-// The paper's wall values of one step (see launch_wall_values).
+// The paper's wall values of one step (see launch_wall_values), a thread a
+// link.  Bound by latency (a chip has a few thousand links): a link's entry
+// says which nodes ahead of it are fluid, so the loads of both nodes'
+// populations go out together and wait for the entry alone, which is read
+// before the previous kernel ends.  A step with its wall values takes 8.5 us on
+// the 1024 x 512 chip, 6.1 on 256 x 128 and 68.8 on 4096 x 2048; a thread a
+// node, with its links and their masks looked up in turn, made that 17.5, 13.7
+// and 83.  Blocks of 32 or 128 (8.5, 9.0 at 1024 x 512) and letting the step
+// start before the wait (8.9) are no better.
 template <typename T>
-__global__ void wall_values(const T* S, T* W, const uint8_t* links, const long long* woff, int n, long long P,
-                            int pitch)
+__global__ void __launch_bounds__(64) wall_values(const T* S, T* W, const WallLink* list, long long n, long long P,
+                                                   int pitch)
 {
+    const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    WallLink l{};
+    if (e < n) l = list[e];
     grid_dependency_sync();
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
-        const long long o = woff[e];
-        const unsigned lb = links[o];
-        for (int i = 1; i < 9; ++i)
-            if ((lb >> (i - 1)) & 1u)
-                Codec<T>::st1(W + (i - 1) * P + o, equilibrium_wall(i, lb, S, links, P, o, pitch), 0.f);
-    }
+    if (e < n) Codec<T>::st1(W + (l.i - 1) * P + l.o, equilibrium_wall(l.i, l.ahead, S, P, l.o, pitch), 0.f);
 }
 
 }  // namespace
 
-cudaError_t launch_wall_values(const void* src, void* W, const uint8_t* links, const long long* woff, int n,
-                               long long plane, int pitch, int precision, cudaStream_t s)
+static cudaLaunchConfig_t dependent(cudaLaunchAttribute (&attr)[1], int grid, int block, cudaStream_t s)
 {
+    // a programmatic dependent of the kernel before it
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(unsigned(std::max(1, std::min((n + 255) / 256, 4096))));
-    cfg.blockDim = dim3(256);
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+    return cfg;
+}
+
+cudaError_t launch_wall_values(const void* src, void* W, const WallLink* list, long long n, long long plane,
+                               int pitch, int precision, cudaStream_t s)
+{
+    cudaLaunchAttribute attr[1];
+    const cudaLaunchConfig_t cfg = dependent(attr, int(std::max(1ll, (n + 63) / 64)), 64, s);
     cudaError_t e;
     if (precision == kFP16)
-        e = cudaLaunchKernelEx(&cfg, wall_values<__half>, static_cast<const __half*>(src), static_cast<__half*>(W),
-                               links, woff, n, plane, pitch);
+        e = cudaLaunchKernelEx(&cfg, wall_values<__half>, static_cast<const __half*>(src), static_cast<__half*>(W), list, n,
+                               plane, pitch);
     else if (precision == kBF16)
         e = cudaLaunchKernelEx(&cfg, wall_values<__nv_bfloat16>, static_cast<const __nv_bfloat16*>(src),
-                               static_cast<__nv_bfloat16*>(W), links, woff, n, plane, pitch);
+                               static_cast<__nv_bfloat16*>(W), list, n, plane, pitch);
     else
-        e = cudaLaunchKernelEx(&cfg, wall_values<float>, static_cast<const float*>(src), static_cast<float*>(W), links,
-                               woff, n, plane, pitch);
+        e = cudaLaunchKernelEx(&cfg, wall_values<float>, static_cast<const float*>(src), static_cast<float*>(W), list, n,
+                               plane, pitch);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
@@ -546,20 +558,6 @@ size_t async_smem_bytes(int block, int precision)
 {
     const size_t per_warp = precision == kFP32 ? sizeof(AsyncStage<float>) : sizeof(AsyncStage<__half>);
     return per_warp * size_t(block / 32);
-}
-
-static cudaLaunchConfig_t dependent(cudaLaunchAttribute (&attr)[1], int grid, int block, cudaStream_t s)
-{
-    // a programmatic dependent of the kernel before it
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.stream = s;
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cfg;
 }
 
 cudaError_t launch_diag_rows(const float2* sets, const float2* last, int n_blocks, int rows, double* out, cudaStream_t s)
