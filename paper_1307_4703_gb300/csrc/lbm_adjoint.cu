@@ -7,13 +7,14 @@
 // the adjoint step is A(t) = F^T M(t) with M(t) = B^T K'^T A(t+1).  The
 // reverse sweep carries M instead of A, so that each reverse step is one
 // launch that reads its neighbours' M(t+1) once:
-//   adjoint_collide  the first reverse step (t = n - 1): A(n) comes from the
-//                    objective; recomputes X = B(F(P(t))) exactly as the step
-//                    kernel does, applies K'(X)^T and B^T, stores M(t);
-//   adjoint_fused    every other step: A(t+1) = F^T M(t+1) per node, a pull
-//                    from x + e_i (bounce-back links return the node's own
-//                    opposite entry) plus the do-nothing outlet term, kept
-//                    in shared memory, then the same work as adjoint_collide.
+//   adjoint_step<true>   the first reverse step (t = n - 1): A(n) comes from
+//                        the objective; recomputes X = B(F(P(t))) exactly as
+//                        the step kernel does, applies K'(X)^T and B^T, stores
+//                        M(t);
+//   adjoint_step<false>  every other step: A(t+1) = F^T M(t+1) per node, a pull
+//                        from x + e_i (bounce-back links return the node's own
+//                        opposite entry) plus the do-nothing outlet term, kept
+//                        in shared memory, then the same work.
 // A(0) itself is not formed: the parameter derivatives are complete once
 // M(0) is.  They accumulate in FP64: d/d(1/tau_g) per block, d/du_in and
 // d/dC_in per port row.
@@ -22,18 +23,21 @@
 namespace lbm {
 namespace {
 
-// A(t+1) of a lane's four nodes in global memory (the first reverse step).
+// A(t+1) of a lane's two nodes in global memory (the first reverse step).
 struct NextGlobal {
     const float* p;  // entry (plane 0, node x0)
     long long P;
     __device__ __forceinline__ float operator()(int i, int k) const { return __ldg(p + i * P + k); }
 };
 
-// Per-warp stage of M(t+1) for a fused reverse step: plane p holds the row
-// that the transposed free flight pulls plane p from (y + e_y of p), columns
-// xs - 4 .. xs + 131 of the tile's segment starting at xs.
-struct MidStage {
-    float pl[kPlanes][kTileNodes + 8];
+// Per-warp stage of M(t+1) for a fused reverse step: pl[p] holds the row that
+// the transposed free flight pulls plane p from (y + e_y of p), columns xs - 4
+// .. xs + 67 of the tile's segment starting at xs; own the tile's own entries
+// of P(t), then of M(t+1), in the planes that bounce-back links return (1 .. 8,
+// then 10 .. 13), where a quad of columns has such a link.
+struct alignas(16) MidStage {
+    float pl[kPlanes][kPairTileNodes + 8];
+    float own[12][kPairTileNodes];
 };
 
 // Row (0 centre, 1 y - 1, 2 y + 1) and column (0 own, 1 x - 1, 2 x + 1) of
@@ -42,8 +46,8 @@ __device__ __forceinline__ constexpr int rev_row(int p) { return src_row(p) == 0
 __device__ __forceinline__ constexpr int rev_col(int p) { return src_col(p) == 0 ? 0 : 3 - src_col(p); }
 __device__ __forceinline__ constexpr int col_shift(int c) { return c == 1 ? -1 : c == 2 ? 1 : 0; }
 
-// A(t+1) of a lane's four nodes from the stage: entry (i, k) sits at column
-// 4 + 4 lane + k + (shift of plane i).  Each entry is the source of exactly
+// A(t+1) of a lane's two nodes from the stage: entry (i, k) sits at column
+// 4 + 2 lane + k + (shift of plane i).  Each entry is the source of exactly
 // one (plane, node), so a lane may overwrite its own entries (bounce-back
 // links, do-nothing terms) without affecting any other lane.
 struct NextStage {
@@ -51,18 +55,17 @@ struct NextStage {
     int lane;
     __device__ __forceinline__ float& operator()(int i, int k) const
     {
-        return st->pl[i][4 + 4 * lane + k + col_shift(rev_col(i))];
+        return st->pl[i][4 + 2 * lane + k + col_shift(rev_col(i))];
     }
 };
 
-// Transpose of the collision and of the port completion for the four nodes
+// Transpose of the collision and of the port completion for the two nodes
 // of one lane.  x holds X (fluid planes as deviations); A(t+1) is read and
-// M(t) formed one node at a time (fewer live registers than whole quads):
+// M(t) formed one node at a time (fewer live registers than whole pairs):
 // node k's entries of M(t) replace its entries of X in x as soon as X of
-// the node has been read, and the quad is stored with 128-bit stores at the
-// end.
+// the node has been read, and the pair is stored at the end.
 template <typename Next>
-__device__ __forceinline__ void collide_adjoint_quad(float4 (&x)[kPlanes], unsigned lk, int x0, int y,
+__device__ __forceinline__ void collide_adjoint_pair(float2 (&x)[kPlanes], unsigned lk, int x0, int y,
                                                      long long oC, const RowBC& bw, const RowBC& be,
                                                      const AdjointArgs& A, const Next& next, KahanF& dwg)
 {
@@ -71,7 +74,7 @@ __device__ __forceinline__ void collide_adjoint_quad(float4 (&x)[kPlanes], unsig
     const bool open_e = be.x >= 0 && ((A.open_mask >> (be.chan_kind & 31)) & 1u);
     const float w = A.omega_f, wgr = A.omega_g;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < 2; ++k) {
         const unsigned lb = (lk >> (8 * k)) & 0xFFu;
         float af[9], ag[5];
         if (lb == kSolid) {
@@ -204,7 +207,7 @@ __device__ __forceinline__ void collide_adjoint_quad(float4 (&x)[kPlanes], unsig
         for (int q = 0; q < 5; ++q) at(x[9 + q], k) = ng[q];
     }
 #pragma unroll
-    for (int i = 0; i < kPlanes; ++i) stg4(A.adj_mid + i * P + oC, x[i]);
+    for (int i = 0; i < kPlanes; ++i) stg2(A.adj_mid + i * P + oC, x[i]);
 }
 
 // Per-block running sum of dJ/d(1/tau_g), one FP64 slot per block: the
@@ -221,31 +224,38 @@ __device__ __forceinline__ void block_add(double* slot, const KahanF& k)
     if (threadIdx.x == 0) {
         DF s = red[0];
         for (int i = 1; i < wpb; ++i) s = df_add(s, red[i]);
-        slot[blockIdx.x] += df_value(s);
+        atomicAdd(slot + blockIdx.x, df_value(s));
     }
 }
 
-// Where a lane's four nodes sit and which neighbouring quads hold fluid
-// (every lane of the warp calls this: it votes).
-struct QuadPos {
+struct PairPos {
     int y, x0, halo_w, halo_e;
     long long oC, oS, oN;
     unsigned lk;
     bool act, ld_w, ld_e;
 };
 
-__device__ __forceinline__ QuadPos quad_pos(const AdjointArgs& A, uint2 tile, int lane)
+// A lane's two wall-link bytes.
+__device__ __forceinline__ unsigned pair_links(const AdjointArgs& A, uint2 tile, int lane)
 {
-    QuadPos q;
-    q.y = int(tile.x >> kColBits);
-    q.x0 = tile_x0(tile) + 4 * lane;
+    const int y = int(tile.x >> kSegBits64), x0 = int(tile.x & ((1u << kSegBits64) - 1)) * kPairTileNodes + 2 * lane;
+    return __ldg(reinterpret_cast<const unsigned short*>(A.links + (long long)y * A.pitch + x0));
+}
+
+// Where a lane's two nodes sit and which neighbouring pairs hold fluid
+// (every lane of the warp calls this: it votes).
+__device__ __forceinline__ PairPos pair_pos(const AdjointArgs& A, uint2 tile, unsigned links, int lane)
+{
+    PairPos q;
+    q.y = int(tile.x >> kSegBits64);
+    q.x0 = int(tile.x & ((1u << kSegBits64) - 1)) * kPairTileNodes + 2 * lane;
     q.oC = (long long)q.y * A.pitch + q.x0;
     q.oS = (long long)(q.y > 0 ? q.y - 1 : q.y) * A.pitch + q.x0;
     q.oN = (long long)(q.y + 1 < A.ny ? q.y + 1 : q.y) * A.pitch + q.x0;
     q.halo_w = q.x0 > 0 ? -1 : 0;
-    q.halo_e = q.x0 + 4 < A.pitch ? 4 : 3;
-    q.lk = __ldg(reinterpret_cast<const unsigned*>(A.links + q.oC));
-    q.act = q.lk != 0xFFFFFFFFu;
+    q.halo_e = q.x0 + 2 < A.pitch ? 2 : 1;
+    q.lk = links;
+    q.act = q.lk != 0xFFFFu;
     const unsigned ball = __ballot_sync(kFull, q.act);
     q.ld_w = ((ball | (ball >> 1)) >> lane) & 1u;
     q.ld_e = ((ball | (ball << 1)) >> lane) & 1u;
@@ -254,15 +264,25 @@ __device__ __forceinline__ QuadPos quad_pos(const AdjointArgs& A, uint2 tile, in
 
 // X = B(F(P(t))) for an active lane: bounce-back, then the forward's port
 // completion, so that x is exactly the pre-collision state of the step.
-__device__ __forceinline__ void complete_quad(float4 (&x)[kPlanes], const QuadPos& q, const RowBC& bw,
-                                              const RowBC& be, const AdjointArgs& A)
+__device__ __forceinline__ void complete_pair(float2 (&x)[kPlanes], const PairPos& q, const RowBC& bw,
+                                              const RowBC& be, const AdjointArgs& A, const MidStage& st, int lane)
 {
     const long long P = A.plane;
-    bounce_back(x, q.lk, A.state, P, q.oC);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const unsigned lb = (q.lk >> (8 * k)) & 0xFFu;
+        if (lb == kSolid) continue;
+#pragma unroll
+        for (int i = 1; i <= 8; ++i) {
+            if (!((lb >> (i - 1)) & 1u)) continue;
+            at(x[i], k) = st.own[opp(i) - 1][2 * lane + k];
+            if (i <= 4) at(x[9 + i], k) = st.own[7 + opp(i)][2 * lane + k];
+        }
+    }
     const bool open_w = bw.x >= 0 && ((A.open_mask >> (bw.chan_kind & 31)) & 1u);
     const bool open_e = be.x >= 0 && ((A.open_mask >> (be.chan_kind & 31)) & 1u);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < 2; ++k) {
         const bool pw = open_w && bw.x == q.x0 + k;
         const bool pe = !pw && open_e && be.x == q.x0 + k;
         if ((pw || pe) && ((q.lk >> (8 * k)) & 0xFFu) != kSolid) {
@@ -271,7 +291,7 @@ __device__ __forceinline__ void complete_quad(float4 (&x)[kPlanes], const QuadPo
             for (int i = 0; i < 9; ++i) f[i] = at(x[i], k);
 #pragma unroll
             for (int i = 0; i < 5; ++i) g[i] = at(x[9 + i], k);
-            complete_port(f, g, pw, pw ? bw : be, A.state, P, q.oC + k);
+            complete_port<false>(f, g, pw, pw ? bw : be, A.state, P, q.oC + k);
 #pragma unroll
             for (int i = 0; i < 9; ++i) at(x[i], k) = f[i];
 #pragma unroll
@@ -280,71 +300,81 @@ __device__ __forceinline__ void complete_quad(float4 (&x)[kPlanes], const QuadPo
     }
 }
 
-// Copies of M(t+1) for the tile into the warp's stage (cp.async, 16 bytes a
-// lane and row, through L2): lane l copies its own 4 values of each row it
-// needs (lanes q0 .. q1 of the tile's fluid range, one more on each side for
-// the shifted planes), lanes 0 and 31 the neighbouring segments' 4 edge
-// values.  Only values that some fluid node of the tile pulls are used.
-__device__ __forceinline__ void issue_mid(const AdjointArgs& A, const QuadPos& q, uint2 tile, MidStage& st, int lane)
+// Copies of M(t+1) for the tile into the warp's stage (cp.async of 16 bytes,
+// through L2): the two halves of the warp take a plane each, its lanes four
+// columns of the row, where the tile's fluid range (pairs q0 .. q1, one more on
+// each side for the shifted planes) needs them; lanes 0 .. 7 the neighbouring
+// segments' edge columns of the eight shifted planes.  Only values that some
+// fluid node of the tile pulls are used.
+__device__ __forceinline__ void issue_mid(const AdjointArgs& A, const PairPos& q, uint2 tile, MidStage& st, int lane)
 {
     const long long P = A.plane;
-    const int xs = q.x0 - 4 * lane;
+    const float* M = A.mid_next;
+    const int xs = q.x0 - 2 * lane;
     const int q0 = int(tile.y & 0xFFu), q1 = int((tile.y >> 8) & 0xFFu);
-    const bool own = lane >= q0 && lane <= q1;
-    const bool wide = lane >= q0 - 1 && lane <= q1 + 1;
+    const int col = 4 * (lane & 15);  // first column of the lane's quad
+    const long long to_col = col - 2 * lane;
+    const bool upper = lane >= 16;
+    if (col / 2 + 1 >= q0 - 1 && col / 2 <= q1 + 1) {
 #pragma unroll
-    for (int p = 0; p < kPlanes; ++p) {
-        const int sr = rev_row(p), sc = rev_col(p);
-        const float* row = A.mid_next + p * P + (sr == 0 ? q.oC : sr == 1 ? q.oS : q.oN) - 4 * lane;
-        if (sc == 0 ? own : wide) cp_async16(&st.pl[p][4 + 4 * lane], row + 4 * lane);
-        if (sc == 1 && lane == 0 && q0 == 0 && xs > 0) cp_async16(&st.pl[p][0], row - 4);
-        if (sc == 2 && lane == 31 && q1 == 31 && xs + kTileNodes < A.pitch)
-            cp_async16(&st.pl[p][4 + kTileNodes], row + kTileNodes);
+        for (int p = 0; p < kPlanes; p += 2) {
+            const int ra = rev_row(p), rb = rev_row(p + 1);
+            const long long a = p * P + (ra == 0 ? q.oC : ra == 1 ? q.oS : q.oN);
+            const long long b = (p + 1) * P + (rb == 0 ? q.oC : rb == 1 ? q.oS : q.oN);
+            cp_async16(&st.pl[upper ? p + 1 : p][4 + col], M + (upper ? b : a) + to_col);
+        }
     }
-    asm volatile("cp.async.commit_group;" ::: "memory");
+    if (lane < 8 && (lane < 4 ? q0 == 0 && xs > 0 : q1 == 31 && xs + kPairTileNodes < A.pitch)) {
+        const int p = (0xA851C763u >> (4 * lane)) & 15;  // 3, 6, 7, 12 from x - 1; 1, 5, 8, 10 from x + 1
+        const long long o = p * P + (p == 5 || p == 6 ? q.oN : p == 7 || p == 8 ? q.oS : q.oC) - 2 * lane;
+        cp_async16(&st.pl[p][lane < 4 ? 0 : 4 + kPairTileNodes], M + o + (lane < 4 ? -4 : kPairTileNodes));
+    }
+}
+
+// Copies of a tile's own entries for its bounce-back links: the planes of P(t)
+// (s = 0) or M(t+1) (s = 1) that a link of the quad returns, by the quad's two
+// lanes in turn.
+__device__ __forceinline__ void issue_own(const float* src, long long P, const PairPos& q, MidStage& st, int s, int lane)
+{
+    const unsigned mine = wall_links2(q.lk);
+    const unsigned wall = mine | __shfl_xor_sync(kFull, mine, 1);  // bit i - 1: direction i comes from a wall
+    if (!wall) return;
+    const int odd = lane & 1, c = 2 * (lane - odd);
+    src += q.oC - 2 * odd;
+#pragma unroll
+    for (int i = 1; i <= 8; ++i) {
+        const int o = opp(i);
+        // returned: of P(t) the entry opposite to the link's direction, of M(t+1)
+        // the entry of the direction itself
+        if (!(wall & (1u << (i - 1)))) continue;
+        const int pl = s == 0 ? o : i;
+        if ((i & 1) == odd) cp_async16(&st.own[pl - 1][c], src + pl * P);
+        else if (i <= 4) cp_async16(&st.own[7 + pl][c], src + (9 + pl) * P);
+    }
 }
 
 // A(t+1) = F^T M(t+1) in the stage, once its copies have landed: a
 // bounce-back link of direction i (the pull source of opp(i) is not fluid)
-// takes the node's own opposite entry of M(t+1) (from global memory, only
-// next to walls); at an open pressure-port node the scalar population with
-// e_x = s gets the do-nothing term of step t+1.  kCoherent: M(t+1) and dn
-// were written by other blocks of the same launch (the multi-step kernel),
-// so they are read through L2.
+// takes the node's own opposite entry of M(t+1); at an open pressure-port node
+// the scalar population with e_x = s gets the do-nothing term of step t+1.
+// kCoherent: dn was written by other blocks of the same launch (the multi-step
+// kernel), so it is read through L2.
 template <bool kCoherent>
-__device__ __forceinline__ float4 ld4_mid(const float* p)
-{
-    if constexpr (kCoherent) return __ldcg(reinterpret_cast<const float4*>(p));
-    else return ldg4(p);
-}
-
-template <bool kCoherent>
-__device__ __forceinline__ void transposed_flight(const NextStage& next, const QuadPos& q, const RowBC& bw,
+__device__ __forceinline__ void transposed_flight(const NextStage& next, const PairPos& q, const RowBC& bw,
                                                   const RowBC& be, const AdjointArgs& A)
 {
-    const long long P = A.plane;
-    const float* __restrict__ M = A.mid_next;
-    unsigned wall = 0;
+    if (wall_links2(q.lk)) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const unsigned lb = (q.lk >> (8 * k)) & 0xFFu;
-        if (lb != kSolid) wall |= lb;
-    }
-    if (wall) {
+        for (int k = 0; k < 2; ++k) {
+            const unsigned lb = (q.lk >> (8 * k)) & 0xFFu;
+            if (lb == kSolid) continue;
+            const int c = 2 * next.lane + k;
 #pragma unroll
-        for (int i = 1; i <= 8; ++i) {
-            const int o = opp(i);
-            if (wall & (1u << (o - 1))) {
-                const float4 own = ld4_mid<kCoherent>(M + o * P + q.oC);
-                const float4 ownc = i <= 4 ? ld4_mid<kCoherent>(M + (9 + o) * P + q.oC) : own;
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const unsigned lb = (q.lk >> (8 * k)) & 0xFFu;
-                    if (lb != kSolid && ((lb >> (o - 1)) & 1u)) {
-                        next(i, k) = at(own, k);
-                        if (i <= 4) next(9 + i, k) = at(ownc, k);
-                    }
-                }
+            for (int i = 1; i <= 8; ++i) {
+                const int o = opp(i);
+                if (!((lb >> (o - 1)) & 1u)) continue;
+                next(i, k) = next.st->own[o - 1][c];
+                if (i <= 4) next(9 + i, k) = next.st->own[7 + o][c];
             }
         }
     }
@@ -353,7 +383,7 @@ __device__ __forceinline__ void transposed_flight(const NextStage& next, const Q
     const bool dn_e = be.x >= 0 && ((m >> (be.chan_kind & 31)) & 1u) && (be.chan_kind >> 8) == 1;
     if (dn_w || dn_e) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < 2; ++k) {
             if (((q.lk >> (8 * k)) & 0xFFu) == kSolid) continue;
             if (dn_w && bw.x == q.x0 + k) next(10, k) += kCoherent ? __ldcg(A.dn + q.y) : A.dn[q.y];
             else if (dn_e && be.x == q.x0 + k) next(12, k) += kCoherent ? __ldcg(A.dn + A.ny + q.y) : A.dn[A.ny + q.y];
@@ -361,69 +391,95 @@ __device__ __forceinline__ void transposed_flight(const NextStage& next, const Q
     }
 }
 
-// The first reverse step: A(t+1) = A(n) is read from global memory.
-__global__ void __launch_bounds__(kAdjointBlock, 4) adjoint_collide(const AdjointArgs A)
+// One tile of a reverse step.  kFirst: A(t+1) = A(n) is read from global
+// memory.  Every later step: A(t+1) = F^T M(t+1) gathered into shared memory;
+// the loads of P(t) into registers and the copies of M(t+1) into the warp's
+// stage are in flight together, then X, A(t+1) in the stage, K'^T and B^T.
+// dn carries the do-nothing terms from one step to the next: the node that
+// reads the entry of step t+1 is the node that then writes the one of step t.
+//
+// Bound by the latency of a tile's chain of loads (a step moves 46 MB from L2
+// and HBM and 24 MB back on the 1024 x 512 chip, 13,000 cycles a tile of which
+// 2,000 are arithmetic), times the tiles a warp takes in turn.  So everything
+// a tile reads is asked for before anything is waited for: P(t) ahead of the
+// previous kernel's end where it is older than that kernel (AdjointArgs::early),
+// the shuffles after the copies of M(t+1), bounce-back entries by cp.async
+// together rather than link by link, the port table for port tiles alone, and
+// the next tile's entry and links a tile ahead.  64-node tiles (two nodes a lane)
+// give each of the 16 warps an SM holds about two tiles there.  A step takes
+// 10.9 us; with 128-node tiles and none of this it took 12.6.  20 warps an SM
+// (96 registers) take 12.3, 24 with spills 13.4: the tiles a warp takes are
+// still two, and they crowd each other.
+template <bool kFirst, bool kCoherent>
+__device__ __forceinline__ void reverse_tile(const AdjointArgs& A, uint2 tile, unsigned links, int lane, MidStage* st,
+                                             KahanF& dwg)
 {
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    const int wpb = blockDim.x >> 5;
     const long long P = A.plane;
-    KahanF dwg;
-    grid_dependency_sync();
-    for (int t = blockIdx.x * wpb + warp; t < A.n_tiles; t += gridDim.x * wpb) {
-        const QuadPos q = quad_pos(A, tile_at(A.tiles, A.n_tiles, t, A.reverse), lane);
-        float4 x[kPlanes];
-        pull_quad<false>(x, A.state, P, q.oC, q.oS, q.oN, q.halo_w, q.halo_e, q.act, q.ld_w, q.ld_e, lane);
-        if (!q.act) continue;
-        const RowBC bw = A.rowbc[q.y];
-        const RowBC be = A.rowbc[A.ny + q.y];
-        complete_quad(x, q, bw, be, A);
-        collide_adjoint_quad(x, q.lk, q.x0, q.y, q.oC, bw, be, A, NextGlobal{A.adj_next + q.oC, P}, dwg);
+    const PairPos q = pair_pos(A, tile, links, lane);
+    issue_own(A.state, P, q, *st, 0, lane);
+    float2 x[kPlanes];
+    PairHalo halo{};
+    load_pair(x, halo, A.state, P, q.oC, q.oS, q.oN, q.halo_w, q.halo_e, q.act, q.ld_w, q.ld_e, lane);
+    if constexpr (!kCoherent) grid_dependency_sync();
+    if constexpr (!kFirst) issue_mid(A, q, tile, *st, lane);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    // no port on either side of the tile: nothing to look up
+    RowBC bw, be;
+    bw.x = be.x = -1;
+    if (tile.y & kPortTile) {
+        bw = A.rowbc[q.y];
+        be = A.rowbc[A.ny + q.y];
     }
-    block_add(A.grad_w, dwg);
-}
-
-// Every later reverse step: A(t+1) = F^T M(t+1) gathered into shared memory
-// (each thread reads back only its own entries, so no barrier), then X,
-// K'^T and B^T as in adjoint_collide.  dn carries the do-nothing terms from
-// one step to the next: the node that reads the entry of step t+1 is the
-// node that then writes the one of step t.
-// One tile of a fused reverse step (the body of adjoint_fused and of the
-// multi-step kernel): the copies of M(t+1) into the warp's stage and the
-// loads of P(t) into registers are in flight together; then X, A(t+1) in
-// the stage, K'^T and B^T.
-template <bool kCoherent>
-__device__ __forceinline__ void fused_tile(const AdjointArgs& A, uint2 tile, int lane, MidStage& st, KahanF& dwg)
-{
-    const long long P = A.plane;
-    const QuadPos q = quad_pos(A, tile, lane);
-    issue_mid(A, q, tile, st, lane);
-    float4 x[kPlanes];
-    pull_quad<false>(x, A.state, P, q.oC, q.oS, q.oN, q.halo_w, q.halo_e, q.act, q.ld_w, q.ld_e, lane);
-    const RowBC bw = A.rowbc[q.y];
-    const RowBC be = A.rowbc[A.ny + q.y];
-    if (q.act) complete_quad(x, q, bw, be, A);
+    shift_pair(x, halo, lane);
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncwarp();
-    const NextStage next{&st, lane};
+    if (q.act) complete_pair(x, q, bw, be, A, *st, lane);
+    if constexpr (!kFirst) {
+        if (__any_sync(kFull, wall_links2(q.lk) != 0)) {
+            __syncwarp();  // every lane has read its entries of P(t)
+            issue_own(A.mid_next, P, q, *st, 1, lane);
+            asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+            __syncwarp();
+        }
+    }
     if (q.act) {
-        transposed_flight<kCoherent>(next, q, bw, be, A);
-        collide_adjoint_quad(x, q.lk, q.x0, q.y, q.oC, bw, be, A, next, dwg);
+        if constexpr (kFirst) {
+            collide_adjoint_pair(x, q.lk, q.x0, q.y, q.oC, bw, be, A, NextGlobal{A.adj_next + q.oC, P}, dwg);
+        } else {
+            const NextStage next{st, lane};
+            transposed_flight<kCoherent>(next, q, bw, be, A);
+            collide_adjoint_pair(x, q.lk, q.x0, q.y, q.oC, bw, be, A, next, dwg);
+        }
     }
     __syncwarp();  // the stage is read before the next tile's copies overwrite it
 }
 
-__global__ void __launch_bounds__(kAdjointBlock, 4) adjoint_fused(const AdjointArgs A)
+template <bool kFirst>
+__global__ void __launch_bounds__(kAdjointBlock, kAdjointBlocks) adjoint_step(const AdjointArgs A)
 {
     extern __shared__ __align__(16) unsigned char next_smem[];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int wpb = blockDim.x >> 5;
-    MidStage& st = reinterpret_cast<MidStage*>(next_smem)[warp];
+    MidStage* st = reinterpret_cast<MidStage*>(next_smem) + warp;
     KahanF dwg;
-    grid_dependency_sync();
-    for (int t = blockIdx.x * wpb + warp; t < A.n_tiles; t += gridDim.x * wpb)
-        fused_tile<false>(A, tile_at(A.tiles, A.n_tiles, t, A.reverse), lane, st, dwg);
+    const int stride = gridDim.x * wpb;
+    int t = blockIdx.x * wpb + warp;
+    uint2 tile = make_uint2(0u, 0u);
+    unsigned links = 0;
+    if (t < A.n_tiles) {
+        tile = tile_at(A.tiles, A.n_tiles, t, A.reverse);
+        links = pair_links(A, tile, lane);
+    }
+    if (kFirst || !A.early) grid_dependency_sync();
+    for (; t < A.n_tiles; t += stride) {
+        reverse_tile<kFirst, false>(A, tile, links, lane, st, dwg);
+        if (t + stride < A.n_tiles) {
+            tile = tile_at(A.tiles, A.n_tiles, t + stride, A.reverse);
+            links = pair_links(A, tile, lane);
+        }
+    }
+    grid_dependency_sync();  // (a block may have had no tile)
     block_add(A.grad_w, dwg);
 }
 
@@ -433,7 +489,7 @@ __global__ void __launch_bounds__(kAdjointBlock, 4) adjoint_fused(const AdjointA
 // masks[j - j_lo + 1]; M alternates between mid_a (M(j_hi + 1) on entry)
 // and mid_b.  The step's own reads of M and dn go through L2.  A barrier
 // that times out stops the kernel with bit 1 of the error word set.
-__global__ void __launch_bounds__(kAdjointBlock, 4)
+__global__ void __launch_bounds__(kAdjointBlock, kAdjointBlocks)
     adjoint_steps_coop(const AdjointArgs A0, int j_hi, int j_lo, const float* state_lo, long long stride,
                        const uint32_t* masks, float* mid_a, float* mid_b, unsigned* count)
 {
@@ -441,7 +497,7 @@ __global__ void __launch_bounds__(kAdjointBlock, 4)
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int wpb = blockDim.x >> 5;
-    MidStage& st = reinterpret_cast<MidStage*>(next_smem)[warp];
+    MidStage* st = reinterpret_cast<MidStage*>(next_smem) + warp;
     KahanF dwg;
     for (int j = j_hi, s = 0; j >= j_lo; --j, ++s) {
         AdjointArgs A = A0;
@@ -451,8 +507,10 @@ __global__ void __launch_bounds__(kAdjointBlock, 4)
         A.mid_next = (s & 1) ? mid_b : mid_a;
         A.adj_mid = (s & 1) ? mid_a : mid_b;
         A.reverse = A0.reverse ^ (s & 1);
-        for (int t = blockIdx.x * wpb + warp; t < A.n_tiles; t += gridDim.x * wpb)
-            fused_tile<true>(A, tile_at(A.tiles, A.n_tiles, t, A.reverse), lane, st, dwg);
+        for (int t = blockIdx.x * wpb + warp; t < A.n_tiles; t += gridDim.x * wpb) {
+            const uint2 tile = tile_at(A.tiles, A.n_tiles, t, A.reverse);
+            reverse_tile<false, true>(A, tile, pair_links(A, tile, lane), lane, st, dwg);
+        }
         if (j > j_lo && !grid_barrier(count, unsigned(s + 1) * gridDim.x + A0.barrier_extra, A0.err)) break;
     }
     block_add(A0.grad_w, dwg);
@@ -504,23 +562,26 @@ __global__ void sum_doubles(const double* v, int n, double* out)
 
 }  // namespace
 
+constexpr size_t kMidSmem = sizeof(MidStage) * (kAdjointBlock / 32);
+
 cudaError_t adjoint_occupancy(int* blocks_per_sm)
 {
-    const size_t smem = adjoint_fused_smem(kAdjointBlock);
-    cudaError_t e = cudaFuncSetAttribute(adjoint_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    cudaError_t e = cudaFuncSetAttribute(adjoint_step<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kMidSmem));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(adjoint_step<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kMidSmem));
     int a = 0, b = 0;
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, adjoint_collide, kAdjointBlock, 0);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, adjoint_fused, kAdjointBlock, smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, adjoint_step<true>, kAdjointBlock, kMidSmem);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, adjoint_step<false>, kAdjointBlock, kMidSmem);
     *blocks_per_sm = a < b ? a : b;
     return e;
 }
 
 cudaError_t adjoint_coop_occupancy(int* blocks_per_sm)
 {
-    const size_t smem = adjoint_fused_smem(kAdjointBlock);
-    cudaError_t e = cudaFuncSetAttribute(adjoint_steps_coop, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    cudaError_t e = cudaFuncSetAttribute(adjoint_steps_coop, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kMidSmem));
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, adjoint_steps_coop,
-                                                                           kAdjointBlock, smem);
+                                                                           kAdjointBlock, kMidSmem);
     return e;
 }
 
@@ -533,7 +594,7 @@ cudaError_t launch_adjoint_steps_coop(const AdjointArgs& a, int j_hi, int j_lo, 
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(kAdjointBlock);
-    cfg.dynamicSmemBytes = adjoint_fused_smem(kAdjointBlock);
+    cfg.dynamicSmemBytes = kMidSmem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;  // all blocks resident, or the launch fails
@@ -552,14 +613,15 @@ cudaError_t launch_adjoint_step(const AdjointArgs& a, bool first, int grid, cuda
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(kAdjointBlock);
-    cfg.dynamicSmemBytes = first ? 0 : adjoint_fused_smem(kAdjointBlock);
+    cfg.dynamicSmemBytes = kMidSmem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaError_t e = first ? cudaLaunchKernelEx(&cfg, adjoint_collide, a) : cudaLaunchKernelEx(&cfg, adjoint_fused, a);
+    cudaError_t e = first ? cudaLaunchKernelEx(&cfg, adjoint_step<true>, a)
+                          : cudaLaunchKernelEx(&cfg, adjoint_step<false>, a);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }

@@ -1801,7 +1801,7 @@ lbm_status lbm_adjoint(lbm_handle h, const lbm_objective* obj, int64_t n, int32_
     LBM_CUDA(h, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
     const int ablock = lbm::kAdjointBlock;
     LBM_CUDA(h, lbm::adjoint_occupancy(&per_sm));
-    const int agrid = std::max(1, std::min((h->n_tiles + ablock / 32 - 1) / (ablock / 32), std::max(1, per_sm) * sms));
+    const int agrid = std::max(1, std::min((h->n_tiles64 + ablock / 32 - 1) / (ablock / 32), std::max(1, per_sm) * sms));
 
     Scratch tmp(h);
     char* ckpt = static_cast<char*>(tmp.get(size_t(n_ck) * S));
@@ -1961,7 +1961,8 @@ lbm_status lbm_adjoint(lbm_handle h, const lbm_objective* obj, int64_t n, int32_
     LBM_CUDA(h, cudaMemcpyAsync(oy, hy.data(), hy.size() * sizeof(int), cudaMemcpyHostToDevice, st));
     LBM_CUDA(h, cudaMemcpyAsync(ot, obj->target, size_t(obj->n) * sizeof(float), cudaMemcpyHostToDevice, st));
     LBM_CUDA(h, cudaMemcpyAsync(ow, obj->weight, size_t(obj->n) * sizeof(float), cudaMemcpyHostToDevice, st));
-    for (float* b : adj) LBM_CUDA(h, cudaMemsetAsync(b, 0, S, st));
+    // (of M(t) only what its writer stored is used: adj[1] and adj[2] need no zeros)
+    LBM_CUDA(h, cudaMemsetAsync(adj[0], 0, S, st));
     LBM_CUDA(h, cudaMemsetAsync(gw, 0, size_t(agrid) * sizeof(double), st));
     LBM_CUDA(h, cudaMemsetAsync(gu, 0, size_t(2) * h->ny * sizeof(double), st));
     LBM_CUDA(h, cudaMemsetAsync(gc, 0, size_t(2) * h->ny * sizeof(double), st));
@@ -1984,8 +1985,8 @@ lbm_status lbm_adjoint(lbm_handle h, const lbm_objective* obj, int64_t n, int32_
     lbm::AdjointArgs A{};
     A.links = h->links;
     A.rowbc = h->rowbc;
-    A.tiles = h->tiles;
-    A.n_tiles = h->n_tiles;
+    A.tiles = h->tiles64;
+    A.n_tiles = h->n_tiles64;
     A.ny = h->ny;
     A.pitch = h->pitch;
     A.plane = h->plane;
@@ -2005,7 +2006,9 @@ lbm_status lbm_adjoint(lbm_handle h, const lbm_objective* obj, int64_t n, int32_
     // adj[0] holds A(n); M(t) alternates between adj[1] and adj[2]
     int mid = 0;  // 0 before the first reverse step, else adj[mid] holds M(t+1)
     // One reverse step t (state `state`): the first one reads A(n), the
-    // others gather M(t + 1).
+    // others gather M(t + 1).  The kernel before one that follows another
+    // reverse step wrote no state, and waited for the one that did.
+    bool after_reverse = false;
     auto reverse_one = [&](int64_t t, const float* state) -> lbm_status {
         A.state = state;
         A.adj_next = adj[0];
@@ -2014,6 +2017,8 @@ lbm_status lbm_adjoint(lbm_handle h, const lbm_objective* obj, int64_t n, int32_
         A.open_mask = h->mask_at(t0 + t);
         A.open_mask_next = h->mask_at(t0 + t + 1);
         A.reverse = int((n - 1 - t) & 1);
+        A.early = after_reverse;
+        after_reverse = true;
         cudaError_t e = lbm::launch_adjoint_step(A, mid == 0, agrid, st);
         if (e != cudaSuccess) return cuda_fail(h, e, "adjoint step launch");
         mid = mid == 1 ? 2 : 1;
@@ -2052,6 +2057,7 @@ lbm_status lbm_adjoint(lbm_handle h, const lbm_objective* obj, int64_t n, int32_
         // recompute the segment's states 1 .. len - 1 from its checkpoint
         // (the last segment's are still there from the forward sweep)
         if (len >= 2 && sg != n_ck - 1) {
+            after_reverse = false;
             r.src = state(0);
             r.dst = state(1);
             r.reverse = 1;

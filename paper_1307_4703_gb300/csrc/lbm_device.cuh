@@ -607,13 +607,15 @@ __device__ __forceinline__ float equilibrium_wall(int i, int ahead, const T* S, 
     return w * (rd + rho * (3.f * eu + 4.5f * eu * eu - 1.5f * (ux * ux + uy * uy)));
 }
 
-template <typename T>
+// kRescale = false: the caller has ports of kinds 0 and 1 only (the call out of
+// line costs registers wherever it is possible).
+template <bool kRescale = true, typename T>
 __device__ __forceinline__ bool complete_port(float (&f)[9], float (&g)[5], bool west, const RowBC& b,
                                               const T* S, long long P, long long own, float gref1 = 0.f,
                                               float wg1 = 0.f, float inv_cs2g = 0.f)
 {
     const int kind = (b.chan_kind >> 8) & 0xFF;
-    if (kind >= 2) {
+    if (kRescale && kind >= 2) {
         PortNode n;
 #pragma unroll
         for (int i = 0; i < 9; ++i) n.f[i] = f[i];
@@ -699,6 +701,63 @@ __device__ __forceinline__ void pull_quad(float4 (&v)[kN], const T* __restrict__
         }
         v[j] = r;
     }
+}
+
+// Free flight (pull) of one lane's two nodes x0, x0 + 1 in two parts, so that a
+// warp can ask for more between them.  load_pair: 64-bit loads of each plane's
+// source row; for the +-1 column shifts, lanes 0 and 31 load the values that
+// come from the neighbouring segments.  shift_pair: the shifts, between lanes by
+// shuffle, which waits for the loads.  act / ld_w / ld_e as in pull_quad.
+struct PairHalo {
+    float h[4];
+};
+__device__ __forceinline__ void load_pair(float2 (&v)[kPlanes], PairHalo& halo, const float* __restrict__ S, long long P,
+                                          long long oC, long long oS, long long oN, int halo_w, int halo_e,
+                                          bool act, bool ld_w, bool ld_e, int lane)
+{
+#pragma unroll
+    for (int p = 0; p < kPlanes; ++p) {
+        const int sr = src_row(p), sc = src_col(p);
+        const bool ld = sc == 0 ? act : sc == 1 ? ld_w : ld_e;
+        v[p] = ld ? ldg2(S + p * P + (sr == 0 ? oC : sr == 1 ? oS : oN)) : make_float2(0.f, 0.f);
+    }
+    // one load an entry: the j-th planes of the two directions pull from the same row
+    const bool west = lane == 0;
+    const bool edge = act && (west || lane == 31);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        constexpr int pw[4] = {1, 5, 8, 10}, pe[4] = {3, 6, 7, 12};
+        static_assert(src_col(pw[0]) == 1 && src_col(pw[1]) == 1 && src_col(pw[2]) == 1 && src_col(pw[3]) == 1);
+        static_assert(src_col(pe[0]) == 2 && src_col(pe[1]) == 2 && src_col(pe[2]) == 2 && src_col(pe[3]) == 2);
+        const int sr = src_row(pw[j]);
+        if (edge)
+            halo.h[j] = __ldg(S + (west ? pw[j] : pe[j]) * P + (sr == 0 ? oC : sr == 1 ? oS : oN) +
+                              (west ? halo_w : halo_e));
+    }
+}
+__device__ __forceinline__ void shift_pair(float2 (&v)[kPlanes], const PairHalo& halo, int lane)
+{
+    int w = 0, e = 0;
+#pragma unroll
+    for (int p = 0; p < kPlanes; ++p) {
+        const int sc = src_col(p);
+        if (sc == 1) {  // from column x - 1
+            const int j = w++;
+            const float a = __shfl_up_sync(kFull, v[p].y, 1);
+            v[p] = make_float2(lane == 0 ? halo.h[j] : a, v[p].x);
+        } else if (sc == 2) {  // from column x + 1
+            const int j = e++;
+            const float a = __shfl_down_sync(kFull, v[p].x, 1);
+            v[p] = make_float2(v[p].y, lane == 31 ? halo.h[j] : a);
+        }
+    }
+}
+// Union of the wall-link bytes of two nodes (the low 16 bits of lk2), solid
+// ones aside.
+__device__ __forceinline__ unsigned wall_links2(unsigned lk2)
+{
+    const unsigned a = lk2 & 0xFFu, b = lk2 >> 8;
+    return (a != kSolid ? a : 0u) | (b != kSolid ? b : 0u);
 }
 
 // Which lanes of a warp tile load plane values, from the tile's table entry

@@ -149,7 +149,7 @@ struct AdjointArgs {
     float* adj_mid;         // M(t), written
     const uint8_t* links;
     const RowBC* rowbc;
-    const uint2* tiles;
+    const uint2* tiles;       // 64-node tiles
     int n_tiles;
     int ny;
     int pitch;
@@ -158,6 +158,7 @@ struct AdjointArgs {
     uint32_t open_mask;       // valve word of step t
     uint32_t open_mask_next;  // valve word of step t+1
     int reverse;              // take the tile table from its end (alternates from launch to launch)
+    int early;                // the previous kernel did not write the state: read it before that kernel ends
     float* dn;              // 2*ny: do-nothing terms passed from step t+1 to step t
     double* grad_w;         // one running sum of dJ/d(1/tau_g) per block
     double* grad_u;         // 2*ny running sums of dJ/du_in
@@ -166,13 +167,8 @@ struct AdjointArgs {
     unsigned barrier_extra; // test hook (see StepArgs)
 };
 
-// Threads per block of the reverse-step kernels; the fused one stages
-// M(t+1) of each warp's tile in shared memory (14 rows of 136 floats a warp).
-constexpr int kAdjointBlock = 128;
-inline size_t adjoint_fused_smem(int block)
-{
-    return size_t(kPlanes) * (kTileNodes + 8) * sizeof(float) * size_t(block / 32);
-}
+// Threads per block of the reverse-step kernels, and the blocks an SM holds.
+constexpr int kAdjointBlock = 128, kAdjointBlocks = 4;
 
 cudaError_t adjoint_occupancy(int* blocks_per_sm);
 // first: the first reverse step (A(n) from adj_next); else the fused step
