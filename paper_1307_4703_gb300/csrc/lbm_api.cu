@@ -154,7 +154,7 @@ struct lbm_ctx {
     void* wallv = nullptr;     // the paper's walls: 8 planes of wall values for the step
     lbm::WallLink* wall_list = nullptr;  // the links it holds values of
     long long n_wall = 0;
-    bool paper_ports = false;  // some port has a rescaling kind (no adjoint)
+    bool paper_ports = false;  // some port has a rescaling kind (no adjoint; step kernels that complete them)
     std::vector<Graph> graphs;
 
     // Whether the valve words stay the same over steps [t0, t0 + len).
@@ -402,7 +402,7 @@ cudaError_t launch_pair(const lbm_ctx* h, const lbm::StepArgs& a, const uint32_t
     lbm::PairArgs p{a, a, h->pair_items, h->pair_first};
     std::memcpy(p.second.open_mask, words, sizeof(words));
     p.second.plane = lbm::kTileNodes;
-    return lbm::launch_step_pair(p, src_map, h->pair_grid, h->precision, s);
+    return lbm::launch_step_pair(p, src_map, h->pair_grid, h->precision, h->paper_ports, s);
 }
 
 // Whether the next two of `left` steps go as one launch.  The last step of a
@@ -959,6 +959,7 @@ lbm_status create_impl(lbm_handle* out, int32_t nx, int32_t ny, const uint8_t* m
     L.precision = opt.precision;
     L.pdl = true;  // consecutive steps overlap launch and set-up with the previous step's tail
     L.walls = opt.wall_scheme == LBM_WALL_EQUILIBRIUM;
+    L.rescale = h->paper_ports;
     if (L.variant == lbm::kVariantBulk) {
         const int nc = opt.consumer_warps ? opt.consumer_warps : kDefaultConsumers;
         L.stages = nc * (opt.pipeline_stages                ? opt.pipeline_stages
@@ -1019,12 +1020,12 @@ lbm_status create_impl(lbm_handle* out, int32_t nx, int32_t ny, const uint8_t* m
     if (opt.variant == 0 && opt.block_threads == 0 && opt.max_blocks == 0 && opt.multi_step == 0 &&
         opt.wall_scheme == LBM_WALL_BOUNCE_BACK && h->pop[0] && h->pop[1]) {
         int pair_per_sm = 0;
-        bool have = lbm::pair_occupancy(h->precision, &pair_per_sm) == cudaSuccess && pair_per_sm > 0;
+        bool have = lbm::pair_occupancy(h->precision, h->paper_ports, &pair_per_sm) == cudaSuccess && pair_per_sm > 0;
         for (int b = 0; b < 2 && have; ++b)
             have = lbm::pair_tensor_map(&h->pair_map[b], h->pop[b], ny, pitch, h->precision) == cudaSuccess;
         if (have) {
             plan = lbm::plan_pairs(h->tiles_rows, rowbc, nx, ny, pitch, h->precision, lbm::pair_warps(h->precision),
-                                   pair_per_sm * sms);
+                                   pair_per_sm * sms, (long long)h->launch.grid * (h->launch.block / 32));
             h->pair_items = static_cast<int4*>(dev_alloc(h, plan.items.size() * sizeof(int4)));
             h->pair_first = static_cast<int*>(dev_alloc(h, plan.block_first.size() * sizeof(int)));
             have = h->pair_items && h->pair_first;
@@ -2341,6 +2342,7 @@ lbm_status lbm_autotune(lbm_handle h, int32_t trial_steps)
         L.precision = h->precision;
         L.pdl = true;
         L.walls = h->wallv != nullptr;
+        L.rescale = h->paper_ports;
         if (L.walls && (c.variant == 3 || c.variant == 4)) continue;
         if (c.variant == 1 || c.variant == 4 || c.variant == 5) {
             L.variant = c.variant == 1 ? lbm::kVariantRegs : c.variant == 4 ? lbm::kVariantAsync : lbm::kVariantPairs;

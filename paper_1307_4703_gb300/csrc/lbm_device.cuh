@@ -489,6 +489,57 @@ __device__ __forceinline__ void bounce_back(float4 (&v)[kPlanes], unsigned lk, c
     }
 }
 
+// Halfway bounce-back in two parts (FP32 storage): bounce_issue copies the own
+// entries that the lane's links return to its part of the warp's stage
+// (cp.async, 16 bytes an entry, no registers), so that they are in flight
+// together and with the loads of the free flight; bounce_staged puts them in
+// place after the copies were waited for.
+struct alignas(16) BounceStage {
+    float own[12][kTileNodes];  // planes opp(1) .. opp(8), then 9 + opp(1) .. 9 + opp(4)
+};
+__device__ __forceinline__ unsigned wall_links(unsigned lk)
+{
+    unsigned wall = 0;  // union of the wall links of the fluid nodes
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const unsigned lb = (lk >> (8 * k)) & 0xFFu;
+        if (lb != kSolid) wall |= lb;
+    }
+    return wall;
+}
+__device__ __forceinline__ void bounce_issue(BounceStage& st, unsigned wall, const float* S, long long P, long long oC,
+                                             int lane)
+{
+    if (wall) {
+#pragma unroll
+        for (int i = 1; i <= 8; ++i) {
+            if (!(wall & (1u << (i - 1)))) continue;
+            cp_async16(&st.own[i - 1][4 * lane], S + opp(i) * P + oC);
+            if (i <= 4) cp_async16(&st.own[7 + i][4 * lane], S + (9 + opp(i)) * P + oC);
+        }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+__device__ __forceinline__ void bounce_staged(float4 (&v)[kPlanes], unsigned lk, unsigned wall, const BounceStage& st,
+                                              int lane)
+{
+    asm volatile("cp.async.wait_group 0;" ::: "memory");  // the lane's own copies
+    if (!wall) return;
+#pragma unroll
+    for (int i = 1; i <= 8; ++i) {
+        if (!(wall & (1u << (i - 1)))) continue;
+        const float4 own = *reinterpret_cast<const float4*>(&st.own[i - 1][4 * lane]);
+        const float4 ownc = i <= 4 ? *reinterpret_cast<const float4*>(&st.own[i <= 4 ? 7 + i : 0][4 * lane]) : own;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if ((lk >> (8 * k + i - 1)) & 1u) {
+                at(v[i], k) = at(own, k);
+                if (i <= 4) at(v[9 + i], k) = at(ownc, k);
+            }
+        }
+    }
+}
+
 // Completion of an open port node (fluid populations as deviations
 // f_i - w_i).  west: the port receives from -x, so the populations with
 // e_x = +1 are unknown (s = +1); otherwise e_x = -1 (s = -1).  The port kind
@@ -831,7 +882,7 @@ __device__ __forceinline__ float2 row_rates(const StepArgs& a, int y)
 // Port completion of node k of the quad (the port rules work on g_i itself,
 // so 16-bit deviations are shifted to g_i around them).  Returns true for an
 // outlet node.
-template <typename T>
+template <bool kRescale = true, typename T>
 __device__ __forceinline__ bool port_node(float (&f)[9], float (&g)[5], bool west, const RowBC& b,
                                           const StepArgs& a, const T* S, long long own)
 {
@@ -841,7 +892,7 @@ __device__ __forceinline__ bool port_node(float (&f)[9], float (&g)[5], bool wes
 #pragma unroll
         for (int i = 1; i < 5; ++i) g[i] += a.gref1;
     }
-    const bool outlet = complete_port(f, g, west, b, S, a.plane, own, a.gref1, a.wg1, a.inv_cs2g);
+    const bool outlet = complete_port<kRescale>(f, g, west, b, S, a.plane, own, a.gref1, a.wg1, a.inv_cs2g);
     if constexpr (kDev) {
         g[0] -= a.gref0;
 #pragma unroll
@@ -990,7 +1041,7 @@ __device__ __forceinline__ NodeMoments collide_node(float (&f)[9], float (&g)[5]
 // the step even where it never runs (a timing copy without it: FP16 44.1 us
 // against 48.0 us on the 4096 x 2048 chip).  The register kernels take the
 // port-free form for those tiles and the pass form for the few others.
-template <typename T, bool kPasses = !kStoresF32<T>, bool kPorts = true>
+template <typename T, bool kPasses = !kStoresF32<T>, bool kPorts = true, bool kRescale = true>
 __device__ __forceinline__ void collide_quad(float4 (&v)[kPlanes], unsigned lk, int x0, const RowBC& bw,
                                              const RowBC& be, const StepArgs& a, const T* S, long long oC,
                                              float2 omega, QuadAcc& acc)
@@ -1026,7 +1077,7 @@ __device__ __forceinline__ void collide_quad(float4 (&v)[kPlanes], unsigned lk, 
                 for (int i = 0; i < 9; ++i) f[i] = at(v[i], k);
 #pragma unroll
                 for (int i = 0; i < 5; ++i) g[i] = at(v[9 + i], k);
-                if (port_node(f, g, pw, pw ? bw : be, a, S, oC + k)) outlet |= 1u << k;
+                if (port_node<kRescale>(f, g, pw, pw ? bw : be, a, S, oC + k)) outlet |= 1u << k;
 #pragma unroll
                 for (int i = 0; i < 9; ++i) at(v[i], k) = f[i];
 #pragma unroll
@@ -1058,7 +1109,7 @@ __device__ __forceinline__ void collide_quad(float4 (&v)[kPlanes], unsigned lk, 
                 const int xk = x0 + k;
                 const bool pw = open_w && bw.x == xk;
                 const bool pe = !pw && open_e && be.x == xk;
-                if (pw || pe) outlet_k = port_node(f, g, pw, pw ? bw : be, a, S, oC + k);
+                if (pw || pe) outlet_k = port_node<kRescale>(f, g, pw, pw ? bw : be, a, S, oC + k);
             }
         }
 

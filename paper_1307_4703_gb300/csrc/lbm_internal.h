@@ -67,6 +67,7 @@ struct StepLaunch {
     int precision = kFP32;  // storage of the populations
     bool pdl = false;       // launch as a programmatic dependent of the previous kernel
     bool walls = false;     // the paper's walls (variants 1 and 2; see StepArgs::wallv)
+    bool rescale = false;   // ports of the rescaling kinds
 };
 
 struct RowBC {
@@ -133,13 +134,15 @@ struct PairArgs {
     const int4* items;
     const int* block_first;
 };
-cudaError_t pair_occupancy(int precision, int* per_sm);
+// rescale: the lattice has ports of the rescaling kinds
+cudaError_t pair_occupancy(int precision, bool rescale, int* per_sm);
 int pair_warps(int precision);  // of a block
 // A tensor map of `planes` planes of ny rows of `pitch` elements of `elem`
 // bytes at base, with boxes of cols x rows of one plane.
 cudaError_t rows_tensor_map(CUtensorMap* map, void* base, int planes, int ny, int pitch, int elem, int cols, int rows);
 cudaError_t pair_tensor_map(CUtensorMap* map, void* pop, int ny, int pitch, int precision);
-cudaError_t launch_step_pair(const PairArgs& p, const CUtensorMap& map, int grid, int precision, cudaStream_t s);
+cudaError_t launch_step_pair(const PairArgs& p, const CUtensorMap& map, int grid, int precision, bool rescale,
+                             cudaStream_t s);
 
 // One adjoint step (lbm_adjoint.cu): A(t) from A(t+1) and the state P(t).
 struct AdjointArgs {

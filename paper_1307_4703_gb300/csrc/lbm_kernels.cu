@@ -435,6 +435,11 @@ int bulk_stage_bytes(int precision)
     return int(precision == kFP32 ? sizeof(Stage) : sizeof(StageT<__half>));
 }
 
+constexpr int kRegsMaxThreads = 256;  // of coupled_step_regs
+
+// Dynamic shared memory of the register kernel that stages its bounce-back entries.
+static size_t staged_smem_bytes(int block) { return sizeof(BounceStage) * size_t(block / 32); }
+
 cudaError_t prepare_step_kernels()
 {
     // The attribute belongs to the kernel, not to a handle: allow the largest
@@ -523,8 +528,11 @@ cudaError_t launch_step(const StepArgs& a, const StepLaunch& l, cudaStream_t s)
         e = cudaLaunchKernelEx(&cfg, coupled_step_regs<__half, false>, b);
     } else if (l.precision == kBF16) {
         e = cudaLaunchKernelEx(&cfg, coupled_step_regs<__nv_bfloat16, false>, b);
-    } else {
+    } else if (l.rescale) {
         e = cudaLaunchKernelEx(&cfg, coupled_step_regs<float, false>, b);
+    } else {
+        cfg.dynamicSmemBytes = staged_smem_bytes(l.block);
+        e = cudaLaunchKernelEx(&cfg, coupled_step_regs<float, false, false, true>, b);
     }
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
@@ -612,7 +620,15 @@ cudaError_t step_kernel_occupancy(const StepLaunch& l, int* blocks_per_sm)
     if (l.precision == kBF16)
         return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, coupled_step_regs<__nv_bfloat16, false>,
                                                              l.block, 0);
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, coupled_step_regs<float, false>, l.block, 0);
+    if (l.rescale)
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, coupled_step_regs<float, false>, l.block, 0);
+    // (blocks of 256 threads want more than the 48 KB a kernel may use unasked)
+    const cudaError_t e =
+        cudaFuncSetAttribute(coupled_step_regs<float, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             int(staged_smem_bytes(kRegsMaxThreads)));
+    if (e != cudaSuccess) return e;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, coupled_step_regs<float, false, false, true>,
+                                                         l.block, staged_smem_bytes(l.block));
 }
 
 cudaError_t launch_init_rest(void* pop, int ny, int pitch, float rho0, float wg0, float wg1,

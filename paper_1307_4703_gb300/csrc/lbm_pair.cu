@@ -26,8 +26,8 @@
 //   - a strip along a side wall names the two lanes at it, and these bounce
 //     back from the staged rows (from global memory, such strips took 1.5
 //     times as long as the others and set the launch's length).
-// Steps of the 4096 x 2048 chip, us: FP32 61.5 one by one, 39.3 here; FP16
-// 37.4 -> 29.9; 64 chips in a batch 111 -> 84 (FP32).  Tried: the second
+// Steps of the 4096 x 2048 chip, us: FP32 59.5 one by one, 39.0 here; FP16
+// 37.4 -> 29.2; 64 chips in a batch 111 -> 79.6 (FP32).  Tried: the second
 // step's rows written by bulk copies from shared memory (50.4 against 46.7
 // us at that stage: 14 copies a row by one warp are slow to issue); rows
 // copied lane by lane (cp.async: FP32 the same, FP16 34.7 against 30.5 us);
@@ -146,8 +146,11 @@ __device__ __forceinline__ void pull_staged(float4 (&v)[kPlanes], const PairSmem
     }
 }
 
-// Completion of the open port node k of a lane's quad.
-template <int k, typename T>
+// Completion of the open port node k of a lane's quad.  kRescale: the lattice
+// has ports of the rescaling kinds, whose completion is a call (complete_port);
+// kernels without it are 2 to 6 % faster (4096 x 2048 in FP32 39.4 -> 39.0 us a
+// step, FP16 30.1 -> 29.3; 256 x 128 2.70 -> 2.60, FP16 2.97 -> 2.79).
+template <bool kRescale, int k, typename T>
 __device__ __forceinline__ void port_at(float4 (&v)[kPlanes], bool west, const RowBC& b, const StepArgs& a, const T* S,
                                         long long oC)
 {
@@ -156,7 +159,7 @@ __device__ __forceinline__ void port_at(float4 (&v)[kPlanes], bool west, const R
     for (int i = 0; i < 9; ++i) f[i] = at(v[i], k);
 #pragma unroll
     for (int i = 0; i < 5; ++i) g[i] = at(v[9 + i], k);
-    port_node(f, g, west, b, a, S, oC + k);
+    port_node<kRescale>(f, g, west, b, a, S, oC + k);
 #pragma unroll
     for (int i = 0; i < 9; ++i) at(v[i], k) = f[i];
 #pragma unroll
@@ -165,7 +168,7 @@ __device__ __forceinline__ void port_at(float4 (&v)[kPlanes], bool west, const R
 
 // Completion of the open port nodes among a lane's quad; bc: the row's west
 // and east port entries.
-template <typename T>
+template <bool kRescale, typename T>
 __device__ __forceinline__ void port_pass(float4 (&v)[kPlanes], int x0, const RowBC* bc, const StepArgs& a, const T* S,
                                           long long oC)
 {
@@ -174,10 +177,10 @@ __device__ __forceinline__ void port_pass(float4 (&v)[kPlanes], int x0, const Ro
         const RowBC b = side == 0 ? bc[0] : bc[1];
         if (b.x < x0 || b.x >= x0 + 4 || !valve_open(a, b.chan_kind)) continue;
         switch (b.x - x0) {
-        case 0: port_at<0>(v, side == 0, b, a, S, oC); break;
-        case 1: port_at<1>(v, side == 0, b, a, S, oC); break;
-        case 2: port_at<2>(v, side == 0, b, a, S, oC); break;
-        default: port_at<3>(v, side == 0, b, a, S, oC); break;
+        case 0: port_at<kRescale, 0>(v, side == 0, b, a, S, oC); break;
+        case 1: port_at<kRescale, 1>(v, side == 0, b, a, S, oC); break;
+        case 2: port_at<kRescale, 2>(v, side == 0, b, a, S, oC); break;
+        default: port_at<kRescale, 3>(v, side == 0, b, a, S, oC); break;
         }
     }
 }
@@ -253,12 +256,12 @@ __device__ __forceinline__ void bounce_side(float4 (&v)[kPlanes], unsigned lk, c
 
 // Walls and ports of the lane's pulled quads; S, P and oC: the nodes' own
 // stored populations.
-template <typename T>
+template <bool kRescale, typename T>
 __device__ __forceinline__ void complete_quad(const StepArgs& a, bool port, float4 (&v)[kPlanes], unsigned lk,
                                               unsigned groups, int x0, const RowBC* bc, const T* S, long long P, long long oC)
 {
     bounce_groups<T>(v, lk, groups, S, P, oC);
-    if (port) port_pass<T>(v, x0, bc, a, S, oC);
+    if (port) port_pass<kRescale, T>(v, x0, bc, a, S, oC);
 }
 
 // Collisions of the lane's quad.
@@ -270,7 +273,7 @@ __device__ __forceinline__ void collide_row(const StepArgs& a, float4 (&v)[kPlan
     bad |= q.bad;
 }
 
-template <typename T>
+template <typename T, bool kRescale>
 __global__ void __launch_bounds__(32 * kPairWarps<T>, kPairBlocks)
     coupled_step_pair(const PairArgs p, const __grid_constant__ CUtensorMap map)
 {
@@ -382,7 +385,7 @@ __global__ void __launch_bounds__(32 * kPairWarps<T>, kPairBlocks)
         // ---- first step of row j, into the ring once the second steps of
         //      the iteration before have read it ----
         if (lk != 0xFFFFFFFFu) {
-            complete_quad(p.first, st.port, v, lk, at_side ? 0x0Au : 0xFFu, st.x0 + 4 * lane, bc, src, P,
+            complete_quad<kRescale>(p.first, st.port, v, lk, at_side ? 0x0Au : 0xFFu, st.x0 + 4 * lane, bc, src, P,
                           (long long)y * pitch + st.x0 + 4 * lane);
             collide_row<T>(p.first, v, lk, rates_of(p.first, rates), bad);
         }
@@ -430,7 +433,7 @@ __global__ void __launch_bounds__(32 * kPairWarps<T>, kPairBlocks)
                 v[q] = r;
             }
             if (lk != 0xFFFFFFFFu)
-                complete_quad(p.second, st.port, v, lk, 0xFFu, st.x0 + 4 * lane, rC.bc,
+                complete_quad<kRescale>(p.second, st.port, v, lk, 0xFFu, st.x0 + 4 * lane, rC.bc,
                               reinterpret_cast<const Shared<T>*>(&rC.pl[0][0]), kTileNodes, 4 * lane);
         }
         __syncwarp();
@@ -458,7 +461,7 @@ __global__ void __launch_bounds__(32 * kPairWarps<T>, kPairBlocks)
     if (__any_sync(kFull, bad) && lane == 0) atomicOr(p.first.err, 1u);
 }
 
-template <typename T>
+template <typename T, bool kRescale>
 cudaError_t launch(const PairArgs& p, const CUtensorMap& map, int grid, cudaStream_t s)
 {
     cudaLaunchConfig_t cfg = {};
@@ -471,27 +474,28 @@ cudaError_t launch(const PairArgs& p, const CUtensorMap& map, int grid, cudaStre
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, coupled_step_pair<T>, p, map);
+    return cudaLaunchKernelEx(&cfg, coupled_step_pair<T, kRescale>, p, map);
 }
 
-template <typename T>
+template <typename T, bool kRescale>
 cudaError_t occupancy(int* per_sm)
 {
-    cudaError_t e = cudaFuncSetAttribute(coupled_step_pair<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(coupled_step_pair<T, kRescale>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          int(sizeof(PairSmem<T>)));
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, coupled_step_pair<T>, 32 * kPairWarps<T>,
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, coupled_step_pair<T, kRescale>, 32 * kPairWarps<T>,
                                                           sizeof(PairSmem<T>));
     return e;
 }
 
 }  // namespace
 
-cudaError_t pair_occupancy(int precision, int* per_sm)
+cudaError_t pair_occupancy(int precision, bool rescale, int* per_sm)
 {
-    if (precision == kFP16) return occupancy<__half>(per_sm);
-    if (precision == kBF16) return occupancy<__nv_bfloat16>(per_sm);
-    return occupancy<float>(per_sm);
+    if (precision == kFP16) return rescale ? occupancy<__half, true>(per_sm) : occupancy<__half, false>(per_sm);
+    if (precision == kBF16)
+        return rescale ? occupancy<__nv_bfloat16, true>(per_sm) : occupancy<__nv_bfloat16, false>(per_sm);
+    return rescale ? occupancy<float, true>(per_sm) : occupancy<float, false>(per_sm);
 }
 
 int pair_warps(int precision) { return precision == kFP32 ? kPairWarps<float> : kPairWarps<__half>; }
@@ -525,11 +529,19 @@ cudaError_t pair_tensor_map(CUtensorMap* map, void* pop, int ny, int pitch, int 
                            pair_warps(precision));
 }
 
-cudaError_t launch_step_pair(const PairArgs& p, const CUtensorMap& map, int grid, int precision, cudaStream_t s)
+template <bool kRescale>
+static cudaError_t launch_precision(const PairArgs& p, const CUtensorMap& map, int grid, int precision, cudaStream_t s)
 {
-    cudaError_t e = precision == kFP16   ? launch<__half>(p, map, grid, s)
-                    : precision == kBF16 ? launch<__nv_bfloat16>(p, map, grid, s)
-                                         : launch<float>(p, map, grid, s);
+    return precision == kFP16   ? launch<__half, kRescale>(p, map, grid, s)
+           : precision == kBF16 ? launch<__nv_bfloat16, kRescale>(p, map, grid, s)
+                                : launch<float, kRescale>(p, map, grid, s);
+}
+
+cudaError_t launch_step_pair(const PairArgs& p, const CUtensorMap& map, int grid, int precision, bool rescale,
+                             cudaStream_t s)
+{
+    const cudaError_t e = rescale ? launch_precision<true>(p, map, grid, precision, s)
+                                  : launch_precision<false>(p, map, grid, precision, s);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }

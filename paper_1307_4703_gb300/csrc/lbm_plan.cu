@@ -283,19 +283,25 @@ std::vector<Run> runs_of(const std::vector<uint2>& tiles, const std::vector<RowB
 }  // namespace
 
 StripPlan plan_pairs(const std::vector<uint2>& tiles, const std::vector<RowBC>& bc, int nx, int ny, int pitch,
-                     int precision, int warps, int resident)
+                     int precision, int warps, int resident, long long single_warps)
 {
     StripPlan p = plan(runs_of(tiles, bc, nx, ny, pitch, 1), kPairCost, 1, warps, resident);
-    // Where two single steps are the better choice (FP32 only): a lattice whose
-    // blocks fill most of the GPU and repeat so many rows that they do more than
-    // 0.85 of the single steps' work.
-    // Measured, single against two-step launches in us a step: 0.59 of the work
-    // 61.2 / 39.3 (4096 x 2048), 0.69 111.3 / 80 (64 chips), 0.81 7.25 / 6.89 (1024 x
-    // 768), 1.2 5.42 / 5.41 (1024 x 512) and 4.90 / 5.12 (700 x 500); a GPU less than
-    // half full: 3.63 / 2.66 (256 x 128), 3.81 / 2.79 (400 x 300).  16-bit storage gains
-    // throughout (37.4 / 30.1, 89.8 / 67.9, 6.20 / 5.55, 5.96 / 5.25, 5.29 / 3.73, 4.81 /
-    // 2.95): its single step is bound by issue and starts up longer.
-    p.worth = precision != kFP32 || 2 * p.grid <= resident || p.work < 0.85 * 2.0 * double(tiles.size());
+    // Where two single steps are the better choice, in us a step, single / two-step
+    // launches.  FP32: a single step whose warps take one tile each is over as soon as
+    // the strips' three or four rows a warp (1024 x 512 5.25 / 5.15, 900 x 700 5.25 /
+    // 6.6, 700 x 500 4.8 / 5.0), unless the strips leave half the blocks' room idle
+    // (256 x 128 3.65 / 2.57, 512 x 256 3.65 / 2.73).  From the second tile a warp on
+    // the strips win, the more the larger the lattice is (1024 x 768 7.1 / 6.7, 1300 x
+    // 800 9.0 / 7.3, 4096 x 2048 59.8 / 39.2; with 3 % obstacles 800 x 500 10.2 / 9.0,
+    // 2001 x 1003 40.7 / 33.1).  16-bit storage, whose single step is bound by issue and
+    // starts up longer, gains nearly throughout (256 x 128 4.8 / 2.8, 1024 x 512 5.4 / 5.0, 1024 x
+    // 768 6.3 / 5.4, 4096 x 2048 37.4 / 29.3; 1300 x 800 7.0 / 7.25).  Neither does where
+    // obstacles break the rows into strips that do far more than the tiles' work: at
+    // 1.7 to 1.8 of it FP32 22.2 / 25.4 and 47.7 / 50.5, at 2.1 FP16 19.5 / 20.7.
+    const bool idle = 2 * p.grid <= resident;
+    const double work = p.work / (2.0 * double(tiles.size()));
+    if (precision == kFP32) p.worth = idle || (work < 1.5 && (long long)tiles.size() > single_warps);
+    else p.worth = idle || work < 1.8;
     return p;
 }
 

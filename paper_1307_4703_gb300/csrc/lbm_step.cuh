@@ -34,9 +34,18 @@ __device__ __forceinline__ TileRange warp_tiles(const StepArgs& a, int warp, int
 // kWhole: every tile of the table with the grid's stride, read from the
 // kernel parameters (the FP32 kernel sits at its register limit, where the
 // range held in registers makes it spill).
-template <typename T, bool kWalls, bool kPortCode, bool kWhole = false>
+// kStaged (FP32 without ports of the rescaling kinds): the bounce-back entries
+// come through shared memory, all in flight with the free flight's loads
+// (bounce_issue), where bounce_back waits for each link's in turn.  Without the
+// rescaling kinds' call the copies' code fits the registers; with it the kernel
+// spills and is slower.  us a step, before / after: 1001 x 517 with 3 %
+// obstacles 11.0 / 10.5, chips of 1024 x 512 5.43 / 5.25, 1024 x 768 7.25 / 7.07, 4096 x
+// 2048 61.5 / 59.5.
+template <typename T, bool kWalls, bool kPortCode, bool kWhole = false, bool kStaged = false>
 __device__ __forceinline__ void regs_loop(const StepArgs& a, TileRange r, int lane, LaneDiag& diag, bool& bad)
 {
+    extern __shared__ __align__(16) unsigned char stage_smem[];
+    BounceStage& stage = reinterpret_cast<BounceStage*>(stage_smem)[threadIdx.x >> 5];
     if constexpr (kWhole) {
         r.tiles = a.tiles;
         r.n = a.n_tiles;
@@ -73,14 +82,17 @@ __device__ __forceinline__ void regs_loop(const StepArgs& a, TileRange r, int la
 
         // ---- free flight (pull): v[p] component k = plane p at (x0+k) - e ----
         float4 v[kPlanes];
+        const unsigned wall = kStaged ? wall_links(lk) : 0u;
+        if constexpr (kStaged) bounce_issue(stage, wall, S, P, oC, lane);
         pull_quad<false>(v, S, P, oC, oS, oN, halo_w, halo_e, act, ld_w, ld_e, lane);
+        if constexpr (kStaged) bounce_staged(v, lk, wall, stage, lane);
         if (act) {
-            bounce_back<T, kWalls>(v, lk, S, P, oC, static_cast<const T*>(a.wallv));
+            if constexpr (!kStaged) bounce_back<T, kWalls>(v, lk, S, P, oC, static_cast<const T*>(a.wallv));
             QuadAcc q;
             if constexpr (kPortCode) {
                 const RowBC bw = a.rowbc[y];
                 const RowBC be = a.rowbc[a.ny + y];
-                collide_quad<T, !kStoresF32<T>, true>(v, lk, x0, bw, be, a, S, oC, row_rates(a, y), q);
+                collide_quad<T, !kStoresF32<T>, true, !kStaged>(v, lk, x0, bw, be, a, S, oC, row_rates(a, y), q);
             } else {
                 collide_quad<T, !kStoresF32<T>, false>(v, lk, x0, RowBC{}, RowBC{}, a, S, oC, row_rates(a, y), q);
             }
@@ -93,7 +105,7 @@ __device__ __forceinline__ void regs_loop(const StepArgs& a, TileRange r, int la
     }
 }
 
-template <typename T, bool kWalls, bool kFold = false>
+template <typename T, bool kWalls, bool kFold = false, bool kStaged = false>
 __global__ void __launch_bounds__(256, 2) coupled_step_regs(const StepArgs a)
 {
     const int lane = threadIdx.x & 31;
@@ -102,7 +114,8 @@ __global__ void __launch_bounds__(256, 2) coupled_step_regs(const StepArgs a)
     LaneDiag diag;
     bool bad = false;
     if constexpr (kStoresF32<T>) {  // one loop over every tile (port_blocks is 0 for FP32)
-        regs_loop<T, kWalls, true, true>(a, TileRange{nullptr, 0, int(blockIdx.x) * wpb + warp, 0}, lane, diag, bad);
+        regs_loop<T, kWalls, true, true, kStaged>(a, TileRange{nullptr, 0, int(blockIdx.x) * wpb + warp, 0}, lane, diag,
+                                                   bad);
     } else {
         bool port_loop;
         const TileRange r = warp_tiles(a, warp, wpb, port_loop);
