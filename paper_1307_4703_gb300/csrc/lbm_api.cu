@@ -1024,7 +1024,7 @@ lbm_status create_impl(lbm_handle* out, int32_t nx, int32_t ny, const uint8_t* m
         for (int b = 0; b < 2 && have; ++b)
             have = lbm::pair_tensor_map(&h->pair_map[b], h->pop[b], ny, pitch, h->precision) == cudaSuccess;
         if (have) {
-            plan = lbm::plan_pairs(h->tiles_rows, rowbc, nx, ny, pitch, h->precision, lbm::pair_warps(h->precision),
+            plan = lbm::plan_pairs(h->tiles_rows, rowbc, nx, ny, pitch, h->precision, h->paper_ports, lbm::pair_warps(h->precision),
                                    pair_per_sm * sms, (long long)h->launch.grid * (h->launch.block / 32));
             h->pair_items = static_cast<int4*>(dev_alloc(h, plan.items.size() * sizeof(int4)));
             h->pair_first = static_cast<int*>(dev_alloc(h, plan.block_first.size() * sizeof(int)));

@@ -1027,6 +1027,134 @@ __device__ __forceinline__ NodeMoments collide_node(float (&f)[9], float (&g)[5]
     }
 }
 
+// collide_node for two nodes at once in packed arithmetic (two FP32 operations
+// an instruction, each rounded as by itself), which halves the instructions of
+// the collision where issue sets the pace.  Products that collide_node leaves to
+// the compiler to fuse into sums are written out here the way that gives its
+// bits.  us a step, one by one / packed: two-step launches of 1024 x 768 6.75 /
+// 6.30, 1001 x 517 with obstacles 10.0 / 9.35, 4096 x 2048 FP16 29.2 / 28.1, 64 chips
+// FP16 65.0 / 61.7; the FP16 single step 37.4 / 36.2.  The FP32 single step, at its
+// 128 registers, spills with it (5.25 / 6.8 at 1024 x 512).
+struct PairMoments {
+    float2 rd, rho, jx, ux, C;
+};
+__device__ __forceinline__ float2 two(float x) { return make_float2(x, x); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, two(-1.f), a); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+
+template <bool kDev>
+__device__ __forceinline__ PairMoments collide_two(float2 (&f)[9], float2 (&g)[5], float2 omega, float dfac,
+                                                   const StepArgs& a)
+{
+    if constexpr (kDev) {
+        const float2 s56 = add2(f[5], f[6]), s78 = add2(f[7], f[8]);
+        const float2 rd = add2(add2(add2(f[0], add2(f[1], f[3])), add2(f[2], f[4])), add2(s56, s78));
+        const float2 rho = add2(two(1.f), rd);
+        const float2 jx = add2(add2(sub2(f[1], f[3]), sub2(f[5], f[6])), sub2(f[8], f[7]));
+        const float2 jy = add2(sub2(f[2], f[4]), sub2(s56, s78));
+        const float2 inv = make_float2(__fdividef(1.f, rho.x), __fdividef(1.f, rho.y));
+        const float2 ux = mul2(jx, inv), uy = mul2(jy, inv);
+        {
+            const float2 om = two(1.f - omega.x), wa = two(omega.x * kWa);
+            const float2 p1 = mul2(jx, ux), p2 = mul2(jy, uy);
+            const float2 B = fma2(two(-1.5f), add2(p1, p2), rd);
+            const float2 j5 = add2(jx, jy), j6 = sub2(jy, jx);
+            const float2 y1 = fma2(two(4.5f), p1, B), y2 = fma2(two(4.5f), p2, B);
+            const float2 Bq = mul2(two(0.25f), B);
+            const float2 y5 = fma2(mul2(two(1.125f), j5), add2(ux, uy), Bq);
+            const float2 y6 = fma2(mul2(two(1.125f), j6), sub2(uy, ux), Bq);
+            f[0] = fma2(wa, mul2(two(4.f), B), mul2(om, f[0]));
+            f[1] = fma2(wa, fma2(two(3.f), jx, y1), mul2(om, f[1]));
+            f[3] = fma2(wa, fma2(two(-3.f), jx, y1), mul2(om, f[3]));
+            f[2] = fma2(wa, fma2(two(3.f), jy, y2), mul2(om, f[2]));
+            f[4] = fma2(wa, fma2(two(-3.f), jy, y2), mul2(om, f[4]));
+            f[5] = fma2(wa, fma2(two(0.75f), j5, y5), mul2(om, f[5]));
+            f[7] = fma2(wa, fma2(two(-0.75f), j5, y5), mul2(om, f[7]));
+            f[6] = fma2(wa, fma2(two(0.75f), j6, y6), mul2(om, f[6]));
+            f[8] = fma2(wa, fma2(two(-0.75f), j6, y6), mul2(om, f[8]));
+        }
+        const float2 C = add2(add2(add2(add2(g[0], g[1]), add2(g[2], g[3])), g[4]), two(kCRef));
+        {
+            const float wg = omega.y;
+            const float2 om = two(1.f - wg);
+            const float2 wC = fma2(C, two(wg * dfac), two(-(wg * kCRef)));
+            const float2 w1C = mul2(two(a.wg1), wC);
+            const float ckc = (wg * a.wg1) * a.inv_cs2g;
+            const float2 ck = mul2(two(ckc), C), nck = mul2(two(-ckc), C);
+            g[0] = fma2(om, g[0], fma2(two(-4.f), w1C, wC));
+            g[1] = fma2(om, g[1], fma2(ck, ux, w1C));
+            g[3] = fma2(om, g[3], fma2(nck, ux, w1C));
+            g[2] = fma2(om, g[2], fma2(ck, uy, w1C));
+            g[4] = fma2(om, g[4], fma2(nck, uy, w1C));
+        }
+        return PairMoments{rd, rho, jx, ux, C};
+    } else {
+        const float2 rd = add2(add2(add2(add2(f[0], f[1]), add2(f[2], f[3])), add2(add2(f[4], f[5]), add2(f[6], f[7]))), f[8]);
+        const float2 rho = add2(two(1.f), rd);
+        const float2 jx = add2(add2(sub2(f[1], f[3]), sub2(f[5], f[6])), sub2(f[8], f[7]));
+        const float2 jy = sub2(add2(sub2(f[2], f[4]), add2(f[5], f[6])), add2(f[7], f[8]));
+        const float2 inv = make_float2(__fdividef(1.f, rho.x), __fdividef(1.f, rho.y));
+        const float2 ux = mul2(jx, inv), uy = mul2(jy, inv);
+        const float2 usq = mul2(two(-1.5f), fma2(ux, ux, mul2(uy, uy)));  // -3/2 u^2
+        {
+            const float2 wo = two(omega.x);
+            auto square = [&](float2 e) { return fma2(mul2(two(4.5f), e), e, usq); };
+            // f + omega (w x - f)
+            auto relax = [&](float2& fi, float w, float2 x) {
+                fi = fma2(wo, fma2(two(w), x, mul2(two(-1.f), fi)), fi);
+            };
+            const float2 q1 = square(ux), q2 = square(uy), q5 = square(add2(ux, uy)), q6 = square(sub2(uy, ux));
+            const float2 t2 = mul2(two(3.f), jy), t5 = fma2(two(3.f), jx, t2), t6 = fma2(two(-3.f), jx, t2);
+            relax(f[0], kWr, fma2(rho, usq, rd));
+            relax(f[1], kWa, fma2(rho, q1, fma2(two(3.f), jx, rd)));
+            relax(f[3], kWa, fma2(rho, q1, fma2(two(-3.f), jx, rd)));
+            relax(f[2], kWa, fma2(rho, q2, add2(rd, t2)));
+            relax(f[4], kWa, fma2(rho, q2, sub2(rd, t2)));
+            relax(f[5], kWd, fma2(rho, q5, add2(rd, t5)));
+            relax(f[7], kWd, fma2(rho, q5, sub2(rd, t5)));
+            relax(f[6], kWd, fma2(rho, q6, add2(rd, t6)));
+            relax(f[8], kWd, fma2(rho, q6, sub2(rd, t6)));
+        }
+        const float2 C = add2(add2(add2(g[0], g[1]), add2(g[2], g[3])), g[4]);
+        {
+            const float2 wg = two(omega.y);
+            const float2 Cd = mul2(C, two(dfac)), c1 = mul2(two(a.wg1), C), c1d = mul2(two(a.wg1), Cd);
+            const float2 ci = mul2(c1, two(a.inv_cs2g)), nci = mul2(c1, two(-a.inv_cs2g));
+            g[0] = fma2(wg, sub2(fma2(two(-4.f), c1d, Cd), g[0]), g[0]);
+            g[1] = fma2(wg, sub2(fma2(ci, ux, c1d), g[1]), g[1]);
+            g[3] = fma2(wg, sub2(fma2(nci, ux, c1d), g[3]), g[3]);
+            g[2] = fma2(wg, sub2(fma2(ci, uy, c1d), g[2]), g[2]);
+            g[4] = fma2(wg, sub2(fma2(nci, uy, c1d), g[4]), g[4]);
+        }
+        return PairMoments{rd, rho, jx, ux, C};
+    }
+}
+
+// The same by collide_node.
+template <bool kDev>
+__device__ __forceinline__ PairMoments collide_each(float2 (&f)[9], float2 (&g)[5], float2 omega, float dfac,
+                                                    const StepArgs& a)
+{
+    NodeMoments m[2];
+#pragma unroll
+    for (int n = 0; n < 2; ++n) {
+        float fn[9], gn[5];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) fn[i] = at(f[i], n);
+#pragma unroll
+        for (int i = 0; i < 5; ++i) gn[i] = at(g[i], n);
+        m[n] = collide_node<kDev>(fn, gn, omega, dfac, a);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) at(f[i], n) = fn[i];
+#pragma unroll
+        for (int i = 0; i < 5; ++i) at(g[i], n) = gn[i];
+    }
+    return PairMoments{make_float2(m[0].rd, m[1].rd), make_float2(m[0].rho, m[1].rho), make_float2(m[0].jx, m[1].jx),
+                       make_float2(m[0].ux, m[1].ux), make_float2(m[0].C, m[1].C)};
+}
+
 // Open ports, moments and both collisions of the quad.  Where the rare work
 // goes depends on the storage type, by measurement: the FP32 kernel waits on
 // its loads and is fastest with the port and solid-node handling inside the
@@ -1036,12 +1164,13 @@ __device__ __forceinline__ NodeMoments collide_node(float (&f)[9], float (&g)[5]
 // port or a solid node enter (FP16 50.1 us, against 52.3 us inside the loop).
 // kPasses selects the passes (the multi-step kernel takes them for FP32 too:
 // there they keep its registers from spilling).  Both forms give the same
-// bits.  kPorts = false leaves the port code out, for tiles whose row
-// segment holds no port node (kPortTile): present in the node loop, it costs
-// the step even where it never runs (a timing copy without it: FP16 44.1 us
-// against 48.0 us on the 4096 x 2048 chip).  The register kernels take the
-// port-free form for those tiles and the pass form for the few others.
-template <typename T, bool kPasses = !kStoresF32<T>, bool kPorts = true, bool kRescale = true>
+// bits.  kPacked: collide_two, for passes.  kPorts = false leaves the port
+// code out, for tiles whose row segment holds no port node (kPortTile):
+// present in the node loop, it costs the step even where it never runs (a
+// timing copy without it: FP16 44.1 us against 48.0 us on the 4096 x 2048
+// chip).  The register kernels take the port-free form for those tiles and the
+// pass form for the few others.
+template <typename T, bool kPasses = !kStoresF32<T>, bool kPorts = true, bool kRescale = true, bool kPacked = false>
 __device__ __forceinline__ void collide_quad(float4 (&v)[kPlanes], unsigned lk, int x0, const RowBC& bw,
                                              const RowBC& be, const StepArgs& a, const T* S, long long oC,
                                              float2 omega, QuadAcc& acc)
@@ -1086,57 +1215,35 @@ __device__ __forceinline__ void collide_quad(float4 (&v)[kPlanes], unsigned lk, 
         }
     }
 
-    float rmin = 1.f;  // smallest density of the quad's fluid nodes (passes)
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const unsigned lb = (lk >> (8 * k)) & 0xFFu;
-        const bool fluid = lb != kSolid;
-        float f[9], g[5];
-#pragma unroll
-        for (int i = 0; i < 9; ++i) f[i] = at(v[i], k);
-#pragma unroll
-        for (int i = 0; i < 5; ++i) g[i] = at(v[9 + i], k);
-        bool outlet_k = (outlet >> k) & 1u;
-        if constexpr (!kPasses) {
-            if (!fluid) {  // solid node: park it at the rest state rho = 1, C = 0
-#pragma unroll
-                for (int i = 0; i < 9; ++i) f[i] = 0.f;
-#pragma unroll
-                for (int i = 0; i < 5; ++i) g[i] = 0.f;
-            }
-            // ---- open valve ports ----
-            if constexpr (kPorts) {
-                const int xk = x0 + k;
-                const bool pw = open_w && bw.x == xk;
-                const bool pe = !pw && open_e && be.x == xk;
-                if (pw || pe) outlet_k = port_node<kRescale>(f, g, pw, pw ? bw : be, a, S, oC + k);
-            }
-        }
-
-        const NodeMoments nm = collide_node<kDev>(f, g, omega, dfac, a);
-        const float rd = nm.rd, rho = nm.rho, jx = nm.jx, ux = nm.ux, C = nm.C;
-#pragma unroll
-        for (int i = 0; i < 9; ++i) at(v[i], k) = f[i];
-#pragma unroll
-        for (int i = 0; i < 5; ++i) at(v[9 + i], k) = g[i];
-
-        if (fluid) {
-            if constexpr (kPasses) {
-                rmin = fminf(rmin, rho);
-            } else {
-                acc.bad |= !(rho > 0.f && rho < INFINITY) || !(fabsf(C) < INFINITY);
-                ++acc.n;
-            }
-            acc.m += rd;
-            acc.c += C;
-            if (outlet_k) {
-                acc.q += jx;  // rho u_x
-                acc.qc += C * ux;
-            }
-        }
-    }
-
     if constexpr (kPasses) {
+        float rmin = 1.f;  // smallest density of the quad's fluid nodes
+#pragma unroll
+        for (int k = 0; k < 4; k += 2) {
+            float2 f[9], g[5];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) f[i] = make_float2(at(v[i], k), at(v[i], k + 1));
+#pragma unroll
+            for (int i = 0; i < 5; ++i) g[i] = make_float2(at(v[9 + i], k), at(v[9 + i], k + 1));
+            PairMoments nm;
+            if constexpr (kPacked) nm = collide_two<kDev>(f, g, omega, dfac, a);
+            else nm = collide_each<kDev>(f, g, omega, dfac, a);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) at(v[i], k) = f[i].x, at(v[i], k + 1) = f[i].y;
+#pragma unroll
+            for (int i = 0; i < 5; ++i) at(v[9 + i], k) = g[i].x, at(v[9 + i], k + 1) = g[i].y;
+#pragma unroll
+            for (int n = 0; n < 2; ++n) {
+                if (((lk >> (8 * (k + n))) & 0xFFu) == kSolid) continue;
+                rmin = fminf(rmin, n ? nm.rho.y : nm.rho.x);
+                acc.m += n ? nm.rd.y : nm.rd.x;
+                const float C = n ? nm.C.y : nm.C.x;
+                acc.c += C;
+                if ((outlet >> (k + n)) & 1u) {
+                    acc.q += n ? nm.jx.y : nm.jx.x;  // rho u_x
+                    acc.qc += C * (n ? nm.ux.y : nm.ux.x);
+                }
+            }
+        }
         // a non-finite density or concentration makes its quad sum non-finite
         acc.bad = !(rmin > 0.f) || !(fabsf(acc.m) < INFINITY) || !(fabsf(acc.c) < INFINITY);
         // ---- solid nodes: parked at the rest state rho = 1, C = 0 (what
@@ -1154,6 +1261,48 @@ __device__ __forceinline__ void collide_quad(float4 (&v)[kPlanes], unsigned lk, 
                 at(v[9], k) = kDev ? -a.gref0 : 0.f;
 #pragma unroll
                 for (int i = 10; i < 14; ++i) at(v[i], k) = kDev ? -a.gref1 : 0.f;
+            }
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const bool fluid = ((lk >> (8 * k)) & 0xFFu) != kSolid;
+            float f[9], g[5];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) f[i] = at(v[i], k);
+#pragma unroll
+            for (int i = 0; i < 5; ++i) g[i] = at(v[9 + i], k);
+            bool outlet_k = false;
+            if (!fluid) {  // solid node: park it at the rest state rho = 1, C = 0
+#pragma unroll
+                for (int i = 0; i < 9; ++i) f[i] = 0.f;
+#pragma unroll
+                for (int i = 0; i < 5; ++i) g[i] = 0.f;
+            }
+            // ---- open valve ports ----
+            if constexpr (kPorts) {
+                const int xk = x0 + k;
+                const bool pw = open_w && bw.x == xk;
+                const bool pe = !pw && open_e && be.x == xk;
+                if (pw || pe) outlet_k = port_node<kRescale>(f, g, pw, pw ? bw : be, a, S, oC + k);
+            }
+
+            const NodeMoments nm = collide_node<kDev>(f, g, omega, dfac, a);
+            const float rd = nm.rd, rho = nm.rho, jx = nm.jx, ux = nm.ux, C = nm.C;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) at(v[i], k) = f[i];
+#pragma unroll
+            for (int i = 0; i < 5; ++i) at(v[9 + i], k) = g[i];
+
+            if (fluid) {
+                acc.bad |= !(rho > 0.f && rho < INFINITY) || !(fabsf(C) < INFINITY);
+                ++acc.n;
+                acc.m += rd;
+                acc.c += C;
+                if (outlet_k) {
+                    acc.q += jx;  // rho u_x
+                    acc.qc += C * ux;
+                }
             }
         }
     }

@@ -465,6 +465,12 @@ cudaError_t prepare_step_kernels()
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(coupled_step_async<__nv_bfloat16, false>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, async_max);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(coupled_step_async<__half, false, false, false>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, async_max);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(coupled_step_async<__nv_bfloat16, false, false, false>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, async_max);
     if (e == cudaSuccess) e = prepare_walls_kernels();
     if (e == cudaSuccess) e = prepare_fold_kernels();
     return e;
@@ -519,8 +525,12 @@ cudaError_t launch_step(const StepArgs& a, const StepLaunch& l, cudaStream_t s)
         e = cudaLaunchKernelEx(&cfg, coupled_step_pipe, a, per);
     } else if (l.variant == kVariantAsync) {
         cfg.dynamicSmemBytes = async_smem_bytes(l.block, l.precision);
-        if (l.precision == kFP16) e = cudaLaunchKernelEx(&cfg, coupled_step_async<__half, false>, b);
-        else if (l.precision == kBF16) e = cudaLaunchKernelEx(&cfg, coupled_step_async<__nv_bfloat16, false>, b);
+        if (l.precision == kFP16)
+            e = l.rescale ? cudaLaunchKernelEx(&cfg, coupled_step_async<__half, false>, b)
+                          : cudaLaunchKernelEx(&cfg, coupled_step_async<__half, false, false, false>, b);
+        else if (l.precision == kBF16)
+            e = l.rescale ? cudaLaunchKernelEx(&cfg, coupled_step_async<__nv_bfloat16, false>, b)
+                          : cudaLaunchKernelEx(&cfg, coupled_step_async<__nv_bfloat16, false, false, false>, b);
         else e = cudaLaunchKernelEx(&cfg, coupled_step_async<float, false>, b);
     } else if (l.variant == kVariantPairs) {
         e = cudaLaunchKernelEx(&cfg, coupled_step_pairs, a);  // FP32 storage only
@@ -604,6 +614,12 @@ cudaError_t step_kernel_occupancy(const StepLaunch& l, int* blocks_per_sm)
                                                              bulk_smem_bytes(l.stages));
     if (l.variant == kVariantAsync) {
         const size_t smem = async_smem_bytes(l.block, l.precision);
+        if (l.precision == kFP16 && !l.rescale)
+            return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                blocks_per_sm, coupled_step_async<__half, false, false, false>, l.block, smem);
+        if (l.precision == kBF16 && !l.rescale)
+            return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                blocks_per_sm, coupled_step_async<__nv_bfloat16, false, false, false>, l.block, smem);
         if (l.precision == kFP16)
             return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, coupled_step_async<__half, false>,
                                                                  l.block, smem);

@@ -26,8 +26,8 @@
 //   - a strip along a side wall names the two lanes at it, and these bounce
 //     back from the staged rows (from global memory, such strips took 1.5
 //     times as long as the others and set the launch's length).
-// Steps of the 4096 x 2048 chip, us: FP32 59.5 one by one, 39.0 here; FP16
-// 37.4 -> 29.2; 64 chips in a batch 111 -> 79.6 (FP32).  Tried: the second
+// Steps of the 4096 x 2048 chip, us: FP32 59.5 one by one, 38.0 here; FP16
+// 36.2 -> 28.1; 64 chips in a batch 111 -> 77.0 (FP32).  Tried: the second
 // step's rows written by bulk copies from shared memory (50.4 against 46.7
 // us at that stage: 14 copies a row by one warp are slow to issue); rows
 // copied lane by lane (cp.async: FP32 the same, FP16 34.7 against 30.5 us);
@@ -149,7 +149,8 @@ __device__ __forceinline__ void pull_staged(float4 (&v)[kPlanes], const PairSmem
 // Completion of the open port node k of a lane's quad.  kRescale: the lattice
 // has ports of the rescaling kinds, whose completion is a call (complete_port);
 // kernels without it are 2 to 6 % faster (4096 x 2048 in FP32 39.4 -> 39.0 us a
-// step, FP16 30.1 -> 29.3; 256 x 128 2.70 -> 2.60, FP16 2.97 -> 2.79).
+// step, FP16 30.1 -> 29.3; 256 x 128 2.70 -> 2.60, FP16 2.97 -> 2.79, before the
+// packed arithmetic).
 template <bool kRescale, int k, typename T>
 __device__ __forceinline__ void port_at(float4 (&v)[kPlanes], bool west, const RowBC& b, const StepArgs& a, const T* S,
                                         long long oC)
@@ -265,11 +266,15 @@ __device__ __forceinline__ void complete_quad(const StepArgs& a, bool port, floa
 }
 
 // Collisions of the lane's quad.
-template <typename T>
+template <bool kRescale, typename T>
 __device__ __forceinline__ void collide_row(const StepArgs& a, float4 (&v)[kPlanes], unsigned lk, float2 omega, bool& bad)
 {
     QuadAcc q;
-    collide_quad<T, true, false>(v, lk, 0, RowBC{}, RowBC{}, a, static_cast<const T*>(nullptr), 0, omega, q);
+    // packed arithmetic spills in 16-bit storage beside the rescaling call (34.4
+    // against 32.1 us a step at 4096 x 2048)
+    constexpr bool kPacked = !kRescale || kStoresF32<T>;
+    collide_quad<T, true, false, kRescale, kPacked>(v, lk, 0, RowBC{}, RowBC{}, a, static_cast<const T*>(nullptr), 0, omega,
+                                                    q);
     bad |= q.bad;
 }
 
@@ -387,7 +392,7 @@ __global__ void __launch_bounds__(32 * kPairWarps<T>, kPairBlocks)
         if (lk != 0xFFFFFFFFu) {
             complete_quad<kRescale>(p.first, st.port, v, lk, at_side ? 0x0Au : 0xFFu, st.x0 + 4 * lane, bc, src, P,
                           (long long)y * pitch + st.x0 + 4 * lane);
-            collide_row<T>(p.first, v, lk, rates_of(p.first, rates), bad);
+            collide_row<kRescale, T>(p.first, v, lk, rates_of(p.first, rates), bad);
         }
         if (t > 0 && !late) late = !mbar_wait(&sm.read, (t - 1) & 1u);
         if (here) {
@@ -439,7 +444,7 @@ __global__ void __launch_bounds__(32 * kPairWarps<T>, kPairBlocks)
         __syncwarp();
         if (lane == 0) mbar_arrive(&sm.read);
         if (lk != 0xFFFFFFFFu) {
-            collide_row<T>(p.second, v, lk, rates_of(p.second, rates), bad);
+            collide_row<kRescale, T>(p.second, v, lk, rates_of(p.second, rates), bad);
             T* __restrict__ D = reinterpret_cast<T*>(p.second.dst) + (long long)y2 * pitch + st.x0 + 4 * lane;
 #pragma unroll
             for (int q = 0; q < kPlanes; ++q) Codec<T>::st4(D + q * P, v[q], 0.f);

@@ -5,6 +5,7 @@
 
 #include "lbm_plan.h"
 
+
 namespace lbm {
 namespace {
 
@@ -78,9 +79,11 @@ int touched(const std::vector<Strip>& strips, const std::vector<Span>& spans, bo
 // and the batch of 64 chips (the splits that were fastest): side walls add the
 // side lanes' work, ports that of a lane that completes its node alone while
 // its warp waits, and walls anywhere a wait for the nodes' own values in global
-// memory.
+// memory.  (Ports of two coupled steps at 24 instead of 22: 1024 x 768 6.2 us a step
+// against 5.4, 64 chips 77.6 against 77.0; at 20 2000 x 1000 10.7 against 10.4.)
 enum Kind { kPlain, kSide, kScattered, kPort, kScatteredPort };
-constexpr int kPairCost[5] = {16, 18, 28, 24, 36};
+constexpr int kPairCost[5] = {16, 18, 28, 22, 33};
+constexpr int kPairRescaleCost[5] = {16, 18, 28, 30, 42};  // with ports of the rescaling kinds (22: 4096 x 2048 44 us, here 39)
 constexpr int kScalarCost[5] = {16, 20, 24, 28, 32};
 
 struct Run {
@@ -283,25 +286,25 @@ std::vector<Run> runs_of(const std::vector<uint2>& tiles, const std::vector<RowB
 }  // namespace
 
 StripPlan plan_pairs(const std::vector<uint2>& tiles, const std::vector<RowBC>& bc, int nx, int ny, int pitch,
-                     int precision, int warps, int resident, long long single_warps)
+                     int precision, bool rescale, int warps, int resident, long long single_warps)
 {
-    StripPlan p = plan(runs_of(tiles, bc, nx, ny, pitch, 1), kPairCost, 1, warps, resident);
+    StripPlan p = plan(runs_of(tiles, bc, nx, ny, pitch, 1), rescale ? kPairRescaleCost : kPairCost, 1, warps, resident);
     // Where two single steps are the better choice, in us a step, single / two-step
-    // launches.  FP32: a single step whose warps take one tile each is over as soon as
-    // the strips' three or four rows a warp (1024 x 512 5.25 / 5.15, 900 x 700 5.25 /
-    // 6.6, 700 x 500 4.8 / 5.0), unless the strips leave half the blocks' room idle
-    // (256 x 128 3.65 / 2.57, 512 x 256 3.65 / 2.73).  From the second tile a warp on
-    // the strips win, the more the larger the lattice is (1024 x 768 7.1 / 6.7, 1300 x
-    // 800 9.0 / 7.3, 4096 x 2048 59.8 / 39.2; with 3 % obstacles 800 x 500 10.2 / 9.0,
-    // 2001 x 1003 40.7 / 33.1).  16-bit storage, whose single step is bound by issue and
-    // starts up longer, gains nearly throughout (256 x 128 4.8 / 2.8, 1024 x 512 5.4 / 5.0, 1024 x
-    // 768 6.3 / 5.4, 4096 x 2048 37.4 / 29.3; 1300 x 800 7.0 / 7.25).  Neither does where
-    // obstacles break the rows into strips that do far more than the tiles' work: at
-    // 1.7 to 1.8 of it FP32 22.2 / 25.4 and 47.7 / 50.5, at 2.1 FP16 19.5 / 20.7.
+    // launches: where obstacles break the rows into strips that do far more than
+    // the tiles' work.  FP32 at 1.7 and 1.8 of it 22.2 / 25.4 and 47.7 / 50.5, at 1.5 a
+    // draw (6.2 / 6.5, 10.5 / 9.4); 16-bit storage, whose single step is bound by issue
+    // and starts up longer, at 2.1 of it 19.5 / 20.7 and at 1.5 8.1 / 4.2.  Elsewhere two
+    // steps are ahead: FP32 256 x 128 3.65 / 2.52, 1024 x 512 5.24 / 4.60, 1024 x 768
+    // 7.1 / 5.4, 4096 x 2048 59.5 / 38.0, with 3 % obstacles 800 x 500 10.2 / 8.5 and
+    // 2001 x 1003 40.7 / 33; FP16 256 x 128 4.8 / 2.7, 1024 x 768 5.6 / 5.2, 4096 x 2048
+    // 36.2 / 28.1 (900 x 700 is the closest: 5.23 / 5.36 in FP32).  With rescaling
+    // ports FP32 strips gain from the third tile of a single step's warps on (1024 x
+    // 768 7.2 / 7.6, 4096 x 2048 54.4 / 39.0).  Strips that leave half the blocks' room
+    // idle are always the shorter way.
     const bool idle = 2 * p.grid <= resident;
     const double work = p.work / (2.0 * double(tiles.size()));
-    if (precision == kFP32) p.worth = idle || (work < 1.5 && (long long)tiles.size() > single_warps);
-    else p.worth = idle || work < 1.8;
+    const bool few = rescale && precision == kFP32 && (long long)tiles.size() <= 2 * single_warps;
+    p.worth = idle || (!few && work < (precision == kFP32 ? 1.5 : 1.8));
     return p;
 }
 

@@ -17,9 +17,10 @@ struct StripPlan {
 };
 
 // tiles: the lattice's 128-node tiles in row order; bc: 2 ny port entries;
-// warps: of a block; resident: blocks in one wave; single_warps: of the single step's grid.
+// rescale: it has ports of the rescaling kinds; warps: of a block; resident:
+// blocks in one wave; single_warps: of the single step's grid.
 StripPlan plan_pairs(const std::vector<uint2>& tiles, const std::vector<RowBC>& bc, int nx, int ny, int pitch,
-                     int precision, int warps, int resident, long long single_warps);
+                     int precision, bool rescale, int warps, int resident, long long single_warps);
 StripPlan plan_scalar(const std::vector<uint2>& tiles, const std::vector<RowBC>& bc, int nx, int ny, int pitch, int levels,
                       int warps, int resident);
 

@@ -182,7 +182,7 @@ __device__ __forceinline__ void issue_tile_async(const StepArgs& a, const T* S, 
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
-template <typename T, bool kWalls, bool kPortCode>
+template <typename T, bool kWalls, bool kPortCode, bool kRescale = true>
 __device__ __forceinline__ void async_loop(const StepArgs& a, TileRange r, AsyncStage<T>& st, int lane,
                                            LaneDiag& diag, bool& bad)
 {
@@ -226,9 +226,9 @@ __device__ __forceinline__ void async_loop(const StepArgs& a, TileRange r, Async
             if constexpr (kPortCode) {
                 const RowBC bw = a.rowbc[y];
                 const RowBC be = a.rowbc[a.ny + y];
-                collide_quad<T, !kStoresF32<T>, true>(v, lk, x0, bw, be, a, S, oC, row_rates(a, y), q);
+                collide_quad<T, !kStoresF32<T>, true, kRescale, !kRescale>(v, lk, x0, bw, be, a, S, oC, row_rates(a, y), q);
             } else {
-                collide_quad<T, !kStoresF32<T>, false>(v, lk, x0, RowBC{}, RowBC{}, a, S, oC, row_rates(a, y), q);
+                collide_quad<T, !kStoresF32<T>, false, kRescale, !kRescale>(v, lk, x0, RowBC{}, RowBC{}, a, S, oC, row_rates(a, y), q);
             }
 #pragma unroll
             for (int p = 0; p < kPlanes; ++p)
@@ -241,7 +241,7 @@ __device__ __forceinline__ void async_loop(const StepArgs& a, TileRange r, Async
     asm volatile("cp.async.wait_group 0;" ::: "memory");  // nothing in flight at exit
 }
 
-template <typename T, bool kWalls, bool kFold = false>
+template <typename T, bool kWalls, bool kFold = false, bool kRescale = true>
 __global__ void __launch_bounds__(256, 2) coupled_step_async(const StepArgs a)
 {
     // named apart from the bulk kernels' 128-byte aligned smem (one symbol per name)
@@ -259,8 +259,8 @@ __global__ void __launch_bounds__(256, 2) coupled_step_async(const StepArgs a)
     } else {
         bool port_loop;
         const TileRange r = warp_tiles(a, warp, wpb, port_loop);
-        if (port_loop) async_loop<T, kWalls, true>(a, r, st, lane, diag, bad);
-        else async_loop<T, kWalls, false>(a, r, st, lane, diag, bad);
+        if (port_loop) async_loop<T, kWalls, true, kRescale>(a, r, st, lane, diag, bad);
+        else async_loop<T, kWalls, false, kRescale>(a, r, st, lane, diag, bad);
     }
     if (__any_sync(kFull, bad) && lane == 0) atomicOr(a.err, 1u);
     block_partials<kFold>(a, diag);
