@@ -15,6 +15,46 @@
 namespace lbm {
 namespace {
 
+// Completion of an open port node, node n of the pair g (node k of its quad),
+// with velocity ux, uy.  Returns true for an outlet node.
+template <typename Own>
+__device__ __forceinline__ bool scalar_port(float2 (&p)[5], int n, bool west, const RowBC& b, float ux, float uy,
+                                            const ScalarArgs& a, const Own& own, int k)
+{
+    float g[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) g[i] = at(p[i], n);
+    const int gi = west ? 1 : 3;
+    const int kind = (b.chan_kind >> 8) & 0xFF;
+    if (kind == 0) {  // held concentration
+        float others = 0.f;
+#pragma unroll
+        for (int i = 0; i < 5; ++i)
+            if (i != gi) others += g[i];
+        g[gi] = b.c - others;
+    } else {          // do-nothing
+        g[gi] = own(gi, k);
+        if (kind == 3) {  // the paper's inlet: scaled to C_in
+            const float Cs = ((g[0] + g[1]) + (g[2] + g[3])) + g[4];
+            if (Cs > 0.f) {
+                const float gc = b.c / Cs;
+#pragma unroll
+                for (int i = 0; i < 5; ++i) g[i] *= gc;
+            } else {
+                const float c1 = a.wg1 * b.c, cx = c1 * a.inv_cs2g * ux, cy = c1 * a.inv_cs2g * uy;
+                g[0] = b.c - 4.f * c1;
+                g[1] = c1 + cx;
+                g[3] = c1 - cx;
+                g[2] = c1 + cy;
+                g[4] = c1 - cy;
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 5; ++i) at(p[i], n) = g[i];
+    return kind != 0 && kind != 3;
+}
+
 // Ports and relaxation of one lane's quad.  v: the pulled scalar populations,
 // walls bounced back, on entry, the post-collision ones on exit; ux4, uy4: the
 // stored field at the quad; own(i, k): the stored population i of node k; sc,
@@ -28,67 +68,47 @@ __device__ __forceinline__ void scalar_nodes(float4 (&v)[5], unsigned lk, int x0
 {
     const bool open_w = kPorts && bw.x >= 0 && ((a.open_mask >> (bw.chan_kind & 31)) & 1u);
     const bool open_e = kPorts && be.x >= 0 && ((a.open_mask >> (be.chan_kind & 31)) & 1u);
+    const float2 wg = two(a.omega_g);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const bool fluid = kAllFluid || ((lk >> (8 * k)) & 0xFFu) != kSolid;
-        float g[5];
+    for (int h = 0; h < 4; h += 2) {
+        float2 g[5];
+        const float2 ux = mul2(two(a.u_scale), make_float2(at(ux4, h), at(ux4, h + 1)));
+        const float2 uy = mul2(two(a.u_scale), make_float2(at(uy4, h), at(uy4, h + 1)));
+        bool fluid[2], pressure_node[2] = {false, false};
 #pragma unroll
-        for (int i = 0; i < 5; ++i) g[i] = fluid ? at(v[i], k) : 0.f;
-        const int xk = x0 + k;
-        const bool pw = open_w && bw.x == xk;
-        const bool pe = !pw && open_e && be.x == xk;
-        bool pressure_node = false;
-        const float ux = a.u_scale * at(ux4, k), uy = a.u_scale * at(uy4, k);
-        if (pw || pe) {
-            const RowBC b = pw ? bw : be;
-            const int gi = pw ? 1 : 3;
-            const int kind = (b.chan_kind >> 8) & 0xFF;
-            if (kind == 0) {  // held concentration
-                float others = 0.f;
+        for (int n = 0; n < 2; ++n) {
+            const int k = h + n;
+            fluid[n] = kAllFluid || ((lk >> (8 * k)) & 0xFFu) != kSolid;
 #pragma unroll
-                for (int i = 0; i < 5; ++i)
-                    if (i != gi) others += g[i];
-                g[gi] = b.c - others;
-            } else {          // do-nothing
-                g[gi] = own(gi, k);
-                pressure_node = kind != 3;
-                if (kind == 3) {  // the paper's inlet: scaled to C_in
-                    const float Cs = ((g[0] + g[1]) + (g[2] + g[3])) + g[4];
-                    if (Cs > 0.f) {
-                        const float gc = b.c / Cs;
-#pragma unroll
-                        for (int i = 0; i < 5; ++i) g[i] *= gc;
-                    } else {
-                        const float c1 = a.wg1 * b.c, cx = c1 * a.inv_cs2g * ux, cy = c1 * a.inv_cs2g * uy;
-                        g[0] = b.c - 4.f * c1;
-                        g[1] = c1 + cx;
-                        g[3] = c1 - cx;
-                        g[2] = c1 + cy;
-                        g[4] = c1 - cy;
-                    }
-                }
-            }
+            for (int i = 0; i < 5; ++i) at(g[i], n) = fluid[n] ? at(v[i], k) : 0.f;
+            const int xk = x0 + k;
+            const bool pw = open_w && bw.x == xk;
+            const bool pe = !pw && open_e && be.x == xk;
+            if (pw || pe) pressure_node[n] = scalar_port(g, n, pw, pw ? bw : be, at(ux, n), at(uy, n), a, own, k);
         }
-        const float C = ((g[0] + g[1]) + (g[2] + g[3])) + g[4];
-        const float wg = a.omega_g;
-        const float c1 = a.wg1 * C, cx = c1 * a.inv_cs2g * ux, cy = c1 * a.inv_cs2g * uy;
-        g[0] += wg * ((C - 4.f * c1) - g[0]);
-        g[1] += wg * ((c1 + cx) - g[1]);
-        g[3] += wg * ((c1 - cx) - g[3]);
-        g[2] += wg * ((c1 + cy) - g[2]);
-        g[4] += wg * ((c1 - cy) - g[4]);
+        // the node form's arithmetic on two nodes an instruction, its products fused
+        // into sums as the compiler fuses them there
+        const float2 C = add2(add2(add2(g[0], g[1]), add2(g[2], g[3])), g[4]);
+        const float2 c1 = mul2(two(a.wg1), C), ci = mul2(c1, two(a.inv_cs2g)), nci = mul2(c1, two(-a.inv_cs2g));
+        g[0] = fma2(wg, sub2(fma2(two(-4.f), c1, C), g[0]), g[0]);
+        g[1] = fma2(wg, sub2(fma2(ci, ux, c1), g[1]), g[1]);
+        g[3] = fma2(wg, sub2(fma2(nci, ux, c1), g[3]), g[3]);
+        g[2] = fma2(wg, sub2(fma2(ci, uy, c1), g[2]), g[2]);
+        g[4] = fma2(wg, sub2(fma2(nci, uy, c1), g[4]), g[4]);
         if (a.decay != 0.f) {  // reaction term R = -k C of Eq. cde, as w_i R
-            const float R = -a.decay * C;
-            g[0] += a.wg0 * R;
+            const float2 R = mul2(two(-a.decay), C);
+            g[0] = fma2(two(a.wg0), R, g[0]);
 #pragma unroll
-            for (int i = 1; i < 5; ++i) g[i] += a.wg1 * R;
+            for (int i = 1; i < 5; ++i) g[i] = fma2(two(a.wg1), R, g[i]);
         }
 #pragma unroll
-        for (int i = 0; i < 5; ++i) at(v[i], k) = g[i];
-        if (fluid) {
-            bad |= !(fabsf(C) < INFINITY);
-            tc += C;
-            if (pressure_node) tq += C * ux;
+        for (int n = 0; n < 2; ++n) {
+#pragma unroll
+            for (int i = 0; i < 5; ++i) at(v[i], h + n) = at(g[i], n);
+            if (!fluid[n]) continue;
+            bad |= !(fabsf(at(C, n)) < INFINITY);
+            tc += at(C, n);
+            if (pressure_node[n]) tq += at(C, n) * at(ux, n);
         }
     }
 }
@@ -489,7 +509,7 @@ __global__ void __launch_bounds__(32 * kScalarW, kScalarBlocks)
             *reinterpret_cast<float4*>(&info.u[0][4 * lane]) = ux4;
             *reinterpret_cast<float4*>(&info.u[1][4 * lane]) = uy4;
             info.links[lane] = lk;
-            if (port && lane < 2) info.bc[lane] = bc[lane];
+            if (port && lane < 2) info.bc[lane] = lane == 0 ? bc[0] : bc[1];
         }
         const bool open1 = __all_sync(kFull, lk == 0u || lk == 0xFFFFFFFFu);  // a row without walls
         if (lk != 0xFFFFFFFFu && open1) {
