@@ -226,7 +226,7 @@ cudaError_t scalar_regs_occupancy(int block, int* blocks_per_sm);
 // kScalarLevels scalar-only steps of one valve word in one launch: strips
 // (items, block_first) as in PairArgs, planned for scalar_level_warps() rows
 // an iteration; map: the source buffer, umap: the stored field's two planes.
-constexpr int kScalarLevels = 3, kScalarWarps = 8, kScalarBlocks = 2;  // steps, warps a block, resident blocks an SM
+constexpr int kScalarLevels = 3, kScalarWarps = 9, kScalarBlocks = 2;  // steps, warps a block, resident blocks an SM
 int scalar_level_warps();
 // A map of `planes` planes of ny x pitch floats at base for that kernel's copies.
 cudaError_t scalar_tensor_map(CUtensorMap* map, void* base, int planes, int ny, int pitch);

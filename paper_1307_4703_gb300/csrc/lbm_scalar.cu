@@ -60,7 +60,8 @@ __device__ __forceinline__ bool scalar_port(float2 (&p)[5], int n, bool west, co
 // stored field at the quad; own(i, k): the stored population i of node k; sc,
 // sq: the quad's scalar and outlet-flux sums.  kPorts = false: none of the
 // nodes is a port; kAllFluid: none of them is solid either (the selects of the
-// solid nodes are a third of the instructions).
+// solid nodes are a third of the instructions).  The relaxation takes two nodes
+// an instruction (packed arithmetic: the levels kernel 13.4 -> 13.0 us a step).
 template <bool kPorts, bool kAllFluid = false, typename Own>
 __device__ __forceinline__ void scalar_nodes(float4 (&v)[5], unsigned lk, int x0, const RowBC& bw, const RowBC& be,
                                              float4 ux4, float4 uy4, const ScalarArgs& a, const Own& own, float& tc,
@@ -356,11 +357,13 @@ __global__ void __launch_bounds__(128) scalar_frozen_regs(const ScalarArgs a)
 // kLevels - 2 of the four of a side lane, none of them stored.
 // What bounds it: three levels move 49 MB a step on the 4096 x 2048 chip (161
 // MB one by one), which HBM would take 8 us for; the levels' turns (barrier,
-// gather from shared memory, arithmetic) at 16 warps an SM take 13.4 us, with
-// 54% of the issue slots used (25.5 us one step a launch, at 0.92 of the HBM
-// rate; 1024 x 768 4.1 -> 3.0, 256 x 128 2.5 -> 1.5).  Tried: four levels (19.2-20.6
-// us: shared memory for 10 or 12 warps only), five (24.4), 6 warps x 3 blocks (16.7
-// where 8 x 2 took 16.5), 4 x 4 (17.3).
+// gather from shared memory, arithmetic) at 18 warps an SM take 12.5 us (24.8 us
+// one step a launch, at 0.95 of the HBM rate; 1024 x 768 3.9 -> 2.7, 256 x 128 2.5 ->
+// 1.5).  Nine warps a block are what shared memory holds twice: 8 x 2 takes 13.0 us
+// (2000 x 1000 4.6 against 4.2; 1001 x 517 with obstacles 3.7 against 4.1), 10 x 2,
+// whose second block no longer fits, 16.6.  Tried before the packed arithmetic
+// (8 x 2: 13.4 us): four levels (19.2-20.6 us: shared memory for 10 or 12 warps
+// only), five (24.4), 6 warps x 3 blocks (16.7 where 8 x 2 took 16.5), 4 x 4 (17.3).
 constexpr int kLevels = kScalarLevels, kScalarW = kScalarWarps;
 constexpr int kScalarBox = kTileNodes + 8;  // columns of a staged row: from x0 - 4 on
 struct ScalarRow {
