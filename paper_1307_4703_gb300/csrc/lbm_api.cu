@@ -1808,15 +1808,18 @@ lbm_status lbm_adjoint(lbm_handle h, const lbm_objective* obj, int64_t n, int32_
     char* ckpt = static_cast<char*>(tmp.get(size_t(n_ck) * S));
     char* seg = seg_slots > 0 ? static_cast<char*>(tmp.get(size_t(seg_slots) * S)) : nullptr;
     float* adj[3] = {static_cast<float*>(tmp.get(S)), static_cast<float*>(tmp.get(S)), static_cast<float*>(tmp.get(S))};
-    float* dn = static_cast<float*>(tmp.get(size_t(2) * h->ny * sizeof(float)));
-    double* gw = static_cast<double*>(tmp.get(size_t(agrid) * sizeof(double)));
-    double* gu = static_cast<double*>(tmp.get(size_t(2) * h->ny * sizeof(double)));
-    double* gc = static_cast<double*>(tmp.get(size_t(2) * h->ny * sizeof(double)));
-    double* dJ = static_cast<double*>(tmp.get(2 * sizeof(double)));
-    int* ox = static_cast<int*>(tmp.get(size_t(obj->n) * sizeof(int)));
-    int* oy = static_cast<int*>(tmp.get(size_t(obj->n) * sizeof(int)));
-    float* ot = static_cast<float*>(tmp.get(size_t(obj->n) * sizeof(float)));
-    float* ow = static_cast<float*>(tmp.get(size_t(obj->n) * sizeof(float)));
+    // the sums (J and dJ/dtau_c, du, dC, a slot a block, the do-nothing terms) in one
+    // buffer, cleared and read back as one; the objective's four arrays in another
+    const size_t n_read = 2 + size_t(4) * h->ny, n_sums = n_read + size_t(agrid) + size_t(h->ny);
+    double* dJ = static_cast<double*>(tmp.get(n_sums * sizeof(double)));
+    double* gu = dJ + 2;
+    double* gc = gu + size_t(2) * h->ny;
+    double* gw = dJ + n_read;
+    float* dn = reinterpret_cast<float*>(gw + agrid);
+    int* ox = static_cast<int*>(tmp.get(size_t(4) * obj->n * sizeof(int)));
+    int* oy = ox + obj->n;
+    float* ot = reinterpret_cast<float*>(oy + obj->n);
+    float* ow = ot + obj->n;
     // multi_step: the valve word of every step t0 .. t0 + n for the reverse kernel
     const bool coop = h->multi_step > 0;
     uint32_t* masks_d = coop ? static_cast<uint32_t*>(tmp.get(size_t(n + 1) * sizeof(uint32_t))) : nullptr;
@@ -1826,8 +1829,7 @@ lbm_status lbm_adjoint(lbm_handle h, const lbm_objective* obj, int64_t n, int32_
         LBM_CUDA(h, lbm::adjoint_coop_occupancy(&cps));
         coop_grid = std::max(1, std::min(agrid, std::max(1, cps) * sms));
     }
-    if (!ckpt || (seg_slots > 0 && !seg) || !adj[0] || !adj[1] || !adj[2] || !dn || !gw || !gu || !gc || !dJ ||
-        !ox || !oy || !ot || !ow || (coop && !masks_d))
+    if (!ckpt || (seg_slots > 0 && !seg) || !adj[0] || !adj[1] || !adj[2] || !dJ || !ox || (coop && !masks_d))
         return fail(h, LBM_ERR_OOM, "adjoint: device memory for %lld checkpoints and %d recomputed states not available",
                     n_ck, seg_slots);
 
@@ -1921,8 +1923,19 @@ lbm_status lbm_adjoint(lbm_handle h, const lbm_objective* obj, int64_t n, int32_
                 LBM_CUDA(h, cudaMemcpyAsync(ckpt + size_t(t / K) * S, h->pop[h->cur], S, cudaMemcpyDeviceToDevice, st));
             a.src = h->pop[h->cur];
             a.dst = h->pop[1 - h->cur];
-            a.reverse = h->order;
             a.open_mask[0] = h->mask_at(t0 + t);
+            if (h->pairs && K - t % K >= 2) {  // two steps up to the next checkpoint
+                a.reverse = h->cur;
+                uint32_t next[lbm::kMaskWords] = {h->mask_at(t0 + t + 1)};
+                cudaError_t e = launch_pair(h, a, next, h->pair_map[h->cur], st);
+                if (e != cudaSuccess) return cuda_fail(h, e, "two-step launch");
+                h->cur = 1 - h->cur;
+                join_buffers(h);
+                h->step += 2;
+                ++t;
+                continue;
+            }
+            a.reverse = h->order;
             cudaError_t e = lbm::launch_step(a, h->launch, st);
             if (e != cudaSuccess) return cuda_fail(h, e, "coupled step launch");
             swap_buffers(h);
@@ -1957,17 +1970,16 @@ lbm_status lbm_adjoint(lbm_handle h, const lbm_objective* obj, int64_t n, int32_
 
     forward_range.end();
     // J and dJ/dP(n)
-    std::vector<int> hx(obj->x, obj->x + obj->n), hy(obj->y, obj->y + obj->n);
-    LBM_CUDA(h, cudaMemcpyAsync(ox, hx.data(), hx.size() * sizeof(int), cudaMemcpyHostToDevice, st));
-    LBM_CUDA(h, cudaMemcpyAsync(oy, hy.data(), hy.size() * sizeof(int), cudaMemcpyHostToDevice, st));
-    LBM_CUDA(h, cudaMemcpyAsync(ot, obj->target, size_t(obj->n) * sizeof(float), cudaMemcpyHostToDevice, st));
-    LBM_CUDA(h, cudaMemcpyAsync(ow, obj->weight, size_t(obj->n) * sizeof(float), cudaMemcpyHostToDevice, st));
+    static_assert(sizeof(int) == sizeof(float), "the arrays are packed as words");
+    std::vector<int> words(size_t(4) * obj->n);
+    std::copy(obj->x, obj->x + obj->n, words.begin());
+    std::copy(obj->y, obj->y + obj->n, words.begin() + obj->n);
+    std::memcpy(words.data() + size_t(2) * obj->n, obj->target, size_t(obj->n) * sizeof(float));
+    std::memcpy(words.data() + size_t(3) * obj->n, obj->weight, size_t(obj->n) * sizeof(float));
+    LBM_CUDA(h, cudaMemcpyAsync(ox, words.data(), words.size() * sizeof(int), cudaMemcpyHostToDevice, st));
     // (of M(t) only what its writer stored is used: adj[1] and adj[2] need no zeros)
     LBM_CUDA(h, cudaMemsetAsync(adj[0], 0, S, st));
-    LBM_CUDA(h, cudaMemsetAsync(gw, 0, size_t(agrid) * sizeof(double), st));
-    LBM_CUDA(h, cudaMemsetAsync(gu, 0, size_t(2) * h->ny * sizeof(double), st));
-    LBM_CUDA(h, cudaMemsetAsync(gc, 0, size_t(2) * h->ny * sizeof(double), st));
-    LBM_CUDA(h, cudaMemsetAsync(dn, 0, size_t(2) * h->ny * sizeof(float), st));
+    LBM_CUDA(h, cudaMemsetAsync(dJ, 0, n_sums * sizeof(double), st));
     std::vector<uint32_t> masks_h;
     if (coop) {
         masks_h.resize(size_t(n + 1));
@@ -2083,11 +2095,12 @@ lbm_status lbm_adjoint(lbm_handle h, const lbm_objective* obj, int64_t n, int32_
         cudaError_t e = lbm::launch_sum_doubles(gw, agrid, dJ + 1, st);
         if (e != cudaSuccess) return cuda_fail(h, e, "gradient reduction launch");
     }
-    double host[2];
-    LBM_CUDA(h, cudaMemcpyAsync(host, dJ, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
-    if (dJ_du_in) LBM_CUDA(h, cudaMemcpyAsync(dJ_du_in, gu, size_t(2) * h->ny * sizeof(double), cudaMemcpyDeviceToHost, st));
-    if (dJ_dC_in) LBM_CUDA(h, cudaMemcpyAsync(dJ_dC_in, gc, size_t(2) * h->ny * sizeof(double), cudaMemcpyDeviceToHost, st));
+    std::vector<double> host(n_read);
+    LBM_CUDA(h, cudaMemcpyAsync(host.data(), dJ, n_read * sizeof(double), cudaMemcpyDeviceToHost, st));
     LBM_CUDA(h, cudaStreamSynchronize(st));
+    const auto side = host.begin() + 2, end = side + 2 * h->ny;
+    if (dJ_du_in) std::copy(side, end, dJ_du_in);
+    if (dJ_dC_in) std::copy(end, host.end(), dJ_dC_in);
     *J = host[0];
     *dJ_dtau_c = -host[1] / (h->tau_c * h->tau_c);  // d(1/tau_c)/dtau_c = -1/tau_c^2
     return read_err_word(h);
