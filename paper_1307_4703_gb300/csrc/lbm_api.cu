@@ -107,6 +107,7 @@ struct lbm_ctx {
     int* pair_first = nullptr;
     CUtensorMap pair_map[2];      // of the two state buffers
     int pair_grid = 0;            // its blocks; 0: this handle has none
+    int pair_warps = 0;           // warps of a block
     bool pairs = false;           // lbm_step takes two steps a launch
     int multi_step = 0;           // lbm_step: steps per cooperative launch (0 = one launch per step)
     int coop_grid = 0;            // blocks of that launch (all resident)
@@ -402,7 +403,7 @@ cudaError_t launch_pair(const lbm_ctx* h, const lbm::StepArgs& a, const uint32_t
     lbm::PairArgs p{a, a, h->pair_items, h->pair_first};
     std::memcpy(p.second.open_mask, words, sizeof(words));
     p.second.plane = lbm::kTileNodes;
-    return lbm::launch_step_pair(p, src_map, h->pair_grid, h->precision, h->paper_ports, s);
+    return lbm::launch_step_pair(p, src_map, h->pair_grid, h->pair_warps, h->precision, h->paper_ports, s);
 }
 
 // Whether the next two of `left` steps go as one launch.  The last step of a
@@ -1019,13 +1020,21 @@ lbm_status create_impl(lbm_handle* out, int32_t nx, int32_t ny, const uint8_t* m
     lbm::StripPlan plan;
     if (opt.variant == 0 && opt.block_threads == 0 && opt.max_blocks == 0 && opt.multi_step == 0 &&
         opt.wall_scheme == LBM_WALL_BOUNCE_BACK && h->pop[0] && h->pop[1]) {
-        int pair_per_sm = 0;
-        bool have = lbm::pair_occupancy(h->precision, h->paper_ports, &pair_per_sm) == cudaSuccess && pair_per_sm > 0;
+        lbm::PairShape shapes[2];
+        int n_shapes = 0;
+        for (int warps : {6, 4, 8}) {
+            int per_sm = 0;
+            if ((warps == 8) == (h->precision == LBM_FP32)) continue;
+            if (lbm::pair_occupancy(h->precision, h->paper_ports, warps, &per_sm) == cudaSuccess && per_sm > 0)
+                shapes[n_shapes++] = {warps, per_sm * sms, sms};
+        }
+        bool have = n_shapes > 0;
+        if (have)
+            plan = lbm::plan_pairs(h->tiles_rows, rowbc, nx, ny, pitch, h->precision, h->paper_ports, shapes, n_shapes,
+                                   (long long)h->launch.grid * (h->launch.block / 32));
         for (int b = 0; b < 2 && have; ++b)
-            have = lbm::pair_tensor_map(&h->pair_map[b], h->pop[b], ny, pitch, h->precision) == cudaSuccess;
+            have = lbm::pair_tensor_map(&h->pair_map[b], h->pop[b], ny, pitch, h->precision, plan.warps) == cudaSuccess;
         if (have) {
-            plan = lbm::plan_pairs(h->tiles_rows, rowbc, nx, ny, pitch, h->precision, h->paper_ports, lbm::pair_warps(h->precision),
-                                   pair_per_sm * sms, (long long)h->launch.grid * (h->launch.block / 32));
             h->pair_items = static_cast<int4*>(dev_alloc(h, plan.items.size() * sizeof(int4)));
             h->pair_first = static_cast<int*>(dev_alloc(h, plan.block_first.size() * sizeof(int)));
             have = h->pair_items && h->pair_first;
@@ -1034,6 +1043,7 @@ lbm_status create_impl(lbm_handle* out, int32_t nx, int32_t ny, const uint8_t* m
         }
         if (have) {
             h->pair_grid = plan.grid;
+            h->pair_warps = plan.warps;
             h->pairs = plan.worth;
         }
     }
@@ -1414,7 +1424,7 @@ lbm_status lbm_step_diagnostics(lbm_handle h, int64_t n, double* out)
     a.diag_ticket = h->err + 1;
     // Runs of steps leave their partials side by side for one reduction launch,
     // a block a step (the same order of additions as lbm_get_diagnostics, the
-    // same bits): 1024 x 768 11.9 -> 8.8 us a step against totals formed at the
+    // same bits): 1024 x 768 11.7 -> 8.5 us a step against totals formed at the
     // end of every step, which the next one waits for.  A step by itself forms
     // its totals in its last block (variants 1 and 4 with blocks of at least
     // lbm::kFoldThreads threads and halfway bounce-back), or leaves them to the
@@ -2419,7 +2429,7 @@ lbm_status lbm_autotune(lbm_handle h, int32_t trial_steps)
     if (e == cudaSuccess && best.grid > 0 && h->pair_grid > 0) {
         CUtensorMap maps[2];
         for (int b = 0; b < 2 && e == cudaSuccess; ++b)
-            e = lbm::pair_tensor_map(&maps[b], bufs[b], h->ny, h->pitch, h->precision);
+            e = lbm::pair_tensor_map(&maps[b], bufs[b], h->ny, h->pitch, h->precision, h->pair_warps);
         const int launches = (trial_steps + 1) / 2;
         int64_t k = 0;
         auto trial_pair = [&]() {

@@ -134,14 +134,14 @@ struct PairArgs {
     const int4* items;
     const int* block_first;
 };
-// rescale: the lattice has ports of the rescaling kinds
-cudaError_t pair_occupancy(int precision, bool rescale, int* per_sm);
-int pair_warps(int precision);  // of a block
+// warps of a block: 4 or 6 (FP32), 8 (16-bit storage); rescale: the lattice
+// has ports of the rescaling kinds.
+cudaError_t pair_occupancy(int precision, bool rescale, int warps, int* per_sm);
 // A tensor map of `planes` planes of ny rows of `pitch` elements of `elem`
 // bytes at base, with boxes of cols x rows of one plane.
 cudaError_t rows_tensor_map(CUtensorMap* map, void* base, int planes, int ny, int pitch, int elem, int cols, int rows);
-cudaError_t pair_tensor_map(CUtensorMap* map, void* pop, int ny, int pitch, int precision);
-cudaError_t launch_step_pair(const PairArgs& p, const CUtensorMap& map, int grid, int precision, bool rescale,
+cudaError_t pair_tensor_map(CUtensorMap* map, void* pop, int ny, int pitch, int precision, int warps);
+cudaError_t launch_step_pair(const PairArgs& p, const CUtensorMap& map, int grid, int warps, int precision, bool rescale,
                              cudaStream_t s);
 
 // One adjoint step (lbm_adjoint.cu): A(t) from A(t+1) and the state P(t).

@@ -11,10 +11,11 @@
 // each other.  The arithmetic of each node is collide_quad on values rounded
 // to the storage type, as in the single-step kernels: the same bits.
 //
-// What bounds it: neither memory (360 MB a launch on the 4096 x 2048 chip,
-// FP32) nor issue alone, but their overlap at 12 warps an SM, which shared
-// memory (FP32: a staged row and 1.3 ring rows a warp, 17.4 KB) and registers
-// allow.  So nothing in the loop waits for global memory:
+// What bounds it: memory first (385 MB a launch on the 4096 x 2048 chip, FP32,
+// which HBM takes 57 us for, against 71), then the barriers' and shared memory's
+// turns at 12 warps an SM, which shared memory (FP32: a staged row and 1.3 to 1.5
+// ring rows a warp) and registers allow; 40% of the issue slots are used, 57% in
+// 16-bit storage at 16 warps.  So nothing in the loop waits for global memory:
 //   - the rows the W warps pull from come as 14 tensor copies a block and
 //     iteration (one box of W rows a plane, each at the plane's own row
 //     offset), shared between the warps and asked for as soon as every warp
@@ -26,14 +27,15 @@
 //   - a strip along a side wall names the two lanes at it, and these bounce
 //     back from the staged rows (from global memory, such strips took 1.5
 //     times as long as the others and set the launch's length).
-// Steps of the 4096 x 2048 chip, us: FP32 59.5 one by one, 38.0 here; FP16
-// 36.2 -> 28.1; 64 chips in a batch 111 -> 77.0 (FP32).  Tried: the second
-// step's rows written by bulk copies from shared memory (50.4 against 46.7
-// us at that stage: 14 copies a row by one warp are slow to issue); rows
-// copied lane by lane (cp.async: FP32 the same, FP16 34.7 against 30.5 us);
-// 4 warps x 3 blocks for FP32 (the large chip the same, 2000 x 1000 12.2
-// against 11.4 us), 4 x 4 for 16-bit (30.5 against 29.9 us; 1024 x 768 6.9
-// against 5.6 us); 12 x 1 (59 us).
+// Steps of the 4096 x 2048 chip, us: FP32 59.5 one by one, 35.5 here; FP16
+// 36.2 -> 28.1; 64 chips in a batch 111 -> 74.7 (FP32).  FP32 blocks are of 6
+// warps (2 an SM) or 4 (3 an SM), whichever the strips of a lattice suit
+// (plan_pairs).  Tried: the second step's rows written by bulk copies from
+// shared memory (50.4 against 46.7 us at that stage: 14 copies a row by one warp
+// are slow to issue); rows copied lane by lane (cp.async: FP32 the same, FP16
+// 34.7 against 30.5 us); 5 x 2 (40.1 where 6 x 2 took 38.0) and 12 x 1 (59 us) for
+// FP32; 4 x 4 (30.5 against 29.9 us), 9 x 2 and 10 x 2 (43 and 45: 96 registers
+// spill) for 16-bit.
 #include <algorithm>
 
 #include <cudaTypedefs.h>
@@ -43,9 +45,8 @@
 namespace lbm {
 namespace {
 
-template <typename T>
-constexpr int kPairWarps = sizeof(T) == 4 ? 6 : 8;
-constexpr int kPairBlocks = 2;  // resident blocks per SM
+// Resident blocks per SM of W warps: what shared memory and registers allow.
+constexpr int pair_blocks(int W) { return W == 4 ? 3 : 2; }
 template <typename T>
 constexpr int kBoxCols = sizeof(T) == 4 ? 136 : 144;  // columns of a staged row: the strip's 128, a halo of at least one
                                                       // on each side, from a 16-byte boundary on
@@ -69,9 +70,8 @@ struct alignas(16) RowStage {
     float2 rates;                    // the row's relaxation rates (batches)
     float2 pad;
 };
-template <typename T>
+template <typename T, int W>
 struct alignas(128) PairSmem {
-    static constexpr int W = kPairWarps<T>;
     struct alignas(128) Box {
         T row[W][kBoxCols<T>];
     } box[kPlanes];    // the W rows each plane is pulled from
@@ -81,10 +81,10 @@ struct alignas(128) PairSmem {
     uint64_t done;     // the iteration's first-step rows are in the ring
     uint64_t read;     // the iteration's second steps have read the ring
 };
-template <typename T>
+template <typename T, int W>
 constexpr bool smem_aligned()
 {
-    using S = PairSmem<T>;
+    using S = PairSmem<T, W>;
     using R = RingRow<T>;
     using G = RowStage<T>;
     return offsetof(S, box) % 128 == 0 && sizeof(typename S::Box) % 128 == 0 && offsetof(S, stage) % 16 == 0 &&
@@ -93,8 +93,9 @@ constexpr bool smem_aligned()
            offsetof(R, rates) % 8 == 0 && sizeof(R) % 16 == 0 && offsetof(G, bc) % 16 == 0 &&
            offsetof(G, side) % 16 == 0 && offsetof(G, rates) % 8 == 0 && sizeof(G) % 16 == 0;
 }
-static_assert(smem_aligned<float>() && smem_aligned<__half>(), "targets of vector accesses, copies and barriers");
-static_assert(sizeof(PairSmem<__half>) == sizeof(PairSmem<__nv_bfloat16>), "one 16-bit layout");
+static_assert(smem_aligned<float, 4>() && smem_aligned<float, 6>() && smem_aligned<__half, 8>(),
+              "targets of vector accesses, copies and barriers");
+static_assert(sizeof(PairSmem<__half, 8>) == sizeof(PairSmem<__nv_bfloat16, 8>), "one 16-bit layout");
 
 // Column of x0 in a staged row (x0 is a multiple of 4).
 template <typename T>
@@ -126,8 +127,8 @@ struct PairStrip {
 
 // The lane's quads of the 14 planes at the pull sources, from row r of the
 // boxes.
-template <typename T>
-__device__ __forceinline__ void pull_staged(float4 (&v)[kPlanes], const PairSmem<T>& sm, int r, int offset, int lane)
+template <typename T, int W>
+__device__ __forceinline__ void pull_staged(float4 (&v)[kPlanes], const PairSmem<T, W>& sm, int r, int offset, int lane)
 {
 #pragma unroll
     for (int p = 0; p < kPlanes; ++p) {
@@ -236,8 +237,9 @@ __device__ __forceinline__ void bounce_groups(float4 (&v)[kPlanes], unsigned lk,
 // Bounce-back at walls to the west and east for a strip's side lane, from its
 // warp's row of the boxes (r; c: the lane's first column in it), which holds
 // the populations along the row, and its stage, which holds the diagonal ones.
-template <typename T>
-__device__ __forceinline__ void bounce_side(float4 (&v)[kPlanes], unsigned lk, const RowStage<T>& st, const PairSmem<T>& sm, int r, int c, int n)
+template <typename T, int W>
+__device__ __forceinline__ void bounce_side(float4 (&v)[kPlanes], unsigned lk, const RowStage<T>& st, const PairSmem<T, W>& sm, int r,
+                                            int c, int n)
 {
     const float4 f1 = Codec<T>::lds4(&sm.box[1].row[r][c], 0.f), f3 = Codec<T>::lds4(&sm.box[3].row[r][c], 0.f);
     const float4 g1 = Codec<T>::lds4(&sm.box[10].row[r][c], 0.f), g3 = Codec<T>::lds4(&sm.box[12].row[r][c], 0.f);
@@ -278,13 +280,13 @@ __device__ __forceinline__ void collide_row(const StepArgs& a, float4 (&v)[kPlan
     bad |= q.bad;
 }
 
-template <typename T, bool kRescale>
-__global__ void __launch_bounds__(32 * kPairWarps<T>, kPairBlocks)
+template <typename T, bool kRescale, int W>
+__global__ void __launch_bounds__(32 * W, pair_blocks(W))
     coupled_step_pair(const PairArgs p, const __grid_constant__ CUtensorMap map)
 {
-    constexpr int W = kPairWarps<T>, R = W + 2;
+    constexpr int R = W + 2;
     extern __shared__ __align__(128) unsigned char pair_smem[];
-    PairSmem<T>& sm = *reinterpret_cast<PairSmem<T>*>(pair_smem);
+    PairSmem<T, W>& sm = *reinterpret_cast<PairSmem<T, W>*>(pair_smem);
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int reverse = p.first.reverse, pitch = p.first.pitch, ny = p.first.ny;
@@ -466,44 +468,69 @@ __global__ void __launch_bounds__(32 * kPairWarps<T>, kPairBlocks)
     if (__any_sync(kFull, bad) && lane == 0) atomicOr(p.first.err, 1u);
 }
 
-template <typename T, bool kRescale>
+template <typename T, bool kRescale, int W>
 cudaError_t launch(const PairArgs& p, const CUtensorMap& map, int grid, cudaStream_t s)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(32 * kPairWarps<T>);
-    cfg.dynamicSmemBytes = sizeof(PairSmem<T>);
+    cfg.blockDim = dim3(32 * W);
+    cfg.dynamicSmemBytes = sizeof(PairSmem<T, W>);
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, coupled_step_pair<T, kRescale>, p, map);
+    return cudaLaunchKernelEx(&cfg, coupled_step_pair<T, kRescale, W>, p, map);
 }
 
-template <typename T, bool kRescale>
+template <typename T, bool kRescale, int W>
 cudaError_t occupancy(int* per_sm)
 {
-    cudaError_t e = cudaFuncSetAttribute(coupled_step_pair<T, kRescale>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         int(sizeof(PairSmem<T>)));
+    cudaError_t e = cudaFuncSetAttribute(coupled_step_pair<T, kRescale, W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         int(sizeof(PairSmem<T, W>)));
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, coupled_step_pair<T, kRescale>, 32 * kPairWarps<T>,
-                                                          sizeof(PairSmem<T>));
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, coupled_step_pair<T, kRescale, W>, 32 * W,
+                                                          sizeof(PairSmem<T, W>));
     return e;
 }
 
+// f.template operator()<T, kRescale, W>() of the instance that a launch takes.
+template <typename F>
+cudaError_t instance(int precision, bool rescale, int warps, const F& f)
+{
+    if (precision == kFP16) return rescale ? f.template operator()<__half, true, 8>() : f.template operator()<__half, false, 8>();
+    if (precision == kBF16)
+        return rescale ? f.template operator()<__nv_bfloat16, true, 8>() : f.template operator()<__nv_bfloat16, false, 8>();
+    if (warps == 4) return rescale ? f.template operator()<float, true, 4>() : f.template operator()<float, false, 4>();
+    return rescale ? f.template operator()<float, true, 6>() : f.template operator()<float, false, 6>();
+}
+struct Occupancy {
+    int* per_sm;
+    template <typename T, bool kRescale, int W>
+    cudaError_t operator()() const
+    {
+        return occupancy<T, kRescale, W>(per_sm);
+    }
+};
+struct Launch {
+    const PairArgs& p;
+    const CUtensorMap& map;
+    int grid;
+    cudaStream_t s;
+    template <typename T, bool kRescale, int W>
+    cudaError_t operator()() const
+    {
+        return launch<T, kRescale, W>(p, map, grid, s);
+    }
+};
+
 }  // namespace
 
-cudaError_t pair_occupancy(int precision, bool rescale, int* per_sm)
+cudaError_t pair_occupancy(int precision, bool rescale, int warps, int* per_sm)
 {
-    if (precision == kFP16) return rescale ? occupancy<__half, true>(per_sm) : occupancy<__half, false>(per_sm);
-    if (precision == kBF16)
-        return rescale ? occupancy<__nv_bfloat16, true>(per_sm) : occupancy<__nv_bfloat16, false>(per_sm);
-    return rescale ? occupancy<float, true>(per_sm) : occupancy<float, false>(per_sm);
+    return instance(precision, rescale, warps, Occupancy{per_sm});
 }
-
-int pair_warps(int precision) { return precision == kFP32 ? kPairWarps<float> : kPairWarps<__half>; }
 
 cudaError_t rows_tensor_map(CUtensorMap* map, void* base, int planes, int ny, int pitch, int elem, int cols, int rows)
 {
@@ -527,26 +554,16 @@ cudaError_t rows_tensor_map(CUtensorMap* map, void* base, int planes, int ny, in
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-cudaError_t pair_tensor_map(CUtensorMap* map, void* pop, int ny, int pitch, int precision)
+cudaError_t pair_tensor_map(CUtensorMap* map, void* pop, int ny, int pitch, int precision, int warps)
 {
     const bool f32 = precision == kFP32;
-    return rows_tensor_map(map, pop, kPlanes, ny, pitch, f32 ? 4 : 2, f32 ? kBoxCols<float> : kBoxCols<__half>,
-                           pair_warps(precision));
+    return rows_tensor_map(map, pop, kPlanes, ny, pitch, f32 ? 4 : 2, f32 ? kBoxCols<float> : kBoxCols<__half>, warps);
 }
 
-template <bool kRescale>
-static cudaError_t launch_precision(const PairArgs& p, const CUtensorMap& map, int grid, int precision, cudaStream_t s)
-{
-    return precision == kFP16   ? launch<__half, kRescale>(p, map, grid, s)
-           : precision == kBF16 ? launch<__nv_bfloat16, kRescale>(p, map, grid, s)
-                                : launch<float, kRescale>(p, map, grid, s);
-}
-
-cudaError_t launch_step_pair(const PairArgs& p, const CUtensorMap& map, int grid, int precision, bool rescale,
+cudaError_t launch_step_pair(const PairArgs& p, const CUtensorMap& map, int grid, int warps, int precision, bool rescale,
                              cudaStream_t s)
 {
-    const cudaError_t e = rescale ? launch_precision<true>(p, map, grid, precision, s)
-                                  : launch_precision<false>(p, map, grid, precision, s);
+    const cudaError_t e = instance(precision, rescale, warps, Launch{p, map, grid, s});
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }

@@ -273,6 +273,7 @@ StripPlan plan(const std::vector<Run>& runs, const int (&costs)[5], int halo, in
     while (split(runs, costs, halo, warps, m, nullptr) > resident) m += std::max(1, m / 64);
     split(runs, costs, halo, warps, m, &out);
     out.grid = int(out.block_first.size()) - 1;
+    out.longest = m;
     // the work of the launch in plain rows of 128 nodes, blocks that end early included
     out.work = double(out.grid) * warps * m / costs[kPlain];
     return out;
@@ -286,9 +287,32 @@ std::vector<Run> runs_of(const std::vector<uint2>& tiles, const std::vector<RowB
 }  // namespace
 
 StripPlan plan_pairs(const std::vector<uint2>& tiles, const std::vector<RowBC>& bc, int nx, int ny, int pitch,
-                     int precision, bool rescale, int warps, int resident, long long single_warps)
+                     int precision, bool rescale, const PairShape* shapes, int n_shapes, long long single_warps)
 {
-    StripPlan p = plan(runs_of(tiles, bc, nx, ny, pitch, 1), rescale ? kPairRescaleCost : kPairCost, 1, warps, resident);
+    // The block shape, where there is a choice (FP32: 2 blocks of 6 warps an SM or 3
+    // of 4): the one whose longest block is over first, an iteration of 4 warps taking
+    // 0.96 of one of 6 on a full SM.  us a step, 6 / 4 warps: equal lengths 4096 x 2048
+    // 38.0 / 35.5, 64 chips 77.0 / 74.7, 1300 x 800 6.9 / 6.6; 99 to 112 (1001 x 517 with
+    // obstacles) 9.4 / 10.9, 44 to 48 (1024 x 768) 5.4 / 6.1.  A block that has an SM to
+    // itself is faster still (400 x 300, 136 / 271 blocks: 2.64 / 3.08; 256 x 128, 54 /
+    // 101 blocks: 2.57 / 2.50).
+    const std::vector<Run> runs = runs_of(tiles, bc, nx, ny, pitch, 1);
+    StripPlan p;
+    int resident = 0;
+    bool alone = false;  // every block of p has an SM to itself
+    double best = 0.;
+    for (int k = 0; k < n_shapes; ++k) {
+        const PairShape& s = shapes[k];
+        StripPlan q = plan(runs, rescale ? kPairRescaleCost : kPairCost, 1, s.warps, s.resident);
+        q.warps = s.warps;
+        const double time = q.longest * (s.warps == 4 ? 0.96 : 1.);
+        const bool spread = q.grid <= s.sms;
+        if (k > 0 && (alone != spread ? alone : time >= best)) continue;
+        best = time;
+        alone = spread;
+        resident = s.resident;
+        p = std::move(q);
+    }
     // Where two single steps are the better choice, in us a step, single / two-step
     // launches: where obstacles break the rows into strips that do far more than
     // the tiles' work.  FP32 at 1.7 and 1.8 of it 22.2 / 25.4 and 47.7 / 50.5, at 1.5 a

@@ -12,15 +12,22 @@ struct StripPlan {
     std::vector<int4> items;       // strips (PairArgs::items)
     std::vector<int> block_first;  // grid + 1 entries
     int grid = 0;
+    int warps = 0;                 // of a block (plan_pairs)
+    int longest = 0;               // cost of the block that takes longest
     double work = 0;
     bool worth = false;            // faster than single steps
 };
 
+// A block shape of the two-step kernel, how many of its blocks are resident at
+// once and on how many SMs.
+struct PairShape {
+    int warps, resident, sms;
+};
 // tiles: the lattice's 128-node tiles in row order; bc: 2 ny port entries;
-// rescale: it has ports of the rescaling kinds; warps: of a block; resident:
-// blocks in one wave; single_warps: of the single step's grid.
+// rescale: it has ports of the rescaling kinds; single_warps: of the single
+// step's grid; warps, resident: of a block, blocks in one wave.
 StripPlan plan_pairs(const std::vector<uint2>& tiles, const std::vector<RowBC>& bc, int nx, int ny, int pitch,
-                     int precision, bool rescale, int warps, int resident, long long single_warps);
+                     int precision, bool rescale, const PairShape* shapes, int n_shapes, long long single_warps);
 StripPlan plan_scalar(const std::vector<uint2>& tiles, const std::vector<RowBC>& bc, int nx, int ny, int pitch, int levels,
                       int warps, int resident);
 
