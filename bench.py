@@ -3,7 +3,9 @@
 A "step" is one coupled time step of the whole chip: pull-stream of f and g,
 bounce-back walls, valve-switched Zou-He ports, moments, collision of f and
 of g with the same step's velocity, and the fused FP64 mass/flux
-diagnostics; one launch of the fused kernel.  The workload is the
+diagnostics; one call of lbm_step(1), one launch of the fused kernel.  The
+line's `run_of_steps` gives the same steps as one call, which takes two of
+them a launch with diagnostics of the last alone.  The workload is the
 4096 x 2048 two-channel chip (3.35 M fluid nodes, 0.94 GB of FP32
 populations per copy, larger than the 129 MB L2), the configuration the HBM
 roofline is quoted on.
@@ -314,6 +316,24 @@ def _adjoint_ratio(device):
             "multi_step_1000": {"ckpt_every_250": out[(1000, 250)], "ckpt_every_1": out[(1000, 1)]}}
 
 
+def _run_of_steps(chip, fluid, steps, stream):
+    """`steps` more steps of the timed chip as one lbm_step call: two steps a
+    launch where the library finds that faster, the state between them never
+    in memory, diagnostics formed by the last step alone."""
+    import torch
+    chip.step(min(steps, 200))
+    chip.synchronize()
+    e0 = torch.cuda.Event(enable_timing=True)
+    e1 = torch.cuda.Event(enable_timing=True)
+    e0.record(stream)
+    chip.step(steps)
+    e1.record(stream)
+    stream.synchronize()
+    ms = e0.elapsed_time(e1)
+    chip.diagnostics()  # raises on a numeric error flag
+    return {"value": fluid * steps / ms / 1e6, "unit": UNIT, "steps": steps, "ms_per_step": ms / max(steps, 1)}
+
+
 def _frozen_scalar(chip, prob, steps, stream, peak):
     """The scalar-only step on stored velocity fields (the paper's own
     workflow): 48 bytes per fluid node and step (5 populations read and
@@ -466,11 +486,12 @@ def _batch(steps, stream, device, peak, n_chips=64):
 
 def _small_chips(steps, stream, device, peak):
     """Chips of a few microseconds per step, where launch costs show: the
-    1024 x 768 chip (the paper's 1 um lattice, 313,600 fluid nodes) with
-    single-step launches, replayed CUDA graphs of 100 steps (both after
+    1024 x 768 chip (the paper's 1 um lattice, 313,600 fluid nodes) as one
+    lbm_step call, replayed CUDA graphs of 100 steps (both after
     lbm_autotune) and runs of up to 1000 steps in one cooperative launch
-    (multi_step); the 1024 x 512 chip (two buffers in L2) with single-step
-    launches and multi_step runs."""
+    (multi_step); the 1024 x 512 chip (two buffers in L2) as one lbm_step
+    call and multi_step runs.  roofline_frac counts 112 bytes per node and
+    step; launches of two steps move about half of them."""
     import torch
     from paper_1307_4703_gb300 import lbm, workloads as W
     out = {}
@@ -589,7 +610,7 @@ def _profile_target(args, device):
         e1.record(stream)
         stream.synchronize()
         us = e0.elapsed_time(e1) * 1e3 / max(args.steps, 1)
-        out = {"kernel": "lbm_scalar_step (default kernel: scalar_frozen_regs)", "workload": prob["name"],
+        out = {"kernel": "lbm_scalar_step(1): scalar_frozen_regs", "workload": prob["name"],
                "us_per_step": us,
                "glups": W.fluid_count(prob) / us / 1e3}
     else:
@@ -674,6 +695,7 @@ def main():
         reference = None
         if ws == 1 and rank == 0:
             extras["cpu_baseline"], reference = _cpu_baseline(args.cpu_seconds)
+        extras["run_of_steps"] = _run_of_steps(chip, fluid, args.steps, stream)
         extras["frozen_scalar_step"] = _frozen_scalar(chip, prob, min(args.steps, 2000), stream, peak)
         extras["reduced_precision_storage"] = _reduced_precision(prob, min(args.steps, 5000), stream, local, peak,
                                                                  reference)
