@@ -1022,9 +1022,9 @@ lbm_status create_impl(lbm_handle* out, int32_t nx, int32_t ny, const uint8_t* m
         opt.wall_scheme == LBM_WALL_BOUNCE_BACK && h->pop[0] && h->pop[1]) {
         lbm::PairShape shapes[2];
         int n_shapes = 0;
-        for (int warps : {6, 4, 8}) {
+        for (int k = 0; k < 2; ++k) {
+            const int warps = h->precision == LBM_FP32 ? 6 - 2 * k : 8 - 2 * k;
             int per_sm = 0;
-            if ((warps == 8) == (h->precision == LBM_FP32)) continue;
             if (lbm::pair_occupancy(h->precision, h->paper_ports, warps, &per_sm) == cudaSuccess && per_sm > 0)
                 shapes[n_shapes++] = {warps, per_sm * sms, sms};
         }

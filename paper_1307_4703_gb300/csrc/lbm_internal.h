@@ -134,7 +134,7 @@ struct PairArgs {
     const int4* items;
     const int* block_first;
 };
-// warps of a block: 4 or 6 (FP32), 8 (16-bit storage); rescale: the lattice
+// warps of a block: 4 or 6 (FP32), 6 or 8 (16-bit storage); rescale: the lattice
 // has ports of the rescaling kinds.
 cudaError_t pair_occupancy(int precision, bool rescale, int warps, int* per_sm);
 // A tensor map of `planes` planes of ny rows of `pitch` elements of `elem`

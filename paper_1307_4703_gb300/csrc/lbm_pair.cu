@@ -29,13 +29,13 @@
 //     times as long as the others and set the launch's length).
 // Steps of the 4096 x 2048 chip, us: FP32 59.5 one by one, 35.5 here; FP16
 // 36.2 -> 28.1; 64 chips in a batch 111 -> 74.7 (FP32).  FP32 blocks are of 6
-// warps (2 an SM) or 4 (3 an SM), whichever the strips of a lattice suit
-// (plan_pairs).  Tried: the second step's rows written by bulk copies from
+// warps (2 an SM) or 4 (3 an SM), 16-bit blocks of 8 or 6 (2 an SM), whichever the
+// strips of a lattice suit (plan_pairs).  Tried: the second step's rows written by bulk copies from
 // shared memory (50.4 against 46.7 us at that stage: 14 copies a row by one warp
 // are slow to issue); rows copied lane by lane (cp.async: FP32 the same, FP16
 // 34.7 against 30.5 us); 5 x 2 (40.1 where 6 x 2 took 38.0) and 12 x 1 (59 us) for
-// FP32; 4 x 4 (30.5 against 29.9 us), 9 x 2 and 10 x 2 (43 and 45: 96 registers
-// spill) for 16-bit.
+// FP32; 4 x 4 (27.9 against 28.1 us, 1024 x 768 5.6 against 4.9), 5 x 3 (29.6), 7 x 2
+// (30.8), 9 x 2 and 10 x 2 (43 and 45: 96 registers spill) for 16-bit.
 #include <algorithm>
 
 #include <cudaTypedefs.h>
@@ -93,9 +93,12 @@ constexpr bool smem_aligned()
            offsetof(R, rates) % 8 == 0 && sizeof(R) % 16 == 0 && offsetof(G, bc) % 16 == 0 &&
            offsetof(G, side) % 16 == 0 && offsetof(G, rates) % 8 == 0 && sizeof(G) % 16 == 0;
 }
-static_assert(smem_aligned<float, 4>() && smem_aligned<float, 6>() && smem_aligned<__half, 8>(),
+static_assert(smem_aligned<float, 4>() && smem_aligned<float, 6>() && smem_aligned<__half, 6>() &&
+                  smem_aligned<__half, 8>(),
               "targets of vector accesses, copies and barriers");
-static_assert(sizeof(PairSmem<__half, 8>) == sizeof(PairSmem<__nv_bfloat16, 8>), "one 16-bit layout");
+static_assert(sizeof(PairSmem<__half, 6>) == sizeof(PairSmem<__nv_bfloat16, 6>) &&
+                  sizeof(PairSmem<__half, 8>) == sizeof(PairSmem<__nv_bfloat16, 8>),
+              "one 16-bit layout");
 
 // Column of x0 in a staged row (x0 is a multiple of 4).
 template <typename T>
@@ -496,14 +499,18 @@ cudaError_t occupancy(int* per_sm)
 }
 
 // f.template operator()<T, kRescale, W>() of the instance that a launch takes.
+template <typename T, int kFew, int kMany, typename F>
+cudaError_t instance_of(bool rescale, int warps, const F& f)
+{
+    if (warps == kFew) return rescale ? f.template operator()<T, true, kFew>() : f.template operator()<T, false, kFew>();
+    return rescale ? f.template operator()<T, true, kMany>() : f.template operator()<T, false, kMany>();
+}
 template <typename F>
 cudaError_t instance(int precision, bool rescale, int warps, const F& f)
 {
-    if (precision == kFP16) return rescale ? f.template operator()<__half, true, 8>() : f.template operator()<__half, false, 8>();
-    if (precision == kBF16)
-        return rescale ? f.template operator()<__nv_bfloat16, true, 8>() : f.template operator()<__nv_bfloat16, false, 8>();
-    if (warps == 4) return rescale ? f.template operator()<float, true, 4>() : f.template operator()<float, false, 4>();
-    return rescale ? f.template operator()<float, true, 6>() : f.template operator()<float, false, 6>();
+    if (precision == kFP16) return instance_of<__half, 6, 8>(rescale, warps, f);
+    if (precision == kBF16) return instance_of<__nv_bfloat16, 6, 8>(rescale, warps, f);
+    return instance_of<float, 4, 6>(rescale, warps, f);
 }
 struct Occupancy {
     int* per_sm;

@@ -289,13 +289,16 @@ std::vector<Run> runs_of(const std::vector<uint2>& tiles, const std::vector<RowB
 StripPlan plan_pairs(const std::vector<uint2>& tiles, const std::vector<RowBC>& bc, int nx, int ny, int pitch,
                      int precision, bool rescale, const PairShape* shapes, int n_shapes, long long single_warps)
 {
-    // The block shape, where there is a choice (FP32: 2 blocks of 6 warps an SM or 3
-    // of 4): the one whose longest block is over first, an iteration of 4 warps taking
-    // 0.96 of one of 6 on a full SM.  us a step, 6 / 4 warps: equal lengths 4096 x 2048
-    // 38.0 / 35.5, 64 chips 77.0 / 74.7, 1300 x 800 6.9 / 6.6; 99 to 112 (1001 x 517 with
-    // obstacles) 9.4 / 10.9, 44 to 48 (1024 x 768) 5.4 / 6.1.  A block that has an SM to
-    // itself is faster still (400 x 300, 136 / 271 blocks: 2.64 / 3.08; 256 x 128, 54 /
-    // 101 blocks: 2.57 / 2.50).
+    // The block shape: the one whose longest block is over first.  FP32, 2 blocks of 6
+    // warps an SM or 3 of 4: an iteration of 4 warps takes 0.96 of one of 6 on a full
+    // SM.  us a step, 6 / 4 warps: equal lengths 4096 x 2048 38.0 / 35.5, 64 chips 77.0 /
+    // 74.7, 1300 x 800 6.9 / 6.6; 99 to 112 (1001 x 517 with obstacles) 9.4 / 10.9, 44 to
+    // 48 (1024 x 768) 5.4 / 6.1.  16-bit, 2 blocks of 8 or of 6: 0.75 to 0.80 of the time.
+    // 8 / 6 warps: 36 to 44 (1024 x 768) 5.16 / 4.86, 32 to 36 (1024 x 512) 4.92 / 4.13, 64
+    // to 80 (2000 x 1000) 9.07 / 8.66, 208 to 273 (4096 x 2048) 28.1 / 28.7, 452 to 585
+    // (64 chips) 60.9 / 63.1.  A block that has an SM to itself is faster still (FP32 400
+    // x 300, 136 / 271 blocks: 2.64 / 3.08; 256 x 128, 54 / 101 blocks: 2.57 / 2.50).
+    const bool f32 = precision == kFP32;
     const std::vector<Run> runs = runs_of(tiles, bc, nx, ny, pitch, 1);
     StripPlan p;
     int resident = 0;
@@ -305,7 +308,7 @@ StripPlan plan_pairs(const std::vector<uint2>& tiles, const std::vector<RowBC>& 
         const PairShape& s = shapes[k];
         StripPlan q = plan(runs, rescale ? kPairRescaleCost : kPairCost, 1, s.warps, s.resident);
         q.warps = s.warps;
-        const double time = q.longest * (s.warps == 4 ? 0.96 : 1.);
+        const double time = q.longest * (k == 0 ? 1. : f32 ? 0.96 : 0.78);
         const bool spread = q.grid <= s.sms;
         if (k > 0 && (alone != spread ? alone : time >= best)) continue;
         best = time;
@@ -327,8 +330,8 @@ StripPlan plan_pairs(const std::vector<uint2>& tiles, const std::vector<RowBC>& 
     // idle are always the shorter way.
     const bool idle = 2 * p.grid <= resident;
     const double work = p.work / (2.0 * double(tiles.size()));
-    const bool few = rescale && precision == kFP32 && (long long)tiles.size() <= 2 * single_warps;
-    p.worth = idle || (!few && work < (precision == kFP32 ? 1.5 : 1.8));
+    const bool few = rescale && f32 && (long long)tiles.size() <= 2 * single_warps;
+    p.worth = idle || (!few && work < (f32 ? 1.5 : 1.8));
     return p;
 }
 

@@ -24,7 +24,8 @@ struct PairShape {
     int warps, resident, sms;
 };
 // tiles: the lattice's 128-node tiles in row order; bc: 2 ny port entries;
-// rescale: it has ports of the rescaling kinds; single_warps: of the single
+// rescale: it has ports of the rescaling kinds; shapes: the usual one first, then
+// the one of fewer warps; single_warps: of the single
 // step's grid; warps, resident: of a block, blocks in one wave.
 StripPlan plan_pairs(const std::vector<uint2>& tiles, const std::vector<RowBC>& bc, int nx, int ny, int pitch,
                      int precision, bool rescale, const PairShape* shapes, int n_shapes, long long single_warps);
