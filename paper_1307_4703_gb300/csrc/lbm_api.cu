@@ -2130,7 +2130,10 @@ float* field_slot(lbm_ctx* h, uint32_t word)
 // handle that cannot have them steps one launch at a time.
 void plan_scalar_levels(lbm_ctx* h)
 {
-    if (!h->scalar_levels) return;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (!h->scalar_levels || cudaStreamIsCapturing(h->stream, &capture) != cudaSuccess ||
+        capture != cudaStreamCaptureStatusNone)
+        return;  // a call being captured may not wait for the stream: the next one plans
     h->scalar_levels = false;  // once
     int per_sm = 0;
     CUtensorMap probe;

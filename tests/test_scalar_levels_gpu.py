@@ -70,3 +70,27 @@ def test_two_channel_chips(nx, ny):
     _same(*chips)
     for c in chips:
         c.close()
+
+
+def test_store_velocity_under_capture():
+    """A velocity field stored by a captured call (which may not wait for the stream, so
+    the strips are not planned there): the scalar steps after its replay are those of a
+    field stored directly."""
+    s = torch.cuda.Stream()
+    chips = [lbm.Chip.from_problem(W.config_small(), stream=s, torch_alloc=True) for _ in range(2)]
+    for c in chips:
+        c.set_valves(1)
+        c.step(5)
+        c.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s):
+        chips[0].store_velocity(1)
+    graph.replay()
+    torch.cuda.synchronize()
+    chips[1].store_velocity(1)
+    for c in chips:
+        c.scalar_step(7)
+    for a, b in zip(chips[0].populations(), chips[1].populations()):
+        assert np.array_equal(a, b)
+    for c in chips:
+        c.close()
