@@ -311,7 +311,7 @@ def _adjoint_ratio(device):
     torch.cuda.empty_cache()
     return {"value": out[(0, 250)]["whole_call"], "workload": "chip-1024x512, 4000 steps, checkpoints every 250",
             "definition": "whole lbm_adjoint call (forward sweep + recomputation + reverse sweep) / forward run "
-                          "of the same steps; one launch per step",
+                          "of the same steps (one lbm_step call)",
             "ckpt_every_250": out[(0, 250)], "ckpt_every_1": out[(0, 1)],
             "multi_step_1000": {"ckpt_every_250": out[(1000, 250)], "ckpt_every_1": out[(1000, 1)]}}
 

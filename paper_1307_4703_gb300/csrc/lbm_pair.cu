@@ -11,10 +11,10 @@
 // each other.  The arithmetic of each node is collide_quad on values rounded
 // to the storage type, as in the single-step kernels: the same bits.
 //
-// What bounds it: memory first (385 MB a launch on the 4096 x 2048 chip, FP32,
-// which HBM takes 57 us for, against 71), then the barriers' and shared memory's
+// What bounds it: memory first (363 MB a launch on the 4096 x 2048 chip, FP32,
+// which HBM takes 54 us for, against 71), then the barriers' and shared memory's
 // turns at 12 warps an SM, which shared memory (FP32: a staged row and 1.3 to 1.5
-// ring rows a warp) and registers allow; 40% of the issue slots are used, 57% in
+// ring rows a warp) and registers allow; 42% of the issue slots are used, 55% in
 // 16-bit storage at 16 warps.  So nothing in the loop waits for global memory:
 //   - the rows the W warps pull from come as 14 tensor copies a block and
 //     iteration (one box of W rows a plane, each at the plane's own row
