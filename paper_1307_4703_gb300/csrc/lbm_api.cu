@@ -108,6 +108,7 @@ struct lbm_ctx {
     CUtensorMap pair_map[2];      // of the two state buffers
     int pair_grid = 0;            // its blocks; 0: this handle has none
     int pair_warps = 0;           // warps of a block
+    bool pairs_keep = false;      // two-step launches that store the state between the steps are used
     bool pairs = false;           // lbm_step takes two steps a launch
     int multi_step = 0;           // lbm_step: steps per cooperative launch (0 = one launch per step)
     int coop_grid = 0;            // blocks of that launch (all resident)
@@ -396,11 +397,12 @@ void swap_buffers(lbm_ctx* h)
 }
 
 // Two steps in one launch: a holds the first one's arguments (src, dst and
-// reverse among them), words the valve words of the second.
+// reverse among them), words the valve words of the second; mid: where the
+// state between them is stored, or null.
 cudaError_t launch_pair(const lbm_ctx* h, const lbm::StepArgs& a, const uint32_t (&words)[lbm::kMaskWords],
-                        const CUtensorMap& src_map, cudaStream_t s)
+                        const CUtensorMap& src_map, cudaStream_t s, void* mid = nullptr)
 {
-    lbm::PairArgs p{a, a, h->pair_items, h->pair_first};
+    lbm::PairArgs p{a, a, h->pair_items, h->pair_first, mid};
     std::memcpy(p.second.open_mask, words, sizeof(words));
     p.second.plane = lbm::kTileNodes;
     return lbm::launch_step_pair(p, src_map, h->pair_grid, h->pair_warps, h->precision, h->paper_ports, s);
@@ -1045,6 +1047,7 @@ lbm_status create_impl(lbm_handle* out, int32_t nx, int32_t ny, const uint8_t* m
             h->pair_grid = plan.grid;
             h->pair_warps = plan.warps;
             h->pairs = plan.worth;
+            h->pairs_keep = plan.worth_keep;
         }
     }
     std::vector<lbm::WallLink> wall_list;
@@ -1871,10 +1874,26 @@ lbm_status lbm_adjoint(lbm_handle h, const lbm_objective* obj, int64_t n, int32_
     // Forward steps t = tstart .. tstart + m - 1 of the run, step t reading
     // slot (t - tstart) of `from` and writing the next slot (every state
     // kept); with multi_step, runs of unchanged valve words go to the
-    // cooperative kernel.
+    // cooperative kernel.  Else two steps go to a launch where that pays
+    // (plan_pairs), the state between them stored as well.
     auto forward_slots = [&](lbm::StepArgs& x, float* from, int64_t tstart, int64_t m) -> lbm_status {
         const long long stride = (long long)(S / sizeof(float));
+        int keep = 0;  // blocks an SM of the launches of two steps; 0: none
+        if (!coop && h->pairs && h->pairs_keep && m >= 2 && lbm::pair_keep_occupancy(h->pair_warps, &keep) != cudaSuccess) keep = 0;
         for (int64_t s = 0; s < m;) {
+            CUtensorMap map;
+            if (keep > 0 && m - s >= 2 &&
+                lbm::pair_tensor_map(&map, from + s * stride, h->ny, h->pitch, h->precision, h->pair_warps) == cudaSuccess) {
+                const uint32_t next[lbm::kMaskWords] = {h->mask_at(t0 + tstart + s + 1)};
+                x.open_mask[0] = h->mask_at(t0 + tstart + s);
+                x.reverse = int((s >> 1) & 1);
+                x.src = from + s * stride;
+                x.dst = from + (s + 2) * stride;
+                cudaError_t e = launch_pair(h, x, next, map, st, from + (s + 1) * stride);
+                if (e != cudaSuccess) return cuda_fail(h, e, "two-step launch");
+                s += 2;
+                continue;
+            }
             const int64_t run = coop ? h->mask_run(t0 + tstart + s, std::min<int64_t>(m - s, h->multi_step)) : 1;
             x.open_mask[0] = h->mask_at(t0 + tstart + s);
             x.reverse = int((tstart + s) & 1);
@@ -1891,9 +1910,9 @@ lbm_status lbm_adjoint(lbm_handle h, const lbm_objective* obj, int64_t n, int32_
         }
         return LBM_OK;
     };
-    if (K == 1 && coop) {
-        // every state kept, runs of steps in cooperative launches; the last
-        // step writes into the other buffer
+    if (K == 1) {
+        // every state kept: the steps write straight into the state array (no
+        // copies, no recomputation), the last one into the other buffer
         LBM_CUDA(h, cudaMemcpyAsync(ckpt, h->pop[h->cur], S, cudaMemcpyDeviceToDevice, st));
         if (lbm_status fs = forward_slots(a, reinterpret_cast<float*>(ckpt), 0, n - 1)) return fs;
         a.src = reinterpret_cast<float*>(ckpt + size_t(n - 1) * S);
@@ -1903,22 +1922,6 @@ lbm_status lbm_adjoint(lbm_handle h, const lbm_objective* obj, int64_t n, int32_
         a.partials = h->partials;
         cudaError_t e = lbm::launch_step(a, h->launch, st);
         if (e != cudaSuccess) return cuda_fail(h, e, "coupled step launch");
-        swap_buffers(h);
-        h->diag_grid = h->launch.grid;
-        h->step += n;
-    } else if (K == 1) {
-        // every state kept: the steps write straight into the state array
-        // (no copies, no recomputation), the last one into the other buffer
-        LBM_CUDA(h, cudaMemcpyAsync(ckpt, h->pop[h->cur], S, cudaMemcpyDeviceToDevice, st));
-        for (int64_t t = 0; t < n; ++t) {
-            a.src = t == 0 ? h->pop[h->cur] : reinterpret_cast<float*>(ckpt + size_t(t) * S);
-            a.dst = t + 1 < n ? reinterpret_cast<float*>(ckpt + size_t(t + 1) * S) : h->pop[1 - h->cur];
-            a.reverse = int(t & 1);
-            a.open_mask[0] = h->mask_at(t0 + t);
-            a.partials = t + 1 < n ? nullptr : h->partials;
-            cudaError_t e = lbm::launch_step(a, h->launch, st);
-            if (e != cudaSuccess) return cuda_fail(h, e, "coupled step launch");
-        }
         swap_buffers(h);
         h->diag_grid = h->launch.grid;
         h->step += n;

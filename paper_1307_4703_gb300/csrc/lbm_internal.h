@@ -133,10 +133,12 @@ struct PairArgs {
     StepArgs second;        // time t + 1: writes dst; plane = kTileNodes (its own-node reads go to the ring)
     const int4* items;
     const int* block_first;
+    void* mid;              // the state between the steps goes here too (FP32 without rescaling ports); null: nowhere
 };
 // warps of a block: 4 or 6 (FP32), 6 or 8 (16-bit storage); rescale: the lattice
 // has ports of the rescaling kinds.
 cudaError_t pair_occupancy(int precision, bool rescale, int warps, int* per_sm);
+cudaError_t pair_keep_occupancy(int warps, int* per_sm);  // of launches with PairArgs::mid
 // A tensor map of `planes` planes of ny rows of `pitch` elements of `elem`
 // bytes at base, with boxes of cols x rows of one plane.
 cudaError_t rows_tensor_map(CUtensorMap* map, void* base, int planes, int ny, int pitch, int elem, int cols, int rows);

@@ -283,7 +283,7 @@ __device__ __forceinline__ void collide_row(const StepArgs& a, float4 (&v)[kPlan
     bad |= q.bad;
 }
 
-template <typename T, bool kRescale, int W>
+template <typename T, bool kRescale, int W, bool kKeep>
 __global__ void __launch_bounds__(32 * W, pair_blocks(W))
     coupled_step_pair(const PairArgs p, const __grid_constant__ CUtensorMap map)
 {
@@ -398,6 +398,13 @@ __global__ void __launch_bounds__(32 * W, pair_blocks(W))
             complete_quad<kRescale>(p.first, st.port, v, lk, at_side ? 0x0Au : 0xFFu, st.x0 + 4 * lane, bc, src, P,
                           (long long)y * pitch + st.x0 + 4 * lane);
             collide_row<kRescale, T>(p.first, v, lk, rates_of(p.first, rates), bad);
+            if constexpr (kKeep) {  // the state between the steps, of the rows and lanes the second step writes
+                if (y >= st.ya && y < st.yb && lane >= st.l0 && lane <= st.l1) {
+                    T* const M = static_cast<T*>(p.mid) + (long long)y * pitch + st.x0 + 4 * lane;
+#pragma unroll
+                    for (int q = 0; q < kPlanes; ++q) Codec<T>::st4(M + q * P, v[q], 0.f);
+                }
+            }
         }
         if (t > 0 && !late) late = !mbar_wait(&sm.read, (t - 1) & 1u);
         if (here) {
@@ -471,7 +478,7 @@ __global__ void __launch_bounds__(32 * W, pair_blocks(W))
     if (__any_sync(kFull, bad) && lane == 0) atomicOr(p.first.err, 1u);
 }
 
-template <typename T, bool kRescale, int W>
+template <typename T, bool kRescale, int W, bool kKeep = false>
 cudaError_t launch(const PairArgs& p, const CUtensorMap& map, int grid, cudaStream_t s)
 {
     cudaLaunchConfig_t cfg = {};
@@ -484,16 +491,16 @@ cudaError_t launch(const PairArgs& p, const CUtensorMap& map, int grid, cudaStre
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, coupled_step_pair<T, kRescale, W>, p, map);
+    return cudaLaunchKernelEx(&cfg, coupled_step_pair<T, kRescale, W, kKeep>, p, map);
 }
 
-template <typename T, bool kRescale, int W>
+template <typename T, bool kRescale, int W, bool kKeep = false>
 cudaError_t occupancy(int* per_sm)
 {
-    cudaError_t e = cudaFuncSetAttribute(coupled_step_pair<T, kRescale, W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(coupled_step_pair<T, kRescale, W, kKeep>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          int(sizeof(PairSmem<T, W>)));
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, coupled_step_pair<T, kRescale, W>, 32 * W,
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, coupled_step_pair<T, kRescale, W, kKeep>, 32 * W,
                                                           sizeof(PairSmem<T, W>));
     return e;
 }
@@ -528,6 +535,8 @@ struct Launch {
     template <typename T, bool kRescale, int W>
     cudaError_t operator()() const
     {
+        if constexpr (sizeof(T) == 4 && !kRescale)
+            if (p.mid != nullptr) return launch<T, kRescale, W, true>(p, map, grid, s);
         return launch<T, kRescale, W>(p, map, grid, s);
     }
 };
@@ -537,6 +546,11 @@ struct Launch {
 cudaError_t pair_occupancy(int precision, bool rescale, int warps, int* per_sm)
 {
     return instance(precision, rescale, warps, Occupancy{per_sm});
+}
+
+cudaError_t pair_keep_occupancy(int warps, int* per_sm)
+{
+    return warps == 4 ? occupancy<float, false, 4, true>(per_sm) : occupancy<float, false, 6, true>(per_sm);
 }
 
 cudaError_t rows_tensor_map(CUtensorMap* map, void* base, int planes, int ny, int pitch, int elem, int cols, int rows)

@@ -332,6 +332,12 @@ StripPlan plan_pairs(const std::vector<uint2>& tiles, const std::vector<RowBC>& 
     const double work = p.work / (2.0 * double(tiles.size()));
     const bool few = rescale && f32 && (long long)tiles.size() <= 2 * single_warps;
     p.worth = idle || (!few && work < (f32 ? 1.5 : 1.8));
+    // With the state between the steps stored as well (a gradient's recomputation):
+    // ahead on lattices that leave the GPU idle (a gradient over 150 steps of 256 x 128
+    // 1605 -> 1447 us, 512 x 256 1270 -> 1210) and on those of more than two rounds of a
+    // single step's tiles (2048 x 1024 3.70 -> 3.51 ms, 4096 x 2048 6.34 -> 6.04); between
+    // them a draw (1024 x 512 3161 / 3194 us, 1500 x 900 2313 / 2322).
+    p.worth_keep = idle || (p.worth && (long long)tiles.size() > 2 * single_warps);
     return p;
 }
 

@@ -16,6 +16,7 @@ struct StripPlan {
     int longest = 0;               // cost of the block that takes longest
     double work = 0;
     bool worth = false;            // faster than single steps
+    bool worth_keep = false;       // also with every state stored
 };
 
 // A block shape of the two-step kernel, how many of its blocks are resident at
