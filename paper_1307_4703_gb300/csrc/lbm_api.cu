@@ -1348,6 +1348,7 @@ lbm_status lbm_step(lbm_handle h, int64_t n)
                 a.src = h->pop[h->cur];
                 a.dst = h->pop[1 - h->cur];
                 a.reverse = h->order;
+                a.partials = m < n - k ? nullptr : h->partials;  // as the other launches: the call's last step's only
                 a.barrier_extra = h->barrier_extra;
                 cudaError_t e =
                     lbm::launch_steps_coop(a, int(m), 0, h->bar, h->coop_grid, kDefaultRegsBlock, h->stream);
