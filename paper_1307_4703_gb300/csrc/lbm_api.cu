@@ -414,6 +414,16 @@ cudaError_t launch_pair(const lbm_ctx* h, const lbm::StepArgs& a, const uint32_t
 // nothing could read.
 bool pair_next(const lbm_ctx* h, int64_t left) { return h->pairs && left >= 3; }
 
+// Whether the handle's stream records a CUDA graph of the caller's, or cannot
+// be used for another stream's recording.
+bool capturing(const lbm_ctx* h)
+{
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->stream, &s) == cudaSuccess) return s != cudaStreamCaptureStatusNone;
+    cudaGetLastError();  // the launches that follow report it
+    return true;
+}
+
 // The cached graph of graph_steps launches for the valve words in
 // a.open_mask starting from buffer cur, captured on first use.
 lbm_status step_graph(lbm_ctx* h, lbm::StepArgs a, const lbm_ctx::Graph** out)
@@ -1338,6 +1348,12 @@ lbm_status lbm_step(lbm_handle h, int64_t n)
     if (lbm_status js = join_scalar(h)) return js;
     lbm::StepArgs a = step_args(h);
     const int G = h->graph_steps;
+    // A graph that the caller records of an even number of steps has to end in
+    // the buffer it begins in, or its second replay would start from the wrong
+    // one: there two-step launches come in twos (n steps swap the buffers as
+    // often as n single ones, but for an even number).
+    const bool in_twos = pair_next(h, n) && capturing(h);
+    int64_t pairs = 0;  // two-step launches of this call
     for (int64_t k = 0; k < n;) {
         h->mask_words(h->step, a.open_mask);
         if (h->multi_step > 0 && n - k >= 2) {
@@ -1375,7 +1391,8 @@ lbm_status lbm_step(lbm_handle h, int64_t n)
         }
         a.src = h->pop[h->cur];
         a.dst = h->pop[1 - h->cur];
-        if (pair_next(h, n - k)) {
+        if (pair_next(h, n - k) && (!in_twos || (pairs & 1) || n - k >= 5)) {
+            ++pairs;
             a.reverse = h->cur;  // alternate the march from launch to launch
             uint32_t next[lbm::kMaskWords];
             h->mask_words(h->step + 1, next);
@@ -2134,9 +2151,7 @@ float* field_slot(lbm_ctx* h, uint32_t word)
 // handle that cannot have them steps one launch at a time.
 void plan_scalar_levels(lbm_ctx* h)
 {
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    if (!h->scalar_levels || cudaStreamIsCapturing(h->stream, &capture) != cudaSuccess ||
-        capture != cudaStreamCaptureStatusNone)
+    if (!h->scalar_levels || capturing(h))
         return;  // a call being captured may not wait for the stream: the next one plans
     h->scalar_levels = false;  // once
     int per_sm = 0;
