@@ -50,18 +50,23 @@ std::vector<Strip> cover(const std::vector<Span>& spans, int nx, int pitch)
     return out;
 }
 
-// Strips of `strips` that a row's spans touch, and whether they cover them all.
-int touched(const std::vector<Strip>& strips, const std::vector<Span>& spans, bool& covered)
+// Which of `strips` a row's spans touch (both in order of their columns, one walk
+// over them), how many, and whether they cover all of the spans.
+int touched(const std::vector<Strip>& strips, const std::vector<Span>& spans, std::vector<char>& hit, bool& covered)
 {
     int hits = 0;
-    covered = true;
-    for (const Strip& t : strips)
-        for (const Span& s : spans)
-            if (s.b < t.end() && t.begin() < s.e) {
-                ++hits;
-                break;
-            }
     size_t k = 0;
+    hit.assign(strips.size(), 0);
+    for (size_t n = 0; n < strips.size(); ++n) {
+        while (k < spans.size() && spans[k].e <= strips[n].begin()) ++k;
+        if (k == spans.size()) break;
+        if (spans[k].b < strips[n].end()) {
+            hit[n] = 1;
+            ++hits;
+        }
+    }
+    covered = true;
+    k = 0;
     for (const Span& s : spans)
         for (int p = s.b; p < s.e;) {
             while (k < strips.size() && strips[k].end() <= p) ++k;
@@ -130,17 +135,18 @@ std::vector<Run> strip_runs(const std::vector<Rows>& groups)
     std::vector<Run> runs;
     std::vector<Strip> cur;
     std::vector<int> open;  // index of each strip's run in `runs`, -1 = none
+    std::vector<char> hit, ahead;
     for (size_t k = 0; k < groups.size(); ++k) {
         const Rows& g = groups[k];
         bool covered = false;
-        if (!g.spans.empty()) touched(cur, g.spans, covered);
-        bool fresh = !covered;
-        if (covered) {  // would other strips do with fewer, and for long enough?
+        const int hits = touched(cur, g.spans, hit, covered);
+        bool fresh = g.spans.empty() || !covered;
+        if (!fresh) {  // would other strips do with fewer, and for long enough?
             int gain = 0;
             for (size_t n = k; n < groups.size() && gain < kBandRows; ++n) {
                 bool c = false;
                 if (groups[n].spans.empty() ||
-                    touched(cur, groups[n].spans, c) <= int(groups[n].own.size()))
+                    (n == k ? hits : touched(cur, groups[n].spans, ahead, c)) <= int(groups[n].own.size()))
                     break;
                 gain += groups[n].yb - groups[n].ya;
             }
@@ -149,11 +155,10 @@ std::vector<Run> strip_runs(const std::vector<Rows>& groups)
         if (fresh) {
             cur = g.own;
             open.assign(cur.size(), -1);
+            touched(cur, g.spans, hit, covered);
         }
         for (size_t n = 0; n < cur.size(); ++n) {
-            bool hit = false;
-            for (const Span& s : g.spans) hit |= s.b < cur[n].end() && cur[n].begin() < s.e;
-            if (!hit) open[n] = -1;
+            if (!hit[n]) open[n] = -1;
             else if (open[n] >= 0) runs[size_t(open[n])].yb = g.yb;
             else {
                 open[n] = int(runs.size());
@@ -174,22 +179,35 @@ std::vector<Run> split_kinds(const std::vector<Run>& runs, const std::vector<Row
     std::vector<int> group_of(static_cast<size_t>(ny));
     for (size_t k = 0; k < groups.size(); ++k)
         for (int y = groups[k].ya; y < groups[k].yb; ++y) group_of[size_t(y)] = int(k);
-    std::vector<std::vector<int>> walls(static_cast<size_t>(ny));  // first columns of each row's tiles with scattered walls
+    // first columns of the tiles with scattered walls, row after row
+    std::vector<int> walls, first_wall;
     for (const uint2& t : tiles)
-        if (t.y & kWallTile)
-            walls[size_t(t.x >> kColBits)].push_back(int(t.x & ((1u << kColBits) - 1)) * kTileStart);
+        if (t.y & kWallTile) {
+            first_wall.resize(size_t(t.x >> kColBits) + 1, int(walls.size()));
+            walls.push_back(int(t.x & ((1u << kColBits) - 1)) * kTileStart);
+        }
+    first_wall.resize(size_t(ny) + 1, int(walls.size()));
+    std::vector<int> port_cols;
+    for (const RowBC& b : bc)
+        if (b.x >= 0 && (port_cols.empty() || port_cols.back() != b.x)) port_cols.push_back(b.x);
+    std::sort(port_cols.begin(), port_cols.end());
     for (const Run& r : runs) {
         const int x0 = r.t.x0, x1 = x0 + kTileNodes;
         // the lanes where the row's fluid begins and ends within the strip; -1: more than two
         auto side = [&](int y) {
             int lanes = 0, n = 0;
-            for (const Span& s : groups[size_t(group_of[size_t(y)])].spans) {
-                if (s.b >= x0 && s.b < x1 && n++ < 2) lanes |= (s.b - x0) / 4 << (kPairLaneBit + 5 * (n - 1));
-                if (s.e > x0 && s.e <= x1 && n++ < 2) lanes |= (s.e - 4 - x0) / 4 << (kPairLaneBit + 5 * (n - 1));
+            const std::vector<Span>& spans = groups[size_t(group_of[size_t(y)])].spans;
+            auto s = std::lower_bound(spans.begin(), spans.end(), x0, [](const Span& a, int x) { return a.e <= x; });
+            for (; s != spans.end() && s->b < x1 && n < 3; ++s) {
+                if (s->b >= x0 && n++ < 2) lanes |= (s->b - x0) / 4 << (kPairLaneBit + 5 * (n - 1));
+                if (s->e <= x1 && n++ < 2) lanes |= (s->e - 4 - x0) / 4 << (kPairLaneBit + 5 * (n - 1));
             }
             return n == 1 || n == 2 ? lanes | kPairSide : n ? -1 : 0;
         };
+        const auto col = std::lower_bound(port_cols.begin(), port_cols.end(), x0);
+        const bool any_port = col != port_cols.end() && *col < x1;
         auto port = [&](int y) {
+            if (!any_port) return false;
             for (int yy = std::max(y - halo, 0); yy <= std::min(y + halo, ny - 1); ++yy)
                 for (int s = 0; s < 2; ++s) {
                     const int px = bc[size_t(s) * ny + yy].x;
@@ -198,9 +216,9 @@ std::vector<Run> split_kinds(const std::vector<Run>& runs, const std::vector<Row
             return false;
         };
         auto scattered = [&](int y) {
-            for (int x : walls[size_t(y)])
-                if (x < x1 && x0 < x + kTileNodes) return true;
-            return false;
+            const auto end = walls.begin() + first_wall[size_t(y) + 1];
+            const auto w = std::upper_bound(walls.begin() + first_wall[size_t(y)], end, x0 - kTileNodes);
+            return w != end && *w < x1;
         };
         for (int y = r.ya; y < r.yb;) {
             const bool ports = port(y);
