@@ -186,3 +186,19 @@ def test_planning_time_follows_the_size(lib):
     def seconds(nx):
         return min(Plan(lib, cells.reshape(-1, nx), levels=k).seconds for k in (0, LEVELS, 0, LEVELS, 0))
     assert seconds(131072) < 4 * seconds(512)
+
+
+@pytest.mark.parametrize("share", [0.2, 0.5, 0.7])
+@pytest.mark.parametrize("nx,ny", [(2001, 1003), (4096, 2048)])
+def test_dense_lattices_stay_in_long_strips(lib, nx, ny, share):
+    """Scattered cells: strips as long as a block's share of the lattice, whatever part of it
+    is solid (half solid fell into pieces of five rows).  A strip writes 120 of its 128
+    columns and computes halo rows above and below it, so with at least ten strips a block's
+    length apart the work is that of the tiles times the cost of an iteration (28 / 16,
+    scalar 24 / 16), 128 / 120 and a tenth for the ends."""
+    solid = np.random.default_rng(3).random((ny, nx)) < share
+    for levels, cost in ((0, 28 / 16), (LEVELS, 24 / 16)):
+        for precision in (FP32, FP16) if not levels else (FP32,):
+            p = Plan(lib, solid, levels=levels, precision=precision)
+            assert len(p.items) <= 2 * p.grid
+            assert p.work < cost * 128 / 120 * 1.2 * p.tiles
