@@ -90,12 +90,17 @@ enum Kind { kPlain, kSide, kScattered, kPort, kScatteredPort };
 constexpr int kPairCost[5] = {16, 18, 28, 22, 33};
 constexpr int kPairRescaleCost[5] = {16, 18, 28, 30, 42};  // with ports of the rescaling kinds (22: 4096 x 2048 44 us, here 39)
 constexpr int kScalarCost[5] = {16, 20, 24, 28, 32};
+// What an FP32 iteration of two coupled steps takes, in units of 0.131 us a step
+// (least squares over some hundred lattices; the costs above are those of the
+// fastest splits).
+constexpr int kPairTime[5] = {16, 17, 21, 22, 25};
 
 struct Run {
     Strip t;
     int ya, yb;
     Kind kind;
-    int side;  // kPairSide and the lanes along the walls
+    int side;   // kPairSide and the lanes along the walls
+    int rough;  // rows with scattered walls
 };
 
 constexpr int kBandRows = 8;  // rows that must gain from new strips before the strips change
@@ -162,7 +167,7 @@ std::vector<Run> strip_runs(const std::vector<Rows>& groups)
             else if (open[n] >= 0) runs[size_t(open[n])].yb = g.yb;
             else {
                 open[n] = int(runs.size());
-                runs.push_back({cur[n], g.ya, g.yb, kPlain, 0});
+                runs.push_back({cur[n], g.ya, g.yb, kPlain, 0, 0});
             }
         }
     }
@@ -245,9 +250,10 @@ std::vector<Run> split_kinds(const std::vector<Run>& runs, const std::vector<Row
             Run* const before = y > r.ya ? &out.back() : nullptr;
             if (before && before->kind == kind && (kind == kScattered || kind == kScatteredPort)) {
                 before->yb = e;
+                before->rough += rough;
                 if (before->side != walls_at) before->side = 0;
             } else {
-                out.push_back({r.t, y, e, kind, walls_at});
+                out.push_back({r.t, y, e, kind, walls_at, rough});
             }
             y = e;
         }
@@ -259,7 +265,7 @@ std::vector<Run> split_kinds(const std::vector<Run>& runs, const std::vector<Row
 // most `m` units of cost a block; returns the blocks this takes.
 int split(const std::vector<Run>& runs, const int (&costs)[5], int halo, int W, int m, StripPlan* out)
 {
-    int blocks = 1, left = m;
+    int blocks = 1, left = m, time = 0;
     if (out) {
         out->items.clear();
         out->block_first.assign(1, 0);
@@ -267,16 +273,26 @@ int split(const std::vector<Run>& runs, const int (&costs)[5], int halo, int W, 
     auto next_block = [&]() {
         ++blocks;
         left = m;
+        time = 0;
         if (out) out->block_first.push_back(int(out->items.size()));
     };
     for (const Run& r : runs) {
         const int cost = costs[r.kind];
+        // (an iteration is as slow as its slowest row: scattered walls in half of the
+        // rows are in 0.7 of the iterations)
+        const int rows = r.yb - r.ya, base = kPairTime[r.kind];
+        const int more = kPairTime[r.kind >= kPort ? kScatteredPort : kScattered] - base;
+        const int step = base + more * std::min(7 * r.rough, 5 * rows) / (5 * rows);
         for (int y = r.ya; y < r.yb;) {
             if (left < m && left / cost * W - 2 * halo < std::min(r.yb - y, W)) next_block();
             const int h = std::min(r.yb - y, std::max(left / cost * W - 2 * halo, 1));
-            left -= (h + 2 * halo + W - 1) / W * cost;
-            if (out)
+            const int iterations = (h + 2 * halo + W - 1) / W;
+            left -= iterations * cost;
+            time += iterations * step;
+            if (out) {
+                out->time = std::max(out->time, time);
                 out->items.push_back(make_int4(r.t.x0, r.t.l0 | (r.t.l1 << 8) | (r.kind >= kPort ? kPairPort : 0) | r.side, y, y + h));
+            }
             y += h;
         }
     }
@@ -345,22 +361,35 @@ StripPlan plan_pairs(const std::vector<uint2>& tiles, const std::vector<RowBC>& 
         resident = s.resident;
         p = std::move(q);
     }
-    // Where two single steps are the better choice, in us a step, single / two-step
-    // launches: where obstacles break the rows into strips that do far more than
-    // the tiles' work.  FP32 at 1.7 and 1.8 of it 22.2 / 25.4 and 47.7 / 50.5, at 1.5 a
-    // draw (6.2 / 6.5, 10.5 / 9.4); 16-bit storage, whose single step is bound by issue
-    // and starts up longer, at 2.1 of it 19.5 / 20.7 and at 1.5 8.1 / 4.2.  Elsewhere two
-    // steps are ahead: FP32 256 x 128 3.65 / 2.52, 1024 x 512 5.24 / 4.60, 1024 x 768
-    // 7.1 / 5.4, 4096 x 2048 59.5 / 38.0, with 3 % obstacles 800 x 500 10.2 / 8.5 and
-    // 2001 x 1003 40.7 / 33; FP16 256 x 128 4.8 / 2.7, 1024 x 768 5.6 / 5.2, 4096 x 2048
-    // 36.2 / 28.1 (900 x 700 is the closest: 5.23 / 5.36 in FP32).  With rescaling
-    // ports FP32 strips gain from the third tile of a single step's warps on (1024 x
-    // 768 7.2 / 7.6, 4096 x 2048 54.4 / 39.0).  Strips that leave half the blocks' room
-    // idle are always the shorter way.
+    // Where two single steps are the better choice: where obstacles break the rows
+    // into strips that do far more than the tiles' work.  Strips that leave half the
+    // blocks' room idle are always the shorter way.
     const bool idle = 2 * p.grid <= resident;
-    const double work = p.work / (2.0 * double(tiles.size()));
-    const bool few = rescale && f32 && (long long)tiles.size() <= 2 * single_warps;
-    p.worth = idle || (!few && work < (f32 ? 1.5 : 1.8));
+    const double n = double(tiles.size()), work = p.work / (2. * n);
+    if (f32 && !rescale) {
+        // The longest block's time against a single step's: a wave of tiles, rounds of
+        // them, or HBM's rate, and what their scattered walls add.  Both are fits, within
+        // 15 % over some three hundred lattices; strips of much more work than the tiles'
+        // have to be ahead by a tenth.  us a step, single / two-step launches: 256 x 128
+        // 3.6 / 2.3, 1024 x 512 5.24 / 4.60, 1024 x 768 7.1 / 5.4, 4096 x 2048 59.5 / 35.5;
+        // random cells, 3 and 70 % solid, 1001 x 517 10.5 / 9.5 and 12.2 / 9.6, 2001 x 1003
+        // 40.7 / 32.4 and 51.3 / 36.5; pillars of 10 cells 24 apart, whose strips fall into
+        // pieces of a dozen rows, 2001 x 1003 39.0 / 31.5 but 900 x 600 9.5 / 10.9 and 700 x
+        // 400 5.7 / 8.6.
+        double scattered = 0.;
+        for (const uint2& t : tiles) scattered += (t.y & kWallTile) != 0;
+        const bool one_round = (long long)tiles.size() <= single_warps;
+        const double single = std::max(one_round ? 3.2 + 0.95e-3 * n : 4.0 + 1.25e-3 * n, 2.1e-3 * n) + 0.5e-3 * scattered;
+        p.worth = idle || (p.warps == 4 ? 0.126 : 0.131) * p.time < (work < 1.5 ? 1.06 : 0.9) * single;
+    } else {
+        // The work alone.  16-bit storage, whose single step is bound by issue and starts
+        // up longer: FP16 256 x 128 4.8 / 2.4, 1024 x 768 5.6 / 4.9, 4096 x 2048 36.2 / 28.1,
+        // at 2.1 of the tiles' work 19.5 / 20.7 and at 1.5 8.1 / 4.2.  With rescaling ports
+        // FP32 strips gain from the third tile of a single step's warps on (1024 x 768
+        // 7.2 / 7.6, 4096 x 2048 54.4 / 39.0).
+        const bool few = f32 && (long long)tiles.size() <= 2 * single_warps;
+        p.worth = idle || (!few && work < (f32 ? 1.5 : 1.8));
+    }
     // With the state between the steps stored as well (a gradient's recomputation):
     // ahead on lattices that leave the GPU idle (a gradient over 150 steps of 256 x 128
     // 1605 -> 1447 us, 512 x 256 1270 -> 1210) and on those of more than two rounds of a

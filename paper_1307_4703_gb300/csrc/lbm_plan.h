@@ -14,6 +14,7 @@ struct StripPlan {
     int grid = 0;
     int warps = 0;                 // of a block (plan_pairs)
     int longest = 0;               // cost of the block that takes longest
+    int time = 0;                  // the longest block's time (kPairTime)
     double work = 0;
     bool worth = false;            // faster than single steps
     bool worth_keep = false;       // also with every state stored

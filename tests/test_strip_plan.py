@@ -202,3 +202,26 @@ def test_dense_lattices_stay_in_long_strips(lib, nx, ny, share):
             p = Plan(lib, solid, levels=levels, precision=precision)
             assert len(p.items) <= 2 * p.grid
             assert p.work < cost * 128 / 120 * 1.2 * p.tiles
+
+
+def _pillars(nx, ny, step, side):
+    solid = np.zeros((ny, nx), np.uint8)
+    for y in range(4, ny - 8, step):
+        for x in range(4 + (y // step % 2) * step // 2, nx - 8, step):
+            solid[y:min(y + side, ny - 4), x:min(x + side, nx - 4)] = 1
+    return solid
+
+
+def test_two_steps_a_launch_where_they_are_faster(lib):
+    """FP32, by the measured times a step that csrc/lbm_plan.cu gives: channel chips and
+    lattices of scattered cells take two steps a launch, pillars whose strips fall into
+    pieces only on large lattices."""
+    for prob in (W.config_small(), W.config_full_chip(), W.config_adjoint_chip(), W.config_large_chip(2000, 1000)):
+        assert Plan(lib, prob["solid"], prob["ports"]).worth, prob["name"]
+    for nx, ny in ((1001, 517), (2001, 1003)):
+        for share in (0.03, 0.2, 0.5, 0.7):
+            assert Plan(lib, np.random.default_rng(5).random((ny, nx)) < share).worth, (nx, ny, share)
+    for nx, ny, step, side, worth in ((2001, 1003, 24, 10, True), (3000, 1500, 24, 10, True), (700, 400, 24, 10, False),
+                                      (900, 600, 24, 10, False), (1001, 517, 24, 10, False), (700, 400, 12, 6, False)):
+        ports = W.random_case(5, nx, ny, solid_frac=0.0)[0]["ports"]
+        assert Plan(lib, _pillars(nx, ny, step, side), ports).worth == worth, (nx, ny, step, side)
