@@ -2147,12 +2147,13 @@ float* field_slot(lbm_ctx* h, uint32_t word)
     if (u) h->fields.push_back({word, u});
     return u;
 }
-// The strips of the several-steps launches, with the first stored field; a
-// handle that cannot have them steps one launch at a time.
+// The strips of the several-steps launches, with the first stored field (or, where
+// that call was captured, with the first scalar steps that are not); a handle that
+// cannot have them steps one launch at a time.
 void plan_scalar_levels(lbm_ctx* h)
 {
     if (!h->scalar_levels || capturing(h))
-        return;  // a call being captured may not wait for the stream: the next one plans
+        return;  // a call being captured may not wait for the stream
     h->scalar_levels = false;  // once
     int per_sm = 0;
     CUtensorMap probe;
@@ -2163,7 +2164,6 @@ void plan_scalar_levels(lbm_ctx* h)
     }
     const lbm::StripPlan p = lbm::plan_scalar(h->tiles_rows, h->rowbc_host, h->nx, h->ny, h->pitch, lbm::kScalarLevels,
                                               lbm::scalar_level_warps(), per_sm * h->sms);
-    if (!p.worth) return;
     h->scalar_items = static_cast<int4*>(dev_alloc(h, p.items.size() * sizeof(int4)));
     h->scalar_first = static_cast<int*>(dev_alloc(h, p.block_first.size() * sizeof(int)));
     if (!h->scalar_items || !h->scalar_first) return;
@@ -2257,6 +2257,7 @@ lbm_status lbm_scalar_step(lbm_handle h, int64_t n, double u_scale)
         h->scalar_grid = std::max(1, std::min((h->n_tiles + tiles_per_block - 1) / tiles_per_block,
                                               std::max(1, per_sm) * h->sms));
     }
+    if (n > lbm::kScalarLevels) plan_scalar_levels(h);
     const int scalar_grid = std::min(h->scalar_grid, h->partials_cap);
     a.n_partials = std::max(h->diag_grid, scalar_grid);
     int g = h->gbuf;  // buffer holding the current scalar planes

@@ -16,8 +16,8 @@ struct StripPlan {
     int longest = 0;               // cost of the block that takes longest
     int time = 0;                  // the longest block's time (kPairTime)
     double work = 0;
-    bool worth = false;            // faster than single steps
-    bool worth_keep = false;       // also with every state stored
+    bool worth = false;            // faster than single steps (plan_pairs)
+    bool worth_keep = false;       // also with every state stored (plan_pairs)
 };
 
 // A block shape of the two-step kernel, how many of its blocks are resident at
@@ -27,10 +27,10 @@ struct PairShape {
 };
 // tiles: the lattice's 128-node tiles in row order; bc: 2 ny port entries;
 // rescale: it has ports of the rescaling kinds; shapes: the usual one first, then
-// the one of fewer warps; single_warps: of the single
-// step's grid; warps, resident: of a block, blocks in one wave.
+// the one of fewer warps; single_warps: of the single step's grid.
 StripPlan plan_pairs(const std::vector<uint2>& tiles, const std::vector<RowBC>& bc, int nx, int ny, int pitch,
                      int precision, bool rescale, const PairShape* shapes, int n_shapes, long long single_warps);
+// levels: steps a launch; warps of a block; resident: blocks in one wave.
 StripPlan plan_scalar(const std::vector<uint2>& tiles, const std::vector<RowBC>& bc, int nx, int ny, int pitch, int levels,
                       int warps, int resident);
 
