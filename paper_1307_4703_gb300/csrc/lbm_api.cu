@@ -1525,7 +1525,7 @@ lbm_status lbm_get_fields_device(lbm_handle h, float* rho, float* ux, float* uy,
     if (check_ctx(h)) return LBM_ERR_ARG;
     if (lbm_status js = join_scalar(h)) return js;
     cudaError_t e = lbm::launch_fields(h->pop[h->cur], h->links, h->nx, h->ny, h->pitch, rho, ux, uy, C, h->wg0,
-                                       h->wg1, h->precision, h->decay, h->stream);
+                                       h->wg1, h->precision, h->decay, h->sms, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "fields kernel launch");
     return LBM_OK;
 }

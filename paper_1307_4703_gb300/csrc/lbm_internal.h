@@ -306,10 +306,10 @@ cudaError_t launch_init_fields(void* pop, const uint8_t* links, int nx, int ny, 
 // null); solid nodes give 0.  The stored populations are post-collision:
 // with decay rate k the collision removed k C, so C is reported as
 // sum g / (1 - k), the concentration before the collision (the moments of f
-// are the same before and after it).
+// are the same before and after it).  sms: of the device.
 cudaError_t launch_fields(const void* pop, const uint8_t* links, int nx, int ny, int pitch,
                           float* rho, float* ux, float* uy, float* C, float wg0, float wg1, int precision,
-                          float decay, cudaStream_t s);
+                          float decay, int sms, cudaStream_t s);
 
 // 16-bit storage <-> the FP32 representation (fluid planes f_i - w_i, scalar
 // planes g_i), element by element over n_elems = 14 * ny * pitch.

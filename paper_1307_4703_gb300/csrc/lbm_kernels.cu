@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(128, kFieldsBlocks) fields_kernel(const T* pop
     const int x = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
     if (x >= nx) return;
     const bool flow = rho_out || ux_out || uy_out;
-    for (int y = blockIdx.y; y < ny; y += gridDim.y) {
+    for (int y = blockIdx.y * blockDim.y + threadIdx.y; y < ny; y += gridDim.y * blockDim.y) {
         const long long o = (long long)y * pitch + x;
         const unsigned lk = __ldg(reinterpret_cast<const unsigned*>(links + o));
         float4 r4 = make_float4(0.f, 0.f, 0.f, 0.f), vx4 = r4, vy4 = r4, c4 = r4;
@@ -684,17 +684,21 @@ cudaError_t launch_init_fields(void* pop, const uint8_t* links, int nx, int ny, 
 
 cudaError_t launch_fields(const void* pop, const uint8_t* links, int nx, int ny, int pitch,
                           float* rho, float* ux, float* uy, float* C, float wg0, float wg1, int precision,
-                          float decay, cudaStream_t s)
+                          float decay, int sms, cudaStream_t s)
 {
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = dependent(attr, (nx + 511) / 512, 128, s);
-    // A block a row, but a few rows each where all blocks then fit in one wave
-    // (1024 x 768: 6.8 -> 6.1 us; with more waves than two, rows in turn lose: 4096 x
-    // 2048 52 -> 70 us).
-    constexpr long long wave = 152 * kFieldsBlocks;
-    const long long blocks = (long long)cfg.gridDim.x * ny;
-    const int rows = blocks <= 2 * wave ? int((blocks + wave - 1) / wave) : 1;
-    cfg.gridDim.y = std::min((ny + rows - 1) / rows, 65535);
+    // Rows of up to 64 quads share a block, two or four of them (all fields of 60 x
+    // 4000 8.4 -> 4.6 us, 200 x 4000 9.9 -> 7.9).
+    const int by = nx <= 128 ? 4 : nx <= 256 ? 2 : 1;
+    cfg.blockDim = dim3(128 / by, by);
+    // A block a row (or group of them), but a few rows each where all blocks then fit
+    // in one wave (1024 x 768: 6.8 -> 6.1 us; with more waves than two, rows in turn
+    // lose: 4096 x 2048 52 -> 70 us).
+    const long long wave = (long long)sms * kFieldsBlocks, groups = (ny + by - 1) / by;
+    const long long blocks = (long long)cfg.gridDim.x * groups;
+    const long long each = blocks <= 2 * wave ? (blocks + wave - 1) / wave : 1;
+    cfg.gridDim.y = unsigned(std::min((groups + each - 1) / each, 65535ll));
     // 128-bit stores need rows of whole quads and aligned arrays
     bool vec = nx % 4 == 0;
     for (const float* p : {rho, ux, uy, C}) vec = vec && reinterpret_cast<uintptr_t>(p) % 16 == 0;
