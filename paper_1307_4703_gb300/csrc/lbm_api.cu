@@ -6,6 +6,7 @@
 // kernels on the handle's stream.  No call here computes any part of the
 // time step on the host.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -14,6 +15,7 @@
 #include <mutex>
 #include <new>
 #include <string>
+#include <system_error>
 #include <thread>
 #include <vector>
 
@@ -866,15 +868,35 @@ lbm_status create_impl(lbm_handle* out, int32_t nx, int32_t ny, const uint8_t* m
     };
     const int n_thr = int(std::max<long long>(
         1, std::min<long long>({16, ny, (long long)std::thread::hardware_concurrency(), (long long)nx * ny >> 17})));
-    std::vector<RowsOut> parts(n_thr);
-    {
+    // fn(first row, end, part) for n_thr parts of the rows at once; a part whose
+    // thread cannot be had is done here.  False: out of host memory.
+    auto over_rows = [&](const auto& fn) {
         std::vector<std::thread> pool;
-        for (int k = 1; k < n_thr; ++k)
-            pool.emplace_back(build_rows, int((long long)ny * k / n_thr), int((long long)ny * (k + 1) / n_thr),
-                              std::ref(parts[k]));
-        build_rows(0, int((long long)ny / n_thr), parts[0]);
+        std::atomic<bool> ok{true};
+        auto part = [&](int k) {
+            try {
+                fn(int((long long)ny * k / n_thr), int((long long)ny * (k + 1) / n_thr), k);
+            } catch (const std::bad_alloc&) {
+                ok = false;
+            }
+        };
+        std::vector<int> here{0};
+        pool.reserve(size_t(n_thr));
+        here.reserve(size_t(n_thr));
+        for (int k = 1; k < n_thr; ++k) {
+            try {
+                pool.emplace_back(part, k);
+            } catch (const std::system_error&) {
+                here.push_back(k);
+            }
+        }
+        for (int k : here) part(k);
         for (auto& t : pool) t.join();
-    }
+        return ok.load();
+    };
+    std::vector<RowsOut> parts(n_thr);
+    if (!over_rows([&](int y0, int y1, int k) { build_rows(y0, y1, parts[size_t(k)]); }))
+        return fail(nullptr, LBM_ERR_OOM, "host allocation failed");
     std::vector<uint2> tiles, tiles64;
     long long fluid = 0;
     for (const RowsOut& r : parts) {
@@ -1060,27 +1082,34 @@ lbm_status create_impl(lbm_handle* out, int32_t nx, int32_t ny, const uint8_t* m
             h->pairs_keep = plan.worth_keep;
         }
     }
-    std::vector<lbm::WallLink> wall_list;
+    std::vector<std::vector<lbm::WallLink>> wall_lists(static_cast<size_t>(n_thr));
     if (opt.wall_scheme == LBM_WALL_EQUILIBRIUM) {
-        static const int ex[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1}, ey[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
-        for (size_t o = 0; o < links.size(); ++o) {
-            if (links[o] == 0 || links[o] == lbm::kSolid) continue;
-            for (int i = 1; i <= 8; ++i) {
-                if (!((links[o] >> (i - 1)) & 1)) continue;
-                // bit of "x + e_i is not fluid": the source of the opposite direction
-                const int back = i <= 4 ? (i + 1) & 3 : ((i - 3) & 3) + 4;
-                int ahead = 0;
-                if (!((links[o] >> back) & 1)) {
-                    const size_t o1 = size_t((long long)o + ex[i] + (long long)ey[i] * pitch);
-                    ahead = (links[o1] >> back) & 1 ? 1 : 2;
+        // the links of the fluid nodes, row after row
+        const bool listed = over_rows([&](int y0, int y1, int k) {
+            std::vector<lbm::WallLink>& list = wall_lists[size_t(k)];
+            const long long step[8] = {1, pitch, -1, -pitch, 1 + pitch, pitch - 1, -1 - pitch, 1 - pitch};  // e_i
+            const int back[8] = {2, 3, 0, 1, 6, 7, 4, 5};  // bit of "x + e_i is not fluid": the opposite direction's
+            for (size_t q = size_t(y0) * pitch, end = size_t(y1) * pitch; q < end; q += 8) {
+                uint64_t eight;  // nodes away from walls, or solid
+                std::memcpy(&eight, &links[q], 8);
+                if (eight == 0 || eight == ~uint64_t(0)) continue;
+                for (size_t o = q; o < q + 8; ++o) {
+                    if (links[o] == lbm::kSolid) continue;
+                    for (unsigned b = links[o]; b; b &= b - 1) {
+                        const int i = __builtin_ctz(b);
+                        int ahead = 0;
+                        if (!((links[o] >> back[i]) & 1))
+                            ahead = (links[size_t((long long)o + step[i])] >> back[i]) & 1 ? 1 : 2;
+                        list.push_back(lbm::wall_link((long long)o, i + 1, ahead));
+                    }
                 }
-                wall_list.push_back({(long long)o, i, ahead});
             }
-        }
-        h->n_wall = (long long)wall_list.size();
+        });
+        if (!listed) return bail(fail(h, LBM_ERR_OOM, "host allocation failed"));
+        for (const auto& list : wall_lists) h->n_wall += (long long)list.size();
         h->wallv = dev_alloc(h, size_t(8) * h->plane * h->elem);
         h->wall_list = static_cast<lbm::WallLink*>(
-            dev_alloc(h, std::max<size_t>(1, wall_list.size()) * sizeof(lbm::WallLink)));
+            dev_alloc(h, size_t(std::max(1ll, h->n_wall)) * sizeof(lbm::WallLink)));
     }
     if (!h->pop[0] || !h->pop[1] || !h->links || !h->rowbc || !h->tiles || !h->tiles64 || !h->partials ||
         !h->err || !h->diag || !h->fields_tmp || (batch && !h->rates) ||
@@ -1101,9 +1130,13 @@ lbm_status create_impl(lbm_handle* out, int32_t nx, int32_t ny, const uint8_t* m
                             cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess && batch)
         e = cudaMemcpyAsync(h->rates, batch->rates.data(), size_t(ny) * sizeof(float4), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess && !wall_list.empty())
-        e = cudaMemcpyAsync(h->wall_list, wall_list.data(), wall_list.size() * sizeof(lbm::WallLink),
-                            cudaMemcpyHostToDevice, st);
+    long long listed = 0;
+    for (const auto& list : wall_lists) {
+        if (e == cudaSuccess && !list.empty())
+            e = cudaMemcpyAsync(h->wall_list + listed, list.data(), list.size() * sizeof(lbm::WallLink),
+                                cudaMemcpyHostToDevice, st);
+        listed += (long long)list.size();
+    }
     if (e == cudaSuccess) e = cudaMemsetAsync(h->err, 0, 2 * sizeof(unsigned), st);
     if (e == cudaSuccess)
         e = cudaMemsetAsync(h->partials, 0, size_t(h->partials_cap) * 4 * sizeof(float2), st);

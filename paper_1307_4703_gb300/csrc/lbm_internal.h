@@ -246,11 +246,10 @@ int bulk_stage_bytes(int precision = 0);
 cudaError_t prepare_step_kernels();
 cudaError_t launch_step(const StepArgs& a, const StepLaunch& l, cudaStream_t s);
 // One missing population of the paper's walls: population i of the fluid node
-// at offset o, and how many of the nodes x + e_i, x + 2 e_i in turn are fluid.
-struct alignas(16) WallLink {
-    long long o;
-    int i, ahead;
-};
+// at offset o, and how many of the nodes x + e_i, x + 2 e_i in turn are fluid, as
+// o << 5 | (i - 1) << 2 | ahead.
+using WallLink = uint64_t;
+inline WallLink wall_link(long long o, int i, int ahead) { return uint64_t(o) << 5 | uint64_t(i - 1) << 2 | uint64_t(ahead); }
 // The paper's wall values for the step that reads src (lbm_device.cuh,
 // equilibrium_wall): the value of each of the n links goes to plane i - 1 of W
 // (8 planes of the storage type), which the step kernels' kWalls

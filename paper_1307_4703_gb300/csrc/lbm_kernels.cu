@@ -383,10 +383,11 @@ __global__ void __launch_bounds__(64) wall_values(const T* S, T* W, const WallLi
                                                    int pitch)
 {
     const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    WallLink l{};
-    if (e < n) l = list[e];
+    const WallLink l = e < n ? list[e] : 0;
+    const long long o = (long long)(l >> 5);
+    const int i = 1 + int((l >> 2) & 7u);
     grid_dependency_sync();
-    if (e < n) Codec<T>::st1(W + (l.i - 1) * P + l.o, equilibrium_wall(l.i, l.ahead, S, P, l.o, pitch), 0.f);
+    if (e < n) Codec<T>::st1(W + (i - 1) * P + o, equilibrium_wall(i, int(l & 3u), S, P, o, pitch), 0.f);
 }
 
 }  // namespace
