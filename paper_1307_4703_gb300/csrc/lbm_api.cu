@@ -6,7 +6,6 @@
 // kernels on the handle's stream.  No call here computes any part of the
 // time step on the host.
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -15,8 +14,6 @@
 #include <mutex>
 #include <new>
 #include <string>
-#include <system_error>
-#include <thread>
 #include <vector>
 
 #include <nvtx3/nvToolsExt.h>
@@ -791,8 +788,10 @@ lbm_status create_impl(lbm_handle* out, int32_t nx, int32_t ny, const uint8_t* m
                 tiles.push_back(make_uint2((uint32_t(y) << lbm::kColBits) | uint32_t(t0 / lbm::kTileStart),
                                            uint32_t(q0) | (uint32_t(q1) << 8) | (scattered ? lbm::kWallTile : 0u)));
             };
-            for (int x = 0; x < nx && fits; ++x) {
-                if (L[x] == lbm::kSolid) continue;
+            for (int x = 0; x < nx && fits; x += 4) {  // (tiles start on whole quads)
+                uint32_t quad;
+                std::memcpy(&quad, L + x, 4);
+                if (quad == 0xFFFFFFFFu) continue;
                 if (t0 < 0 || x >= t0 + lbm::kTileNodes) {
                     if (t0 >= 0) push();
                     t0 = x / gran * gran;
@@ -803,7 +802,9 @@ lbm_status create_impl(lbm_handle* out, int32_t nx, int32_t ny, const uint8_t* m
                 }
                 q1 = (x - t0) / 4;
                 scattered |= wall >= 0 && q1 > wall;
-                if (L[x] != 0 && q1 > q0) wall = q1;
+                if (quad != 0 && q1 > q0)
+                    for (int k = 0; k < 4; ++k)
+                        if (L[x + k] != 0 && L[x + k] != lbm::kSolid) wall = q1;
             }
             if (fits) {
                 if (t0 >= 0) push();
@@ -866,33 +867,11 @@ lbm_status create_impl(lbm_handle* out, int32_t nx, int32_t ny, const uint8_t* m
             std::swap(rows[1], rows[2]);
         }
     };
-    const int n_thr = int(std::max<long long>(
-        1, std::min<long long>({16, ny, (long long)std::thread::hardware_concurrency(), (long long)nx * ny >> 17})));
-    // fn(first row, end, part) for n_thr parts of the rows at once; a part whose
-    // thread cannot be had is done here.  False: out of host memory.
+    const int n_thr = lbm::parts_for((long long)nx * ny, 1 << 17, ny);
+    // fn(first row, end, part) for n_thr parts of the rows
     auto over_rows = [&](const auto& fn) {
-        std::vector<std::thread> pool;
-        std::atomic<bool> ok{true};
-        auto part = [&](int k) {
-            try {
-                fn(int((long long)ny * k / n_thr), int((long long)ny * (k + 1) / n_thr), k);
-            } catch (const std::bad_alloc&) {
-                ok = false;
-            }
-        };
-        std::vector<int> here{0};
-        pool.reserve(size_t(n_thr));
-        here.reserve(size_t(n_thr));
-        for (int k = 1; k < n_thr; ++k) {
-            try {
-                pool.emplace_back(part, k);
-            } catch (const std::system_error&) {
-                here.push_back(k);
-            }
-        }
-        for (int k : here) part(k);
-        for (auto& t : pool) t.join();
-        return ok.load();
+        return lbm::over_parts(
+            n_thr, [&](int k) { fn(int((long long)ny * k / n_thr), int((long long)ny * (k + 1) / n_thr), k); });
     };
     std::vector<RowsOut> parts(n_thr);
     if (!over_rows([&](int y0, int y1, int k) { build_rows(y0, y1, parts[size_t(k)]); }))
@@ -1063,9 +1042,13 @@ lbm_status create_impl(lbm_handle* out, int32_t nx, int32_t ny, const uint8_t* m
                 shapes[n_shapes++] = {warps, per_sm * sms, sms};
         }
         bool have = n_shapes > 0;
-        if (have)
-            plan = lbm::plan_pairs(h->tiles_rows, rowbc, nx, ny, pitch, h->precision, h->paper_ports, shapes, n_shapes,
-                                   (long long)h->launch.grid * (h->launch.block / 32));
+        try {
+            if (have)
+                plan = lbm::plan_pairs(h->tiles_rows, rowbc, nx, ny, pitch, h->precision, h->paper_ports, shapes, n_shapes,
+                                       (long long)h->launch.grid * (h->launch.block / 32));
+        } catch (const std::bad_alloc&) {
+            have = false;
+        }
         for (int b = 0; b < 2 && have; ++b)
             have = lbm::pair_tensor_map(&h->pair_map[b], h->pop[b], ny, pitch, h->precision, plan.warps) == cudaSuccess;
         if (have) {
@@ -2195,8 +2178,13 @@ void plan_scalar_levels(lbm_ctx* h)
         cudaGetLastError();
         return;
     }
-    const lbm::StripPlan p = lbm::plan_scalar(h->tiles_rows, h->rowbc_host, h->nx, h->ny, h->pitch, lbm::kScalarLevels,
-                                              lbm::scalar_level_warps(), per_sm * h->sms);
+    lbm::StripPlan p;
+    try {
+        p = lbm::plan_scalar(h->tiles_rows, h->rowbc_host, h->nx, h->ny, h->pitch, lbm::kScalarLevels,
+                             lbm::scalar_level_warps(), per_sm * h->sms);
+    } catch (const std::bad_alloc&) {
+        return;
+    }
     h->scalar_items = static_cast<int4*>(dev_alloc(h, p.items.size() * sizeof(int4)));
     h->scalar_first = static_cast<int*>(dev_alloc(h, p.block_first.size() * sizeof(int)));
     if (!h->scalar_items || !h->scalar_first) return;

@@ -131,8 +131,14 @@ std::vector<Rows> row_groups(const std::vector<uint2>& tiles, int nx, int ny, in
                        [](const Span& a, const Span& b) { return a.b == b.b && a.e == b.e; }))
             out.back().yb = y + 1;
         else
-            out.push_back({y, y + 1, spans, cover(spans, nx, pitch)});
+            out.push_back({y, y + 1, spans, {}});
     }
+    const int parts = parts_for((long long)out.size() * (pitch / kTileNodes), 1 << 14, (long long)out.size());
+    const bool ok = over_parts(parts, [&](int k) {
+        for (size_t g = out.size() * size_t(k) / size_t(parts); g < out.size() * size_t(k + 1) / size_t(parts); ++g)
+            out[g].own = cover(out[g].spans, nx, pitch);
+    });
+    if (!ok) throw std::bad_alloc();
     return out;
 }
 
@@ -185,7 +191,6 @@ std::vector<Run> strip_runs(const std::vector<Rows>& groups)
 std::vector<Run> split_kinds(const std::vector<Run>& runs, const std::vector<Rows>& groups,
                              const std::vector<uint2>& tiles, const std::vector<RowBC>& bc, int ny, int halo)
 {
-    std::vector<Run> out;
     std::vector<int> group_of(static_cast<size_t>(ny));
     for (size_t k = 0; k < groups.size(); ++k)
         for (int y = groups[k].ya; y < groups[k].yb; ++y) group_of[size_t(y)] = int(k);
@@ -201,7 +206,7 @@ std::vector<Run> split_kinds(const std::vector<Run>& runs, const std::vector<Row
     for (const RowBC& b : bc)
         if (b.x >= 0 && (port_cols.empty() || port_cols.back() != b.x)) port_cols.push_back(b.x);
     std::sort(port_cols.begin(), port_cols.end());
-    for (const Run& r : runs) {
+    auto split_run = [&](const Run& r, std::vector<Run>& out) {
         const int x0 = r.t.x0, x1 = x0 + kTileNodes;
         // the lanes where the row's fluid begins and ends within the strip; -1: more than two
         auto side = [&](int y) {
@@ -258,7 +263,18 @@ std::vector<Run> split_kinds(const std::vector<Run>& runs, const std::vector<Row
             }
             y = e;
         }
-    }
+    };
+    long long rows = 0;
+    for (const Run& r : runs) rows += r.yb - r.ya;
+    const int parts = parts_for(rows, 1 << 14, (long long)runs.size());
+    std::vector<std::vector<Run>> done(static_cast<size_t>(parts));
+    const bool ok = over_parts(parts, [&](int k) {
+        for (size_t n = runs.size() * size_t(k) / size_t(parts); n < runs.size() * size_t(k + 1) / size_t(parts); ++n)
+            split_run(runs[n], done[size_t(k)]);
+    });
+    if (!ok) throw std::bad_alloc();
+    std::vector<Run> out = std::move(done[0]);
+    for (size_t k = 1; k < done.size(); ++k) out.insert(out.end(), done[k].begin(), done[k].end());
     return out;
 }
 

@@ -2,11 +2,50 @@
 // strips (lbm_plan.cu).
 #pragma once
 
+#include <algorithm>
+#include <atomic>
+#include <new>
+#include <system_error>
+#include <thread>
 #include <vector>
 
 #include "lbm_internal.h"
 
 namespace lbm {
+
+// fn(0) .. fn(n - 1) on a host thread each; a part whose thread cannot be had is
+// done here.  False: one ran out of memory.
+template <typename Fn>
+bool over_parts(int n, const Fn& fn)
+{
+    std::atomic<bool> ok{true};
+    auto part = [&](int k) {
+        try {
+            fn(k);
+        } catch (const std::bad_alloc&) {
+            ok = false;
+        }
+    };
+    std::vector<std::thread> threads;
+    std::vector<int> here{0};
+    threads.reserve(size_t(n));
+    here.reserve(size_t(n));
+    for (int k = 1; k < n; ++k) {
+        try {
+            threads.emplace_back(part, k);
+        } catch (const std::system_error&) {
+            here.push_back(k);
+        }
+    }
+    for (int k : here) part(k);
+    for (std::thread& t : threads) t.join();
+    return ok;
+}
+// Parts for `work` units of which `each` are worth a thread.
+inline int parts_for(long long work, long long each, long long most)
+{
+    return int(std::max(1ll, std::min({16ll, most, (long long)std::thread::hardware_concurrency(), work / each})));
+}
 
 struct StripPlan {
     std::vector<int4> items;       // strips (PairArgs::items)
