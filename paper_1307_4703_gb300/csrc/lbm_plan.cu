@@ -387,17 +387,19 @@ StripPlan plan_pairs(const std::vector<uint2>& tiles, const std::vector<RowBC>& 
         // The longest block's time against a single step's: a wave of tiles, rounds of
         // them, or HBM's rate, and what their scattered walls add.  Both are fits, within
         // 15 % over some three hundred lattices; strips of much more work than the tiles'
-        // have to be ahead by a tenth.  us a step, single / two-step launches: 256 x 128
-        // 3.6 / 2.3, 1024 x 512 5.24 / 4.60, 1024 x 768 7.1 / 5.4, 4096 x 2048 59.5 / 35.5;
-        // random cells, 3 and 70 % solid, 1001 x 517 10.5 / 9.5 and 12.2 / 9.6, 2001 x 1003
-        // 40.7 / 32.4 and 51.3 / 36.5; pillars of 10 cells 24 apart, whose strips fall into
-        // pieces of a dozen rows, 2001 x 1003 39.0 / 31.5 but 900 x 600 9.5 / 10.9 and 700 x
-        // 400 5.7 / 8.6.
+        // have to be ahead by a tenth, those of few scattered walls may seem as much
+        // behind (batches of 3 and 4 chips 5.6 / 5.4, 5.5 / 5.2).  us a step, single /
+        // two-step launches: 256 x 128 3.6 / 2.3, 1024 x 512 5.24 / 4.60, 1024 x 768 7.1 /
+        // 5.4, 4096 x 2048 59.5 / 35.5; random cells, 3 and 70 % solid, 1001 x 517 10.5 / 9.5
+        // and 12.2 / 9.6, 2001 x 1003 40.7 / 32.4 and 51.3 / 36.5; pillars of 10 cells 24
+        // apart, whose strips fall into pieces of a dozen rows, 2001 x 1003 39.3 / 31.4 but
+        // 900 x 600 9.5 / 10.9 and 700 x 400 5.7 / 8.6.
         double scattered = 0.;
         for (const uint2& t : tiles) scattered += (t.y & kWallTile) != 0;
         const bool one_round = (long long)tiles.size() <= single_warps;
         const double single = std::max(one_round ? 3.2 + 0.95e-3 * n : 4.0 + 1.25e-3 * n, 2.1e-3 * n) + 0.5e-3 * scattered;
-        p.worth = idle || (p.warps == 4 ? 0.126 : 0.131) * p.time < (work < 1.5 ? 1.06 : 0.9) * single;
+        const double margin = work >= 1.5 ? 0.9 : 8. * scattered < n ? 1.15 : 1.06;
+        p.worth = idle || (p.warps == 4 ? 0.126 : 0.131) * p.time < margin * single;
     } else {
         // The work alone.  16-bit storage, whose single step is bound by issue and starts
         // up longer: FP16 256 x 128 4.8 / 2.4, 1024 x 768 5.6 / 4.9, 4096 x 2048 36.2 / 28.1,

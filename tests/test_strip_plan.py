@@ -225,3 +225,22 @@ def test_two_steps_a_launch_where_they_are_faster(lib):
                                       (900, 600, 24, 10, False), (1001, 517, 24, 10, False), (700, 400, 12, 6, False)):
         ports = W.random_case(5, nx, ny, solid_frac=0.0)[0]["ports"]
         assert Plan(lib, _pillars(nx, ny, step, side), ports).worth == worth, (nx, ny, step, side)
+
+
+@pytest.mark.parametrize("n,seed", [(3, 1), (4, W.SEED + 4), (4, 2), (16, 1)])
+def test_small_batches_take_two_steps_a_launch(lib, n, seed):
+    """Batches as lbm_create_batch stacks them (one solid row between chips): two steps a
+    launch are the faster way from three chips on."""
+    probs = W.config_batch(n, seed=seed)
+    nx = max(q["nx"] for q in probs)
+    rows, ports, y = [], [], 0
+    for k, q in enumerate(probs):
+        if k:
+            rows.append(np.ones((1, nx), np.uint8))
+            y += 1
+        m = np.ones((q["ny"], nx), np.uint8)
+        m[:, :q["nx"]] = q["solid"]
+        rows.append(m)
+        ports += [dict(r, y0=r["y0"] + y, y1=r["y1"] + y) for r in q["ports"]]
+        y += q["ny"]
+    assert Plan(lib, np.concatenate(rows), ports).worth
