@@ -140,8 +140,9 @@ struct lbm_ctx {
     std::vector<Inst> inst;  // empty for a single chip
     float4* rates = nullptr; // per-row relaxation rates of a batch
 
-    // CUDA graphs of graph_steps consecutive step launches, one per valve
-    // words, starting buffer and order, captured on a private stream.
+    // CUDA graphs of the launches that take graph_steps consecutive steps (one
+    // or two a launch), one per valve words, starting buffer and order, captured
+    // on a private stream.
     struct Graph {
         uint32_t words[lbm::kMaskWords];
         int parity, order;
@@ -423,7 +424,7 @@ bool capturing(const lbm_ctx* h)
     return true;
 }
 
-// The cached graph of graph_steps launches for the valve words in
+// The cached graph of the launches of graph_steps steps for the valve words in
 // a.open_mask starting from buffer cur, captured on first use.
 lbm_status step_graph(lbm_ctx* h, lbm::StepArgs a, const lbm_ctx::Graph** out)
 {

@@ -1,15 +1,16 @@
-// lbm_scalar.cu -- scalar-only step on a stored velocity field.
+// lbm_scalar.cu -- scalar-only steps on a stored velocity field.
 //
 // The paper's own workflow (section "Results"): the flow reaches its steady
 // state quickly, so the stationary velocity field of each valve state is
 // computed once and the advection-diffusion solver reads it, with a larger
 // time step for the scalar (the field is rescaled by the ratio of the time
-// steps).  One launch advances the scalar lattice by one step: pull-stream of
-// g with bounce-back, held concentration / do-nothing at open ports, and BGK
-// relaxation towards the equilibrium of Eq. cdeequilibrium with the stored
-// (scaled) velocity.  Per fluid node and step it reads 5 scalar populations
-// and the 2 velocity components and writes 5 populations: 48 bytes, against
-// 112 for the coupled step.
+// steps).  A step of the scalar lattice is pull-stream of g with bounce-back,
+// held concentration / do-nothing at open ports, and BGK relaxation towards
+// the equilibrium of Eq. cdeequilibrium with the stored (scaled) velocity.
+// The kernels of one step (scalar_frozen_regs, scalar_frozen_bulk) read 5 scalar
+// populations and the 2 velocity components per fluid node and write 5
+// populations: 48 bytes, against 112 for the coupled step.
+// scalar_frozen_levels takes three steps a launch, which move that once.
 #include "lbm_device.cuh"
 
 namespace lbm {
