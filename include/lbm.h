@@ -326,8 +326,8 @@ lbm_status lbm_set_velocity_field(lbm_handle h, uint32_t open_mask, const float*
  * multiplied by u_scale, with the same scalar ports and walls as lbm_step
  * (held concentration, do-nothing, no-flux).  The fluid populations do not
  * change; the step counter advances.  With scalar_variant 0, steps of one
- * valve word go three to a launch, with the same bits; the call's last step
- * is always one by itself.  LBM_ERR_STATE (nothing launched) if a
+ * valve word go three to a launch where that is faster, with the same bits;
+ * the call's last step is always one by itself.  LBM_ERR_STATE (nothing launched) if a
  * valve word the steps use has no stored field.  Diagnostics: out[1] and
  * out[3] of lbm_get_diagnostics come from the last scalar step, out[0] and
  * out[2] stay those of the last coupled step. */

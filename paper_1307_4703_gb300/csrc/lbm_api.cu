@@ -2186,6 +2186,7 @@ void plan_scalar_levels(lbm_ctx* h)
     } catch (const std::bad_alloc&) {
         return;
     }
+    if (!p.worth) return;
     h->scalar_items = static_cast<int4*>(dev_alloc(h, p.items.size() * sizeof(int4)));
     h->scalar_first = static_cast<int*>(dev_alloc(h, p.block_first.size() * sizeof(int)));
     if (!h->scalar_items || !h->scalar_first) return;

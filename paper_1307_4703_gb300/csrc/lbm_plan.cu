@@ -91,9 +91,9 @@ enum Kind { kPlain, kSide, kScattered, kPort, kScatteredPort };
 constexpr int kPairCost[5] = {16, 18, 28, 22, 33};
 constexpr int kPairRescaleCost[5] = {16, 18, 28, 30, 42};  // with ports of the rescaling kinds (22: 4096 x 2048 44 us, here 39)
 constexpr int kScalarCost[5] = {16, 20, 24, 28, 32};
-// What an FP32 iteration of two coupled steps takes, in units of 0.131 us a step
-// (least squares over some hundred lattices; the costs above are those of the
-// fastest splits).
+// What an iteration of two coupled steps takes next to a plain one (16), by least
+// squares over some hundred lattices, FP32 and 16-bit alike (the costs above are
+// those of the fastest splits).
 constexpr int kPairTime[5] = {16, 17, 21, 22, 25};
 
 struct Run {
@@ -341,6 +341,30 @@ StripPlan plan(const std::vector<Run>& runs, const int (&costs)[5], int halo, in
     return out;
 }
 
+double scattered_tiles(const std::vector<uint2>& tiles)
+{
+    double n = 0.;
+    for (const uint2& t : tiles) n += (t.y & kWallTile) != 0;
+    return n;
+}
+
+// A single step's time, us: of n tiles in one wave, in several, at the rate of
+// memory, and what each tile of scattered walls adds.  These fits and those of the
+// several-steps launches' times are within some 15 % over 340 lattices.
+struct SingleTime {
+    double wave, per_tile, waves, per_tile_waves, memory, wall;
+};
+constexpr SingleTime kSingle[2][2] = {  // FP32 and 16-bit storage; the second with ports of the rescaling kinds
+    {{3.2, 0.95e-3, 4.0, 1.25e-3, 2.1e-3, 0.5e-3}, {4.1, 0.87e-3, 3.2, 1.54e-3, 2.3e-3, 0.5e-3}},
+    {{4.7, 0.2e-3, 2.9, 1.02e-3, 1.33e-3, 1.0e-3}, {5.0, 0.3e-3, 3.3, 1.17e-3, 1.5e-3, 1.0e-3}}};
+constexpr SingleTime kSingleScalar = {2.5, 0.36e-3, 2.0, 0.6e-3, 0.875e-3, 0.1e-3};
+double single_step(const SingleTime& f, const std::vector<uint2>& tiles, long long warps)
+{
+    const double n = double(tiles.size());
+    const double t = (long long)tiles.size() <= warps ? f.wave + f.per_tile * n : f.waves + f.per_tile_waves * n;
+    return std::max(t, f.memory * n) + f.wall * scattered_tiles(tiles);
+}
+
 std::vector<Run> runs_of(const std::vector<uint2>& tiles, const std::vector<RowBC>& bc, int nx, int ny, int pitch, int halo)
 {
     const std::vector<Rows> groups = row_groups(tiles, nx, ny, pitch);
@@ -378,37 +402,33 @@ StripPlan plan_pairs(const std::vector<uint2>& tiles, const std::vector<RowBC>& 
         resident = s.resident;
         p = std::move(q);
     }
-    // Where two single steps are the better choice: where obstacles break the rows
-    // into strips that do far more than the tiles' work.  Strips that leave half the
-    // blocks' room idle are always the shorter way.
+    // Where single steps are the better choice: where obstacles break the rows into
+    // pieces, each with its neighbours' rows around it.  Strips that leave half the
+    // blocks' room idle are always the shorter way; elsewhere the longest block's time
+    // is set against a single step's.  The margins are those that leave the least time
+    // on the table: FP32 strips of much more work than the tiles' have to be ahead by a
+    // tenth, those of few scattered walls may seem as much behind (batches of 3 and 4
+    // chips 5.6 / 5.4, 5.5 / 5.2), and with rescaling ports they gain from the third
+    // tile of a single step's warps on.  us a step, single / two-step launches: FP32 256
+    // x 128 3.6 / 2.3, 1024 x 512 5.24 / 4.60, 1024 x 768 7.1 / 5.4, 4096 x 2048 59.5 /
+    // 35.5; random cells, 3 and 70 % solid, 1001 x 517 10.5 / 9.5 and 12.2 / 9.6, 2001 x
+    // 1003 40.7 / 32.4 and 51.3 / 36.5; pillars of 10 cells 24 apart, whose strips fall
+    // into pieces of a dozen rows, 2001 x 1003 39.3 / 31.4 but 900 x 600 9.5 / 10.9 and 700
+    // x 400 5.7 / 8.6; with rescaling ports 4096 x 2048 54.4 / 39.0, 1024 x 768 7.2 / 7.6,
+    // channels of 12 rows in 40 2001 x 1003 14.1 / 18.7.  FP16 256 x 128 4.8 / 2.4, 1024 x
+    // 768 5.6 / 4.9, 4096 x 2048 36.2 / 28.1, half solid 154 / 102; walls every ninth row
+    // 2001 x 1003 21.4 / 26.3.
     const bool idle = 2 * p.grid <= resident;
     const double n = double(tiles.size()), work = p.work / (2. * n);
-    if (f32 && !rescale) {
-        // The longest block's time against a single step's: a wave of tiles, rounds of
-        // them, or HBM's rate, and what their scattered walls add.  Both are fits, within
-        // 15 % over some three hundred lattices; strips of much more work than the tiles'
-        // have to be ahead by a tenth, those of few scattered walls may seem as much
-        // behind (batches of 3 and 4 chips 5.6 / 5.4, 5.5 / 5.2).  us a step, single /
-        // two-step launches: 256 x 128 3.6 / 2.3, 1024 x 512 5.24 / 4.60, 1024 x 768 7.1 /
-        // 5.4, 4096 x 2048 59.5 / 35.5; random cells, 3 and 70 % solid, 1001 x 517 10.5 / 9.5
-        // and 12.2 / 9.6, 2001 x 1003 40.7 / 32.4 and 51.3 / 36.5; pillars of 10 cells 24
-        // apart, whose strips fall into pieces of a dozen rows, 2001 x 1003 39.3 / 31.4 but
-        // 900 x 600 9.5 / 10.9 and 700 x 400 5.7 / 8.6.
-        double scattered = 0.;
-        for (const uint2& t : tiles) scattered += (t.y & kWallTile) != 0;
-        const bool one_round = (long long)tiles.size() <= single_warps;
-        const double single = std::max(one_round ? 3.2 + 0.95e-3 * n : 4.0 + 1.25e-3 * n, 2.1e-3 * n) + 0.5e-3 * scattered;
-        const double margin = work >= 1.5 ? 0.9 : 8. * scattered < n ? 1.15 : 1.06;
-        p.worth = idle || (p.warps == 4 ? 0.126 : 0.131) * p.time < margin * single;
+    double margin = 1.1, two;
+    if (f32) {
+        if (rescale) margin = (long long)tiles.size() <= 2 * single_warps ? 0. : 1.;
+        else margin = work >= 1.5 ? 0.9 : 8. * scattered_tiles(tiles) < n ? 1.15 : 1.06;
+        two = (rescale ? (p.warps == 4 ? 0.157 : 0.155) : (p.warps == 4 ? 0.126 : 0.131)) * p.time;
     } else {
-        // The work alone.  16-bit storage, whose single step is bound by issue and starts
-        // up longer: FP16 256 x 128 4.8 / 2.4, 1024 x 768 5.6 / 4.9, 4096 x 2048 36.2 / 28.1,
-        // at 2.1 of the tiles' work 19.5 / 20.7 and at 1.5 8.1 / 4.2.  With rescaling ports
-        // FP32 strips gain from the third tile of a single step's warps on (1024 x 768
-        // 7.2 / 7.6, 4096 x 2048 54.4 / 39.0).
-        const bool few = f32 && (long long)tiles.size() <= 2 * single_warps;
-        p.worth = idle || (!few && work < (f32 ? 1.5 : 1.8));
+        two = (rescale ? 0.7 : 0.2) + (p.warps == 6 ? 0.109 : rescale ? 0.147 : 0.138) * p.time;
     }
+    p.worth = idle || two < margin * single_step(kSingle[f32 ? 0 : 1][rescale], tiles, single_warps);
     // With the state between the steps stored as well (a gradient's recomputation):
     // ahead on lattices that leave the GPU idle (a gradient over 150 steps of 256 x 128
     // 1605 -> 1447 us, 512 x 256 1270 -> 1210) and on those of more than two rounds of a
@@ -418,14 +438,18 @@ StripPlan plan_pairs(const std::vector<uint2>& tiles, const std::vector<RowBC>& 
     return p;
 }
 
-// No rule: several steps a launch are ahead nearly everywhere (100 lattices from 300
-// x 200 to 4096 x 2048, us a step, one step a launch / three: scattered cells 3 to 70
-// % solid 1001 x 517 4.5 / 4.2 and 4.8 / 4.4, 2001 x 1003 13.7 / 9.7 and 14.2 / 10.1, 4096
-// x 2048 61.4 / 39.0; at worst, pillars of 10 cells 24 apart, 1001 x 517 4.2 / 4.7).
+// Worth it unless the lattice is mostly solid: us a step, one step a launch / three,
+// scattered cells 3 and 70 % solid 1001 x 517 4.5 / 4.2 and 4.8 / 4.4, 2001 x 1003 13.7 / 9.7
+// and 14.2 / 10.1, 4096 x 2048 61.4 / 39.0; 95 % solid, islands of a few nodes, 2001 x 1003
+// 9.5 / 35.4; walls every ninth row there 11.8 / 13.2; at worst, pillars of 10 cells 24
+// apart, 1001 x 517 4.2 / 4.7.
 StripPlan plan_scalar(const std::vector<uint2>& tiles, const std::vector<RowBC>& bc, int nx, int ny, int pitch, int levels,
                       int warps, int resident)
 {
-    return plan(runs_of(tiles, bc, nx, ny, pitch, levels - 1), kScalarCost, levels - 1, warps, resident);
+    StripPlan p = plan(runs_of(tiles, bc, nx, ny, pitch, levels - 1), kScalarCost, levels - 1, warps, resident);
+    // (a single step's wave is 16 warps an SM, here two blocks)
+    p.worth = 0.0607 * p.longest < 1.05 * single_step(kSingleScalar, tiles, 8ll * resident);
+    return p;
 }
 
 }  // namespace lbm

@@ -55,7 +55,7 @@ struct StripPlan {
     int longest = 0;               // cost of the block that takes longest
     int time = 0;                  // the longest block's time (kPairTime)
     double work = 0;
-    bool worth = false;            // faster than single steps (plan_pairs)
+    bool worth = false;            // faster than single steps
     bool worth_keep = false;       // also with every state stored (plan_pairs)
 };
 

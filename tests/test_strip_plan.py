@@ -227,6 +227,30 @@ def test_two_steps_a_launch_where_they_are_faster(lib):
         assert Plan(lib, _pillars(nx, ny, step, side), ports).worth == worth, (nx, ny, step, side)
 
 
+def test_other_launches_where_they_are_faster(lib):
+    """16-bit storage, ports of the rescaling kinds and scalar-only steps, as above: islands
+    of a few nodes, walls every ninth row and rows of narrow channels go one step a launch,
+    though their neighbours in kind do not."""
+    nx, ny = 2001, 1003
+    prob = W.random_case(5, nx, ny, solid_frac=0.95)[0]
+    assert not Plan(lib, prob["solid"], prob["ports"], levels=LEVELS).worth
+    for share in (0.03, 0.5, 0.7):
+        solid = np.random.default_rng(5).random((ny, nx)) < share
+        assert Plan(lib, solid, levels=LEVELS).worth and Plan(lib, solid, precision=FP16).worth
+    y = np.arange(ny)[:, None] + np.zeros(nx, int)
+    inner = np.zeros((ny, nx), bool)
+    inner[:, 4:-4] = True
+    ports = W.random_case(5, nx, ny, solid_frac=0.0)[0]["ports"]
+    rows, channels = (y % 9 == 4) & inner, (y % 40 >= 12) & inner
+    assert not Plan(lib, rows, ports, precision=FP16).worth
+    assert not Plan(lib, channels, ports, rescale=True).worth
+    assert Plan(lib, channels, ports).worth
+    chip = W.config_large_chip()
+    for precision in (FP32, FP16):
+        for rescale in (False, True):
+            assert Plan(lib, chip["solid"], chip["ports"], precision=precision, rescale=rescale).worth
+
+
 @pytest.mark.parametrize("n,seed", [(3, 1), (4, W.SEED + 4), (4, 2), (16, 1)])
 def test_small_batches_take_two_steps_a_launch(lib, n, seed):
     """Batches as lbm_create_batch stacks them (one solid row between chips): two steps a
